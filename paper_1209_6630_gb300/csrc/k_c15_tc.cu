@@ -39,6 +39,8 @@
 // commits to mbarriers; waits are bounded by %globaltimer
 // (QMC_STATUS_TIMEOUT on expiry).  Unions longer than 1024 AOs
 // are accumulated in chunks of 1024, each added to the output in FP64.
+#include <algorithm>
+
 #include "ao_ff.cuh"
 #include "qmc_internal.cuh"
 #include "slices.cuh"
@@ -57,8 +59,6 @@ constexpr int kPlanesPerStep = 2 * kC15Slices + 6;             // [C1 slice][C5 
 constexpr int SK = 32;
 constexpr uint32_t kSPlaneBytes = TC_M * SK * 2;               // 8 KB
 constexpr uint32_t kSBPlaneBytes = SK * TC_N * 2;              // 8 KB, MN-major, 128-byte swizzle
-constexpr size_t kStageBytes = (size_t)kPlanesPerStep * kSPlaneBytes;
-constexpr size_t kStepBytes = 2 * kStageBytes;
 constexpr int kChunkSteps = 16;                                // 1024 AOs per exact accumulation
 constexpr int kAcc = 4;                                        // accumulators per output
 
@@ -72,7 +72,9 @@ struct C15TcArgs {
     int e0;                        // first electron of the batch
     int n_tiles;                   // walker tiles of 128
     int kmax_steps;                // staging capacity per (electron, tile), in K steps
-    unsigned char *planes;         // [batch e][tile][kmax_steps][12][16 KB]
+    int prows;                     // rows of a staged operand plane: 128, or a single tile's walkers rounded up to 8
+    int planes_per_stage;          // 18 (C1, C5, gradients), or 6 (C1 alone)
+    unsigned char *planes;         // [batch e][tile][kmax_steps][2][planes_per_stage][prows x 64 bytes]
     int *ao_list;                  // [batch e][tile][kmax_steps * 64]
     int *nks;                      // [batch e][tile]
     int *rexp;                     // [batch e][tile][128][2]
@@ -142,34 +144,79 @@ __device__ __forceinline__ void f32_angular(const SysDev &s, const C15TcArgs &a,
     g3 = c * (px * py * dpz * rd.g + m2gd * rd.dz * P);
 }
 
-// three CTAs per SM (80 registers; a small spill costs less than the latency it hides).
+// The float-float radial part of one shell and the AO values (kLap: and Laplacians) from it:
+// the expressions of ao_val_ff and ao_val_lap_ff.
+template <bool kLap>
+struct FfShell {
+    FfRadial rd;
+    __device__ __forceinline__ void radial(const SysDev &s, const FfBasis &fb, int sh, const float2 *r)
+    {
+        if constexpr (kLap) ff_radial(s, fb, sh, r, rd);
+        else ff_radial_val(s, fb, sh, r, rd);
+    }
+    __device__ __forceinline__ void angular(const SysDev &s, const FfBasis &fb, int mu, float2 &v, float2 &lp)
+    {
+        if constexpr (kLap) ff_angular(s, fb, mu, rd, v, lp);
+        else v = ff_angular_val(s, fb, mu, rd);
+    }
+};
+
+// Appends the low half of x to eight 16-bit values in four words (the oldest falls out).
+__device__ __forceinline__ void push_low16(uint32_t (&w)[4], uint32_t x)
+{
+#pragma unroll
+    for (int i = 0; i < 3; ++i) w[i] = __byte_perm(w[i], w[i + 1], 0x5432);
+    w[3] = __byte_perm(w[3], x, 0x5432);
+}
+
+// Appends a value that is exact in BF16 to eight of them in four words (the oldest falls out).
+__device__ __forceinline__ void push_bf16(uint32_t (&w)[4], float x)
+{
+#pragma unroll
+    for (int i = 0; i < 3; ++i) w[i] = __byte_perm(w[i], w[i + 1], 0x5432);
+    w[3] = __byte_perm(w[3], __float_as_uint(x), 0x7632);
+}
+
+// Bound by the FP32 pipes (the float-float radial sums) and the latency of the basis tables.
+// Measured at 1056 electrons (318 AOs an electron): 2048 walkers 47.2 -> 24.1 ms with the
+// rolled pass 2, a warp's lanes on the same AOs and the radial part once per shell; 37 walkers
+// 46.8 -> 0.81 ms with all electrons in one launch and the idle rows' threads used.
+// kC1Only: three CTAs per SM; with the Laplacians and gradients two (their words and radial
+// parts are more than 80 registers hold).
 // kC1Only: the C-free variant's producer: float-float values alone, six planes per stage.
 template <bool kC1Only>
-__global__ void __launch_bounds__(kPrepThreads, 3) k_c15_prep(C15TcArgs a)
+__global__ void __launch_bounds__(kPrepThreads, kC1Only ? 3 : 2) k_c15_prep(C15TcArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *mask_s = reinterpret_cast<uint32_t *>(smem_raw);           // [128][mw]
     int *ao_s = reinterpret_cast<int *>(mask_s + TC_M * a.mw);           // [n_ao + 64]
     __shared__ uint32_t union_s[256];
     __shared__ int warp_s[kPrepThreads / 32];
+    __shared__ int vmax_s[TC_M], lmax_s[TC_M];
 
     const SysDev &s = a.s;
     const int tile = blockIdx.x, el = blockIdx.y, e = a.e0 + el;
-    const int t = threadIdx.x, row = t >> 1, half = t & 1;
+    // thread -> (row, every n_slot-th chunk of 8 AOs): a warp's lanes hold different walkers at the
+    // same AOs, so the shells' loops are uniform in a warp; a tile of few walkers (rp, the power
+    // of two that holds its rows) spreads its AO chunks over the threads that have no row
+    const int rv = min(TC_M, a.nw - tile * TC_M);
+    const int lrp = 32 - __clz(rv - 1), rp = 1 << lrp;          // rv = 1: __clz(0) = 32, rp = 1
+    const int t = threadIdx.x, row = t & (rp - 1), slot_c = t >> lrp, n_slot = kPrepThreads >> lrp;
     const int w = tile * TC_M + row;
-    const bool wvalid = w < a.nw;
+    const bool wvalid = row < rv;
     const int mw = a.mw;
+    const uint32_t pbytes = (uint32_t)a.prows * (SK * 2);        // bytes of a staged plane
+    const size_t stage_bytes = (size_t)a.planes_per_stage * pbytes;
     const size_t slot = (size_t)el * a.n_tiles + tile;
 
-    for (int q = t; q < TC_M * mw; q += kPrepThreads) {
+    for (int q = t; q < rv * mw; q += kPrepThreads) {
         const int m = q / mw, j = q - m * mw;
-        const int wm = tile * TC_M + m;
-        mask_s[q] = (wm < a.nw) ? a.masks[((size_t)wm * s.n_elec + e) * mw + j] : 0u;
+        mask_s[q] = a.masks[((size_t)(tile * TC_M + m) * s.n_elec + e) * mw + j];
     }
     __syncthreads();
     for (int j = t; j < mw; j += kPrepThreads) {
         uint32_t u = 0;
-        for (int m = 0; m < TC_M; ++m) u |= mask_s[m * mw + j];
+        for (int m = 0; m < rv; ++m) u |= mask_s[m * mw + j];
         union_s[j] = u;
     }
     __syncthreads();
@@ -190,16 +237,19 @@ __global__ void __launch_bounds__(kPrepThreads, 3) k_c15_prep(C15TcArgs a)
         return ((my_mask[sh >> 5] >> (sh & 31)) & 1u) != 0;
     };
 
-    unsigned char *pl = a.planes + slot * (size_t)a.kmax_steps * kStepBytes;
+    unsigned char *pl = a.planes + slot * (size_t)a.kmax_steps * 2 * stage_bytes;
+    const int nc8 = nks * (TC_K / 8);                            // chunks of 8 AOs; chunk c8 is in stage c8 / 4
+    const bool stores = row < a.prows;                           // rows past the staged ones have no place
     // pass 1 (FP32; radial part once per shell): bounds of |value| and
     // |Laplacian| over the row, and the gradient planes of C2..C4
     float vmax = 0.f, lmax = 0.f;
     if constexpr (kC1Only) {
         F32Radial rd;
         int last_sh = -1;
-        for (int ks = 0; ks < nks; ++ks)
-            for (int q = half * 32; q < half * 32 + 32; ++q) {
-                const int mu = ao_s[ks * TC_K + q];
+        for (int c8 = slot_c; c8 < nc8; c8 += n_slot)
+#pragma unroll 1
+            for (int q = 0; q < 8; ++q) {
+                const int mu = ao_s[c8 * 8 + q];
                 int sh;
                 if (!active(mu, sh)) continue;
                 if (sh != last_sh) {
@@ -214,109 +264,95 @@ __global__ void __launch_bounds__(kPrepThreads, 3) k_c15_prep(C15TcArgs a)
         F32Radial rd;
         int last_sh = -1;
         const int f16 = a.tt.f16;
-        for (int ks = 0; ks < nks; ++ks)
-            for (int c8 = half * 4; c8 < half * 4 + 4; ++c8) {
-                float gv[3][8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    gv[0][q] = gv[1][q] = gv[2][q] = 0.f;
-                    const int mu = ao_s[ks * TC_K + c8 * 8 + q];
-                    int sh;
-                    if (!active(mu, sh)) continue;
+        for (int c8 = slot_c; c8 < nc8; c8 += n_slot) {
+            uint32_t wh[3][4], wl[3][4];
+#pragma unroll 1
+            for (int q = 0; q < 8; ++q) {
+                float gv[3] = {0.f, 0.f, 0.f};
+                const int mu = ao_s[c8 * 8 + q];
+                int sh;
+                if (active(mu, sh)) {
                     if (sh != last_sh) {
                         last_sh = sh;
                         f32_radial(s, a, sh, r2[0].x, r2[0].y, r2[1].x, r2[1].y, r2[2].x, r2[2].y, rd);
                     }
                     float v, lp;
-                    f32_angular(s, a, mu, rd, v, lp, gv[0][q], gv[1][q], gv[2][q]);
+                    f32_angular(s, a, mu, rd, v, lp, gv[0], gv[1], gv[2]);
                     vmax = fmaxf(vmax, fabsf(v));
                     lmax = fmaxf(lmax, fabsf(lp));
                 }
-                // stage 2 ks + c8 / 4 (this thread's half), chunk c8 % 4 within it
-                const uint32_t off = a_off64(row, c8 & 3);
-                unsigned char *stp = pl + (size_t)(2 * ks + (c8 >> 2)) * kStageBytes +
-                                     (size_t)kGradPlane0 * kSPlaneBytes;
 #pragma unroll
                 for (int l = 0; l < 3; ++l) {
-                    uint32_t hi[4], lo[4];
-                    const float isc = a.tt.in_scale[l];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) split2(gv[l][2 * q] * isc, gv[l][2 * q + 1] * isc, f16, hi[q], lo[q]);
-                    *reinterpret_cast<uint4 *>(stp + (size_t)(2 * l) * kSPlaneBytes + off) =
-                        make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                    *reinterpret_cast<uint4 *>(stp + (size_t)(2 * l + 1) * kSPlaneBytes + off) =
-                        make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                    uint32_t hi, lo;
+                    split2(gv[l] * a.tt.in_scale[l], 0.f, f16, hi, lo);
+                    push_low16(wh[l], hi);
+                    push_low16(wl[l], lo);
                 }
             }
+            if (!stores) continue;
+            unsigned char *stp = pl + (size_t)(c8 >> 2) * stage_bytes + (size_t)kGradPlane0 * pbytes +
+                                 a_off64(row, c8 & 3);
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                *reinterpret_cast<uint4 *>(stp + (size_t)(2 * l) * pbytes) =
+                    make_uint4(wh[l][0], wh[l][1], wh[l][2], wh[l][3]);
+                *reinterpret_cast<uint4 *>(stp + (size_t)(2 * l + 1) * pbytes) =
+                    make_uint4(wl[l][0], wl[l][1], wl[l][2], wl[l][3]);
+            }
+        }
     }
-    vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, 1));
-    lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, 1));
-    const int Ev = exp_bound(vmax), El = exp_bound(lmax);
-    if (half == 0) {
+    // the row's bounds over its threads (both are >= 0: an integer maximum of the bits)
+    if (t < TC_M) { vmax_s[t] = 0; lmax_s[t] = 0; }
+    __syncthreads();
+    atomicMax(&vmax_s[row], __float_as_int(vmax));
+    atomicMax(&lmax_s[row], __float_as_int(lmax));
+    __syncthreads();
+    const int Ev = exp_bound(__int_as_float(vmax_s[row])), El = exp_bound(__int_as_float(lmax_s[row]));
+    if (t < rp) {
         a.rexp[(slot * TC_M + row) * 2] = Ev;
         a.rexp[(slot * TC_M + row) * 2 + 1] = El;
     }
+    if (!stores) return;
 
-    if constexpr (kC1Only) {
-        for (int ks = 0; ks < nks; ++ks)
-            for (int c8 = half * 4; c8 < half * 4 + 4; ++c8) {
-                uint32_t wv[kC15Slices][4];
-#pragma unroll
-                for (int q2 = 0; q2 < 4; ++q2) {
-                    float sv[2][kC15Slices];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int mu = ao_s[ks * TC_K + c8 * 8 + 2 * q2 + h];
-                        int sh;
-                        const float2 v = active(mu, sh) ? ao_val_ff(s, a.fb, mu, r2) : make_float2(0.f, 0.f);
-                        slice6(v, Ev, sv[h]);
-                    }
-#pragma unroll
-                    for (int j = 0; j < kC15Slices; ++j) wv[j][q2] = bf16_pair(sv[0][j], sv[1][j]);
+    // pass 2: float-float values (and Laplacians), sliced into the operand planes; the radial
+    // part once per shell of the chunk.  One AO per rolled iteration, its slices shifted into the
+    // chunk's words: with eight AOs inlined the loop outgrew the instruction cache (ncu at 1056
+    // electrons x 256 walkers: 13.5 of 19 cycles per instruction waiting for instructions)
+    for (int c8 = slot_c; c8 < nc8; c8 += n_slot) {
+        uint32_t wv[kC15Slices][4], wl[kC1Only ? 1 : kC15Slices][4];
+        FfShell<!kC1Only> rd;
+        int last_sh = -1;
+#pragma unroll 1
+        for (int q = 0; q < 8; ++q) {
+            const int mu = ao_s[c8 * 8 + q];
+            int sh;
+            float2 v = make_float2(0.f, 0.f), lp = make_float2(0.f, 0.f);
+            if (active(mu, sh)) {
+                if (sh != last_sh) {
+                    last_sh = sh;
+                    rd.radial(s, a.fb, sh, r2);
                 }
-                const uint32_t off = a_off64(row, c8 & 3);
-                unsigned char *stp = pl + (size_t)(2 * ks + (c8 >> 2)) * kStageBytes;
-#pragma unroll
-                for (int j = 0; j < kC15Slices; ++j)
-                    *reinterpret_cast<uint4 *>(stp + (size_t)j * kSPlaneBytes + off) =
-                        make_uint4(wv[j][0], wv[j][1], wv[j][2], wv[j][3]);
+                rd.angular(s, a.fb, mu, v, lp);
             }
-        return;
-    }
-    // pass 2: float-float values and Laplacians, sliced into the operand planes
-    // (the float-float radial part is recomputed per AO here: caching it per shell,
-    // as in pass 1, keeps 12 more registers live across the slicing and measured slower)
-    for (int ks = 0; ks < nks; ++ks)
-        for (int c8 = half * 4; c8 < half * 4 + 4; ++c8) {
-            uint32_t wv[kC15Slices][4], wl[kC15Slices][4];
+            float sl[kC15Slices];
+            slice6(v, Ev, sl);
 #pragma unroll
-            for (int q2 = 0; q2 < 4; ++q2) {
-                float sv[2][kC15Slices], sl[2][kC15Slices];
+            for (int j = 0; j < kC15Slices; ++j) push_bf16(wv[j], sl[j]);
+            if constexpr (!kC1Only) {
+                slice6(lp, El, sl);
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int mu = ao_s[ks * TC_K + c8 * 8 + 2 * q2 + h];
-                    int sh;
-                    float2 v = make_float2(0.f, 0.f), lp = make_float2(0.f, 0.f);
-                    if (active(mu, sh)) ao_val_lap_ff(s, a.fb, mu, r2, v, lp);
-                    slice6(v, Ev, sv[h]);
-                    slice6(lp, El, sl[h]);
-                }
-#pragma unroll
-                for (int j = 0; j < kC15Slices; ++j) {
-                    wv[j][q2] = bf16_pair(sv[0][j], sv[1][j]);
-                    wl[j][q2] = bf16_pair(sl[0][j], sl[1][j]);
-                }
-            }
-            const uint32_t off = a_off64(row, c8 & 3);
-            unsigned char *stp = pl + (size_t)(2 * ks + (c8 >> 2)) * kStageBytes;
-#pragma unroll
-            for (int j = 0; j < kC15Slices; ++j) {
-                *reinterpret_cast<uint4 *>(stp + (size_t)j * kSPlaneBytes + off) =
-                    make_uint4(wv[j][0], wv[j][1], wv[j][2], wv[j][3]);
-                *reinterpret_cast<uint4 *>(stp + (size_t)(kC15Slices + j) * kSPlaneBytes + off) =
-                    make_uint4(wl[j][0], wl[j][1], wl[j][2], wl[j][3]);
+                for (int j = 0; j < kC15Slices; ++j) push_bf16(wl[j], sl[j]);
             }
         }
+        unsigned char *stp = pl + (size_t)(c8 >> 2) * stage_bytes + a_off64(row, c8 & 3);
+#pragma unroll
+        for (int j = 0; j < kC15Slices; ++j) {
+            *reinterpret_cast<uint4 *>(stp + (size_t)j * pbytes) = make_uint4(wv[j][0], wv[j][1], wv[j][2], wv[j][3]);
+            if constexpr (!kC1Only)
+                *reinterpret_cast<uint4 *>(stp + (size_t)(kC15Slices + j) * pbytes) =
+                    make_uint4(wl[j][0], wl[j][1], wl[j][2], wl[j][3]);
+        }
+    }
 }
 
 // Bounded wait of a whole warp, which stays converged (every lane polls; the phase, once
@@ -409,8 +445,10 @@ __global__ void __launch_bounds__(kMmaThreads, 1) k_c15_mma(C15TcArgs a)
         // MO-coefficient rows by 16-byte cp.async; each lane waits for its own copies, makes
         // them visible to the tensor cores' proxy and arrives
         const int cl = t - 32 * kMmaEpWarps;                 // 0 .. 32 * kMmaCpWarps - 1
-        const unsigned char *Ag = a.planes + slot * (size_t)a.kmax_steps * kStepBytes +
-                                  (size_t)o * kC15Slices * kSPlaneBytes;     // o = 2: the gradient planes
+        const uint32_t pbytes = (uint32_t)a.prows * (SK * 2);
+        const size_t stage_bytes = (size_t)a.planes_per_stage * pbytes;
+        const unsigned char *Ag = a.planes + slot * (size_t)a.kmax_steps * 2 * stage_bytes +
+                                  (size_t)o * kC15Slices * pbytes;           // o = 2: the gradient planes
         const int nbplanes = grad ? 2 : kC15Slices;
         const uint16_t *__restrict__ Bsl = a.slice[spin];
         const size_t slice_stride = (size_t)s.n_ao * nspad;
@@ -419,8 +457,13 @@ __global__ void __launch_bounds__(kMmaThreads, 1) k_c15_mma(C15TcArgs a)
             if (sg >= 2 && !c15_wait_warp(EMPTY(buf), ((sg >> 1) - 1) & 1, kWait, &s_abort, lane)) break;
             unsigned char *Ab = base + buf * kBufBytes, *Bb = Ab + kC15Slices * kSPlaneBytes;
             if (cl == 0) {
-                mbar_expect_tx(FULL(buf), kC15Slices * kSPlaneBytes);
-                bulk_g2s(smem_u32(Ab), Ag + (size_t)sg * kStageBytes, kC15Slices * kSPlaneBytes, FULL(buf));
+                mbar_expect_tx(FULL(buf), kC15Slices * pbytes);
+                if (pbytes == kSPlaneBytes)
+                    bulk_g2s(smem_u32(Ab), Ag + (size_t)sg * stage_bytes, kC15Slices * kSPlaneBytes, FULL(buf));
+                else            // a single tile's short planes; the rows past them feed only unread TMEM lanes
+                    for (int j = 0; j < kC15Slices; ++j)
+                        bulk_g2s(smem_u32(Ab + j * kSPlaneBytes), Ag + (size_t)sg * stage_bytes + (size_t)j * pbytes,
+                                 pbytes, FULL(buf));
             }
             for (int q = cl; q < nbplanes * SK * (TC_N / 8); q += 32 * kMmaCpWarps) {
                 const int j = q / (SK * (TC_N / 8));
@@ -618,28 +661,66 @@ bool c15tc_fits(const SysDev &s, int mw)
     return nmax <= 1024 && mw <= 256 && sm_mma <= 227 * 1024 && sm_prep <= 227 * 1024;
 }
 
-// Electrons per producer / MMA launch pair: enough CTAs per launch for large
-// batches of walkers (fewer launches, so fewer partly filled last waves), a
-// small staging buffer for small ones; spread evenly over the launches.
-size_t c15tc_batch(int n_elec, int n_tiles)
+// The staging of one (electron, walker tile): operand planes, AO list, row exponents.
+struct C15Slot {
+    int prows, planes;
+    size_t kmax, plane_bytes, bytes;
+};
+
+static C15Slot c15tc_slot(const SysDev &s, int nw, bool c1_only)
 {
-    const int b = n_tiles >= 8 ? 128 : (n_tiles >= 2 ? 32 : 16);
-    if (n_elec <= b) return (size_t)(n_elec > 0 ? n_elec : 1);
-    const int nl = (n_elec + b - 1) / b;                   // launches, then the electrons spread evenly
-    return (size_t)((n_elec + nl - 1) / nl);
+    C15Slot l;
+    l.prows = nw >= TC_M ? TC_M : (nw + 7) / 8 * 8;
+    l.planes = c1_only ? kC15Slices : kPlanesPerStep;
+    l.kmax = (size_t)(s.n_ao + TC_K - 1) / TC_K;
+    l.plane_bytes = l.kmax * 2 * l.planes * l.prows * (SK * 2);
+    l.bytes = l.plane_bytes + l.kmax * TC_K * 4 + 4 + TC_M * 2 * 4;
+    return l;
 }
 
-size_t c15tc_bytes(const SysDev &s, int nw)
+// Electrons per producer / MMA launch pair, spread evenly over the launches.  The least that
+// a workspace must hold: a few electrons for few walker tiles (one walker's scratch stays
+// small); never smaller for more tiles, so what holds a walker chunk holds a shorter one.
+static size_t c15tc_spread(int n_elec, size_t b)
+{
+    if ((size_t)n_elec <= b) return (size_t)(n_elec > 0 ? n_elec : 1);
+    const size_t nl = (n_elec + b - 1) / b;                // launches, then the electrons spread evenly
+    return (n_elec + nl - 1) / nl;
+}
+
+static size_t c15tc_least(int n_elec, int n_tiles)
+{
+    return c15tc_spread(n_elec, n_tiles >= 8 ? 128 : (n_tiles >= 2 ? 32 : 16));
+}
+
+// The batch that fills the card: a launch of 2048 (electron, tile) pairs is at least four
+// waves of the producer's three CTAs on each of 152 SMs (at 1056 electrons x 37 walkers,
+// batches of 16 left the producer 16 CTAs a launch: 46.8 ms in 66 launches), within 8 GiB.
+static size_t c15tc_want(const SysDev &s, int nw, bool c1_only)
 {
     const size_t tiles = (size_t)(nw + TC_M - 1) / TC_M;
-    const size_t kmax = (size_t)(s.n_ao + TC_K - 1) / TC_K;
-    const size_t per = kmax * kStepBytes + kmax * TC_K * 4 + 4 + TC_M * 2 * 4;
-    return c15tc_batch(s.n_elec, (int)tiles) * tiles * per + 4096;
+    const size_t room = (size_t(8) << 30) / (tiles * c15tc_slot(s, nw, c1_only).bytes);
+    const size_t b = std::min((2048 + tiles - 1) / tiles, std::max(room, size_t(1)));
+    return std::max(c15tc_least(s.n_elec, (int)tiles), c15tc_spread(s.n_elec, b));
+}
+
+size_t c15tc_bytes(const SysDev &s, int nw, bool c1_only, bool want)
+{
+    const size_t tiles = (size_t)(nw + TC_M - 1) / TC_M;
+    const size_t b = want ? c15tc_want(s, nw, c1_only) : c15tc_least(s.n_elec, (int)tiles);
+    return b * tiles * c15tc_slot(s, nw, c1_only).bytes + 4096;
+}
+
+size_t c15tc_tile_bytes(const SysDev &s, int nw)
+{
+    const size_t tiles = (size_t)(nw + TC_M - 1) / TC_M;
+    return c15tc_least(s.n_elec, (int)tiles) * tiles * c15tc_slot(s, TC_M, false).bytes + 4096;
 }
 
 cudaError_t launch_c15_tc(const SysDev &s, const FfBasis &fb, const MixedTables &mt, const TcTables &tt, int nw,
                           const double *R, const uint32_t *masks, int mw, double *X, double *L5, float *Cg,
-                          uint32_t *wstatus, void *scratch, cudaStream_t st, const WaitCfg &wc, bool c1_only)
+                          uint32_t *wstatus, void *scratch, size_t scratch_bytes, cudaStream_t st, const WaitCfg &wc,
+                          bool c1_only)
 {
     if (nw == 0) return cudaSuccess;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
@@ -650,11 +731,17 @@ cudaError_t launch_c15_tc(const SysDev &s, const FfBasis &fb, const MixedTables 
     a.R = R; a.masks = masks; a.mw = mw; a.nw = nw;
     a.n_tiles = (nw + TC_M - 1) / TC_M;
     a.kmax_steps = (s.n_ao + TC_K - 1) / TC_K;
-    const size_t nb = c15tc_batch(s.n_elec, a.n_tiles);
+    const C15Slot sl = c15tc_slot(s, nw, c1_only);
+    a.prows = sl.prows;
+    a.planes_per_stage = sl.planes;
+    // as many electrons per launch as the scratch holds, up to the batch that fills the card
+    if (scratch_bytes < c15tc_bytes(s, nw, c1_only, false)) return cudaErrorMemoryAllocation;
+    const size_t room = (scratch_bytes - 4096) / ((size_t)a.n_tiles * sl.bytes);
+    const size_t nb = std::min(c15tc_want(s, nw, c1_only), c15tc_spread(s.n_elec, room));
     char *p = static_cast<char *>(scratch);
     const size_t ntl = nb * a.n_tiles;
     a.planes = reinterpret_cast<unsigned char *>(p);
-    p += ntl * a.kmax_steps * kStepBytes;
+    p += ntl * sl.plane_bytes;
     a.ao_list = reinterpret_cast<int *>(p);
     p += ntl * a.kmax_steps * TC_K * 4;
     a.nks = reinterpret_cast<int *>(p);

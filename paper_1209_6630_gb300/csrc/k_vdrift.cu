@@ -27,6 +27,8 @@
 // (float-float, radial part once per shell) of the AO at r_e, multiplied by v
 // and accumulated as float pairs on the FP32 pipes.
 // Output vd[w][e] = (drift_x, drift_y, drift_z, lap_e).
+#include <algorithm>
+
 #include "ao_ff.cuh"
 #include "qmc_internal.cuh"
 #include "slices.cuh"
@@ -64,6 +66,7 @@ struct VdArgs {
     int e0;                        // first electron of this launch's batch
     unsigned char *astage;         // per CTA of the batch: the sliced D^-1 rows, one A image per K stage
     size_t astage_per;             // bytes per CTA
+    int prows;                     // rows of a staged plane: 128, or a single tile's walkers rounded up to 8
 };
 
 __global__ void k_vd_rowexp(int nw, int n_up, int n_dn, size_t msz, const double *__restrict__ Dinv,
@@ -81,6 +84,26 @@ __global__ void k_vd_rowexp(int nw, int n_up, int n_dn, size_t msz, const double
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) rexp[row] = exp_bound(m);
+}
+
+// The four order sums of 16 columns of this warp's TMEM lanes (integers in their units) added
+// as float pairs: column c0 + q to out[q * ld].
+__device__ __forceinline__ void vd_sums(uint32_t tmem_lanes, int c0, float2 *out, int ld)
+{
+    uint32_t v0[16], v1[16], v2[16], v3[16];
+    tmem_ld16(tmem_lanes + (uint32_t)(0 * kVdN + c0), v0);
+    tmem_ld16(tmem_lanes + (uint32_t)(1 * kVdN + c0), v1);
+    tmem_ld16(tmem_lanes + (uint32_t)(2 * kVdN + c0), v2);
+    tmem_ld16(tmem_lanes + (uint32_t)(3 * kVdN + c0), v3);
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        float s, e, s2, e2;
+        ff::two_sum(__uint_as_float(v0[q]), __uint_as_float(v1[q]), s, e);
+        ff::two_sum(s, __uint_as_float(v2[q]), s2, e2);
+        e = __fadd_rn(e, e2);
+        ff::two_sum(s2, __uint_as_float(v3[q]), s, e2);
+        out[q * ld] = ff::renorm(s, __fadd_rn(e, e2));
+    }
 }
 
 // Two CTAs per SM (256 threads, N = 64 AOs per tile, one operand stage of
@@ -107,13 +130,13 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
     const int mw = a.mw;
 
     // union of the tile's active shells for electron e, and its AO list
-    for (int j = t; j < mw; j += kVdThreads) {
-        uint32_t u = 0;
-        for (int m = 0; m < TC_M; ++m) {
-            const int w = tile * TC_M + m;
-            if (w < a.nw) u |= a.masks[((size_t)w * N + e) * mw + j];
-        }
-        un_s[j] = u;
+    const int rv = min(TC_M, a.nw - tile * TC_M);             // walkers of this tile
+    for (int j = t; j < mw; j += kVdThreads) un_s[j] = 0;
+    __syncthreads();
+    for (int q = t; q < rv * mw; q += kVdThreads) {           // independent loads: a word each
+        const int m = q / mw, j = q - m * mw;
+        const uint32_t u = a.masks[((size_t)(tile * TC_M + m) * N + e) * mw + j];
+        if (u) atomicOr(&un_s[j], u);
     }
     __syncthreads();
     const int K = aos_from_mask_n(s, un_s, mw, ao_s, warp_s);
@@ -144,7 +167,8 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
 
     // this CTA's D^-1 rows cut into six exact slices once, for every K stage (the AO tiles
     // reuse them): thread -> (row, chunk of 8 MOs), two per thread
-    for (int q = t; q < TC_M * 4; q += kVdThreads) {
+    const uint32_t pbytes = (uint32_t)a.prows * (kVdK * 2);   // a staged plane's rows (the others feed unread lanes)
+    for (int q = t; q < a.prows * 4; q += kVdThreads) {
         const int prow = q >> 2, pc = q & 3;
         const int pw = tile * TC_M + prow;
         const bool pvalid = pw < a.nw;
@@ -160,10 +184,10 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
                 const double d = (pvalid && k < ns) ? drow[k] : 0.0;
                 slice6(ff::from_double(d), Ep, sl[i]);
             }
-            unsigned char *Ad = ast + (size_t)sg * kC15Slices * kVdPlane;
+            unsigned char *Ad = ast + (size_t)sg * kC15Slices * pbytes;
 #pragma unroll
             for (int j = 0; j < kC15Slices; ++j)
-                *reinterpret_cast<uint4 *>(Ad + j * kVdPlane + a_off64(prow, pc)) =
+                *reinterpret_cast<uint4 *>(Ad + j * pbytes + a_off64(prow, pc)) =
                     make_uint4(bf16_pair(sl[0][j], sl[1][j]), bf16_pair(sl[2][j], sl[3][j]),
                                bf16_pair(sl[4][j], sl[5][j]), bf16_pair(sl[6][j], sl[7][j]));
         }
@@ -173,10 +197,20 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
     const uint32_t cb = smem_u32(&cbar);
     int ncopy = 0;
 
-    // epilogue role: walker row erow (TMEM lane), columns cg * 32 .. + 32 of an AO tile of 64
-    const int erow = (warp & 3) * 32 + lane, cg = warp >> 2;
+    // epilogue role: a full tile has walker row erow (TMEM lane), columns cg * 32 .. + 32 of an AO
+    // tile of 64.  A tile of at most 64 walkers hands the columns of a row to 256 / rp threads
+    // (rp: the power of two that holds the rows), each a run of 64 rp / 256 of them, through
+    // shared memory: the AO derivatives of one walker's column group are a serial chain, and most
+    // lanes have no row there (1056 electrons x 37 walkers, with all electrons in one launch:
+    // 16.8 -> 2.8 ms).
+    const int lrp = 32 - __clz(rv - 1);                       // rv = 1: __clz(0) = 32
+    const bool small = lrp < 7;
+    const int erow = small ? t & ((1 << lrp) - 1) : (warp & 3) * 32 + lane;
+    const int cg = small ? t >> lrp : warp >> 2;              // column group
+    const int ncg = small ? kVdThreads >> lrp : 2;            // column groups, each of len columns
+    const int len = small ? max(1, kVdN >> (8 - lrp)) : 32;
     const int ew = tile * TC_M + erow;
-    const bool evalid = ew < a.nw;
+    const bool evalid = erow < rv;
     const int Ee = evalid ? a.rexp[(size_t)ew * N + e] : 0;
     const double *rw = a.R + ((size_t)(evalid ? ew : 0) * N + e) * 3;
     const float2 r2[3] = {ff::from_double(rw[0]), ff::from_double(rw[1]), ff::from_double(rw[2])};
@@ -194,10 +228,13 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
         for (int sg = 0; sg < nst; ++sg) {
             // the stage buffer: A (the staged D^-1 slices) and B (the rows of A of this AO tile)
             const int k0 = sg * kVdK;
-            const unsigned char *As = ast + (size_t)sg * kC15Slices * kVdPlane;
+            const unsigned char *As = ast + (size_t)sg * kC15Slices * pbytes;
             if (t == 0) {                                  // the staged D^-1 slices: one bulk copy
-                mbar_expect_tx(cb, kC15Slices * kVdPlane);
-                bulk_g2s(smem_u32(Ab), As, kC15Slices * kVdPlane, cb);
+                mbar_expect_tx(cb, kC15Slices * pbytes);
+                if (pbytes == kVdPlane) bulk_g2s(smem_u32(Ab), As, kC15Slices * kVdPlane, cb);
+                else
+                    for (int j = 0; j < kC15Slices; ++j)
+                        bulk_g2s(smem_u32(Ab + j * kVdPlane), As + (size_t)j * pbytes, pbytes, cb);
             }
             for (int q = t; q < kC15Slices * kVdN * 4; q += kVdThreads) {
                 const int j = q / (kVdN * 4), rem = q - j * (kVdN * 4);
@@ -248,35 +285,31 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
         // epilogue: v for 32 AOs of this walker row, then the AO derivatives at r_e
         FfRadial rd;
         int last_sh = -1;
-        float2 *vbuf = reinterpret_cast<float2 *>(base);   // [16][256]: the stage buffer is idle here
-        for (int h = 0; h < 2; ++h) {
-            const int c0 = cg * 32 + h * 16;
-            {
-                uint32_t v0[16], v1[16], v2[16], v3[16];
-                tmem_ld16(tmem + tlane + (uint32_t)(0 * kVdN + c0), v0);
-                tmem_ld16(tmem + tlane + (uint32_t)(1 * kVdN + c0), v1);
-                tmem_ld16(tmem + tlane + (uint32_t)(2 * kVdN + c0), v2);
-                tmem_ld16(tmem + tlane + (uint32_t)(3 * kVdN + c0), v3);
-                // the four order sums (integers in their units) added as a float pair
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    float s, e, s2, e2;
-                    ff::two_sum(__uint_as_float(v0[q]), __uint_as_float(v1[q]), s, e);
-                    ff::two_sum(s, __uint_as_float(v2[q]), s2, e2);
-                    e = __fadd_rn(e, e2);
-                    ff::two_sum(s2, __uint_as_float(v3[q]), s, e2);
-                    vbuf[q * kVdThreads + t] = ff::renorm(s, __fadd_rn(e, e2));
-                }
-            }
+        // the stage buffer is idle here: [16][256] of the threads' own columns, or [64][64 rows]
+        float2 *vbuf = reinterpret_cast<float2 *>(base);
+        const int vld = small ? TC_M / 2 : kVdThreads;
+        if (small) {
+            const int lrow = (warp & 3) * 32 + lane;       // TMEM lane
+            if ((warp & 3) * 32 < rv)                      // (whole warps)
+                for (int h = 0; h < 2; ++h)
+                    vd_sums(tmem + tlane, (warp >> 2) * 32 + h * 16, vbuf + ((warp >> 2) * 32 + h * 16) * vld + lrow, vld);
+            __syncthreads();
+        }
+        for (int h = 0; h < (small ? 1 : 2); ++h) {
+            const int c0 = small ? cg * len : cg * 32 + h * 16;
+            const float2 *vcol = small ? vbuf + c0 * vld + erow : vbuf + t;
+            if (!small) vd_sums(tmem + tlane, c0, vbuf + t, vld);
             if (!evalid) continue;
+            const int nq = small ? len : 16;
 #pragma unroll 1
-            for (int q = 0; q < 16; ++q) {
+            for (int q = 0; q < nq; ++q) {
+                if (c0 + q >= kVdN) break;                 // (rp <= 2: more threads than columns)
                 const int mu = ao_s[at * kVdN + c0 + q];
                 if (mu < 0) break;
                 const int sh = s.ao_shell[mu];
                 if (!((my_mask[sh >> 5] >> (sh & 31)) & 1u)) continue;
                 const int ex = Ee + a.gexp[spin][mu];
-                const float2 vr = vbuf[q * kVdThreads + t];
+                const float2 vr = vcol[q * vld];
                 const float2 vmu = make_float2(scale_pow2(vr.x, ex), scale_pow2(vr.y, ex));   // exact scaling
                 if (sh != last_sh) {
                     last_sh = sh;
@@ -307,6 +340,7 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
                 lap = ff::fma2(lap, vmu, lp);
             }
         }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // vbuf before the next tile's bulk copy
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();                                   // TMEM and vbuf read before the next tile
     }
@@ -319,20 +353,21 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" :: "r"(tmem) : "memory");
-    // the two column groups' partial sums of each row, added in a fixed order
-    double *red = reinterpret_cast<double *>(base);        // [2 groups][128 rows][4]; operands no longer read
-    red[((size_t)cg * TC_M + erow) * 4 + 0] = ff::val(b0);
-    red[((size_t)cg * TC_M + erow) * 4 + 1] = ff::val(b1);
-    red[((size_t)cg * TC_M + erow) * 4 + 2] = ff::val(b2);
-    red[((size_t)cg * TC_M + erow) * 4 + 3] = ff::val(lap);
+    // the column groups' partial sums of each row, added in a fixed order
+    double *red = reinterpret_cast<double *>(base);        // [groups][rows][4]; operands no longer read
+    const int rows = kVdThreads / ncg;                     // 128, or rp
+    double *mine = red + ((size_t)cg * rows + erow) * 4;
+    mine[0] = ff::val(b0);
+    mine[1] = ff::val(b1);
+    mine[2] = ff::val(b2);
+    mine[3] = ff::val(lap);
     __syncthreads();
-    for (int q = t; q < TC_M * 4; q += kVdThreads) {
+    for (int q = t; q < rv * 4; q += kVdThreads) {
         const int r = q >> 2, c = q & 3;
         const int w = tile * TC_M + r;
-        if (w < a.nw) {
-            const double x = red[((size_t)0 * TC_M + r) * 4 + c] + red[((size_t)1 * TC_M + r) * 4 + c];
-            a.vd[((size_t)w * N + e) * 4 + c] = ok ? x : __longlong_as_double(0x7ff8000000000000ll);
-        }
+        double x = red[(size_t)r * 4 + c];
+        for (int g = 1; g < ncg; ++g) x += red[((size_t)g * rows + r) * 4 + c];
+        a.vd[((size_t)w * N + e) * 4 + c] = ok ? x : __longlong_as_double(0x7ff8000000000000ll);
     }
 }
 
@@ -344,37 +379,61 @@ bool vdrift_fits(const SysDev &s)
     return sm <= 227 * 1024;
 }
 
-// electrons per launch (the A staging holds one image per CTA of a batch): up to 264 from 2
-// walker tiles on (fewer launches, so fewer partly filled last waves), else up to 64 (one
-// walker's scratch stays small); spread evenly over the launches.  Never smaller for more
-// tiles, so the staging carved for a walker chunk holds a shorter one's.
-int vdrift_batch(const SysDev &s, int tiles)
+// Electrons per launch (the A staging holds one image per CTA of a batch), spread evenly over
+// the launches.  The least that a workspace must hold: up to 264 from 2 walker tiles on, else
+// up to 64 (one walker's scratch stays small); never smaller for more tiles, so what holds a
+// walker chunk holds a shorter one.
+static int vdrift_spread(int n_elec, size_t b)
 {
-    const int kMax = tiles >= 2 ? 264 : 64;
-    if (s.n_elec <= kMax) return s.n_elec;
-    const int nl = (s.n_elec + kMax - 1) / kMax;
-    return (s.n_elec + nl - 1) / nl;
+    if ((size_t)n_elec <= b) return n_elec;
+    const int nl = (int)((n_elec + b - 1) / b);
+    return (n_elec + nl - 1) / nl;
 }
 
-size_t vdrift_stage_per(const SysDev &s)
+static int vdrift_least(const SysDev &s, int tiles) { return vdrift_spread(s.n_elec, tiles >= 2 ? 264 : 64); }
+
+static size_t vdrift_stage_per(const SysDev &s, int nw)
 {
     const int nsmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     const size_t nst = (size_t)((nsmax + 63) / 64 * 64) / kVdK;
-    return nst * kC15Slices * kVdPlane;
+    const size_t prows = nw >= TC_M ? TC_M : (nw + 7) / 8 * 8;
+    return nst * kC15Slices * prows * (kVdK * 2);
 }
 
-size_t vdrift_bytes(const SysDev &s, int nw)
+// The batch that fills the card: 2432 (electron, tile) pairs are eight waves of two CTAs on
+// each of 152 SMs, within 4 GiB.
+static int vdrift_want(const SysDev &s, int nw)
 {
     const size_t tiles = (size_t)(nw + TC_M - 1) / TC_M;
-    return ((sizeof(int) * (size_t)nw * s.n_elec + 255) / 256) * 256 +
-           tiles * (size_t)vdrift_batch(s, (int)tiles) * vdrift_stage_per(s);
+    const size_t room = (size_t(4) << 30) / (tiles * std::max(vdrift_stage_per(s, nw), size_t(1)));
+    const size_t b = std::min((2432 + tiles - 1) / tiles, std::max(room, size_t(1)));
+    return std::max(vdrift_least(s, (int)tiles), vdrift_spread(s.n_elec, b));
+}
+
+static size_t vdrift_head(const SysDev &s, int nw)           // the row exponents of D^-1
+{
+    return ((sizeof(int) * (size_t)nw * s.n_elec + 255) / 256) * 256;
+}
+
+size_t vdrift_bytes(const SysDev &s, int nw, bool want)
+{
+    const size_t tiles = (size_t)(nw + TC_M - 1) / TC_M;
+    return vdrift_head(s, nw) +
+           tiles * (size_t)(want ? vdrift_want(s, nw) : vdrift_least(s, (int)tiles)) * vdrift_stage_per(s, nw);
+}
+
+size_t vdrift_tile_bytes(const SysDev &s, int nw)
+{
+    const size_t tiles = (size_t)(nw + TC_M - 1) / TC_M;
+    return vdrift_head(s, nw) + tiles * (size_t)vdrift_least(s, (int)tiles) * vdrift_stage_per(s, TC_M);
 }
 
 cudaError_t launch_vdrift(const SysDev &s, const FfBasis &fb, const MixedTables &mt, int nw, const double *R,
                           const uint32_t *masks, int mw, const double *Dinv, double *vd, uint32_t *wstatus,
-                          void *scratch, cudaStream_t st, const WaitCfg &wc)
+                          void *scratch, size_t scratch_bytes, cudaStream_t st, const WaitCfg &wc)
 {
     if (nw == 0) return cudaSuccess;
+    if (scratch_bytes < vdrift_bytes(s, nw, false)) return cudaErrorMemoryAllocation;
     if (!vdrift_fits(s)) return cudaErrorInvalidConfiguration;
     VdArgs a;
     a.s = s; a.fb = fb; a.R = R; a.masks = masks; a.mw = mw; a.nw = nw; a.Dinv = Dinv;
@@ -388,8 +447,9 @@ cudaError_t launch_vdrift(const SysDev &s, const FfBasis &fb, const MixedTables 
     a.vd = vd;
     a.wstatus = wstatus;
     a.pgf = mt.pgf; a.pcf = mt.pcf; a.scf = mt.scf; a.Qhi = mt.Qhi; a.Qlo = mt.Qlo;
-    a.astage = static_cast<unsigned char *>(scratch) + ((sizeof(int) * (size_t)nw * s.n_elec + 255) / 256) * 256;
-    a.astage_per = vdrift_stage_per(s);
+    a.astage = static_cast<unsigned char *>(scratch) + vdrift_head(s, nw);
+    a.astage_per = vdrift_stage_per(s, nw);
+    a.prows = nw >= TC_M ? TC_M : (nw + 7) / 8 * 8;
     a.wait_ns = wc.limit_ns;
     const size_t rows = (size_t)nw * s.n_elec;
     k_vd_rowexp<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(nw, s.n_up, s.n_dn, a.msz, Dinv,
@@ -398,7 +458,9 @@ cudaError_t launch_vdrift(const SysDev &s, const FfBasis &fb, const MixedTables 
     cudaError_t e = cudaFuncSetAttribute(k_vd_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     const int tiles = (nw + TC_M - 1) / TC_M;
-    const int nb = vdrift_batch(s, tiles);
+    // as many electrons per launch as the scratch holds, up to the batch that fills the card
+    const size_t room = (scratch_bytes - vdrift_head(s, nw)) / (tiles * std::max(a.astage_per, size_t(1)));
+    const int nb = std::min(vdrift_want(s, nw), vdrift_spread(s.n_elec, std::max(room, size_t(1))));
     for (int e0 = 0; e0 < s.n_elec; e0 += nb) {
         a.e0 = e0;
         const int ne = s.n_elec - e0 < nb ? s.n_elec - e0 : nb;

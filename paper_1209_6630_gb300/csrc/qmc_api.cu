@@ -751,8 +751,16 @@ Plan make_plan(const qmc_system *sys, int precision, bool need_dinv, int c15_ove
 
 struct Carve {
     double *X; void *Cd; double *L5; double *D; double *la; double *sg; uint32_t *st; uint32_t *masks;
-    float2 *work; uint8_t *redo; void *redo_scratch; void *c15tc; void *gjtc; double *vd; void *vdscr;
+    float2 *work; uint8_t *redo; void *redo_scratch; void *gjtc; double *vd;
+    // staging of the tensor-core products, then of the C-free drift (one after the other): what is left
+    void *stage; size_t stage_bytes;
 };
+
+// The staging of nw walkers: the least that works, or what lets each launch fill the card.
+size_t stage_for(const Plan &p, int nw, bool want)
+{
+    return std::max(p.c15tc ? c15tc_bytes(*p.sd, nw, p.cfree, want) : 0, p.cfree ? vdrift_bytes(*p.sd, nw, want) : 0);
+}
 
 // Arrays for `nw` walkers laid out array by array inside ws.
 bool carve(const Plan &p, int nw, void *ws, size_t ws_bytes, Carve &c)
@@ -762,12 +770,10 @@ bool carve(const Plan &p, int nw, void *ws, size_t ws_bytes, Carve &c)
     auto take = [&](size_t bytes) { char *r = b + o; o = al(o + bytes); return r; };
     c.X = reinterpret_cast<double *>(take(p.msz * 8 * nw));
     c.vd = nullptr;
-    c.vdscr = nullptr;
     if (p.cfree) {
         c.Cd = nullptr;
         c.L5 = nullptr;
         c.vd = reinterpret_cast<double *>(take(p.cd_bytes * nw));
-        c.vdscr = take(vdrift_bytes(*p.sd, nw));
     } else if (p.mixed) {
         c.Cd = take(p.msz * 3 * 4 * nw);
         c.L5 = reinterpret_cast<double *>(take(p.msz * 8 * nw));
@@ -784,29 +790,52 @@ bool carve(const Plan &p, int nw, void *ws, size_t ws_bytes, Carve &c)
     c.work = (p.ffgj && !p.tcgj) ? reinterpret_cast<float2 *>(take(p.msz * 8 * nw)) : nullptr;
     c.redo = p.ffgj ? reinterpret_cast<uint8_t *>(take(2 * (size_t)nw)) : nullptr;
     c.redo_scratch = p.ffgj ? take(p.redo_bytes) : nullptr;
-    c.c15tc = p.c15tc ? take(c15tc_bytes(*p.sd, nw)) : nullptr;
     c.gjtc = p.tcgj ? take(gjtc_bytes(p.sd->n_up, p.sd->n_dn, nw)) : nullptr;
-    return o <= ws_bytes;
+    c.stage = b + o;
+    c.stage_bytes = o <= ws_bytes ? ws_bytes - o : 0;
+    return o + stage_for(p, nw, false) <= ws_bytes;
 }
 
-size_t bytes_for(const Plan &p, int nw)
+// The arrays of nw walkers without the staging.
+size_t array_bytes(const Plan &p, int nw)
 {
     size_t o = al(p.msz * 8 * nw);
-    if (p.cfree) o += al(p.cd_bytes * nw) + al(vdrift_bytes(*p.sd, nw));
+    if (p.cfree) o += al(p.cd_bytes * nw);
     else o += p.mixed ? al(p.msz * 3 * 4 * nw) + al(p.msz * 8 * nw) : al(p.msz * 4 * 8 * nw);
     o += p.dinv ? al(p.msz * 8 * nw) : 0;
     o += al(16 * (size_t)nw) * 2 + al(4 * (size_t)nw);
     o += p.mask_bytes ? al(p.mask_bytes * nw) : 0;
     o += (p.ffgj && !p.tcgj) ? al(p.msz * 8 * nw) : 0;
     o += p.ffgj ? al(2 * (size_t)nw) + al(p.redo_bytes) : 0;
-    o += p.c15tc ? al(c15tc_bytes(*p.sd, nw)) : 0;
     o += p.tcgj ? al(gjtc_bytes(p.sd->n_up, p.sd->n_dn, nw)) : 0;
     return o;
 }
 
-int chunk_walkers(const Plan &p, int W, size_t ws_bytes)
+// The rule by which a workspace holds nw walkers (the least that is accepted for them): the
+// arrays and a staging of full 128-row tiles, one for the products and one for the drift.
+// stage_for needs less, but the rule stays: the tiles of 128 walkers start at a chunk's first
+// walker, and the FP32 sums of C2..C4 depend on which walkers share a tile, so a workspace of
+// a given size goes on giving the same chunks and results.
+size_t bytes_for(const Plan &p, int nw)
 {
-    int lo = 0, hi = std::min(W, 65535);
+    return array_bytes(p, nw) + (p.c15tc ? al(c15tc_tile_bytes(*p.sd, nw)) : 0) +
+           (p.cfree ? al(vdrift_tile_bytes(*p.sd, nw)) : 0);
+}
+
+// What the size queries report: room for launches that fill the card.
+size_t bytes_wanted(const Plan &p, int nw)
+{
+    return std::max(bytes_for(p, nw), array_bytes(p, nw) + al(stage_for(p, nw, true)));
+}
+
+// Walkers per chunk of a call of W walkers.  What bytes_wanted has beyond bytes_for does not
+// enter (q: the plan that the size query takes).
+int chunk_walkers(const Plan &p, const Plan &q, int W, size_t ws_bytes)
+{
+    const int Wq = std::min(W, 65535);
+    const size_t least = bytes_for(q, Wq), wanted = bytes_wanted(q, Wq);
+    ws_bytes = ws_bytes >= wanted ? ws_bytes - (wanted - least) : std::min(ws_bytes, least);
+    int lo = 0, hi = Wq;
     while (lo < hi) {
         const int mid = lo + (hi - lo + 1) / 2;
         if (bytes_for(p, mid) <= ws_bytes) lo = mid; else hi = mid - 1;
@@ -869,15 +898,15 @@ cudaError_t run_products(const qmc_system *sys, int precision, int nw, const dou
     tt.pgf = mt.pgf; tt.pcf = mt.pcf; tt.scf = mt.scf; tt.Qhi = mt.Qhi; tt.Qlo = mt.Qlo;
     if (p.cfree) {
         // the C-free variant: C1 alone here; drift and Laplacian after a4 (launch_vdrift)
-        e = launch_c15_tc(s, mt.ffb, mt, tt, nw, Rc, c.masks, mt.mask_words, c.X, nullptr, nullptr, c.st, c.c15tc,
-                          st, wc, true);
+        e = launch_c15_tc(s, mt.ffb, mt, tt, nw, Rc, c.masks, mt.mask_words, c.X, nullptr, nullptr, c.st, c.stage,
+                          c.stage_bytes, st, wc, true);
         if (e != cudaSuccess) return e;
         return mark(5);
     }
     if (p.c15tc) {
         // C1, C5 and C2..C4 from one producer pass per (electron, walker tile)
         e = launch_c15_tc(s, mt.ffb, mt, tt, nw, Rc, c.masks, mt.mask_words, c.X, c.L5,
-                          static_cast<float *>(c.Cd), c.st, c.c15tc, st, wc);
+                          static_cast<float *>(c.Cd), c.st, c.stage, c.stage_bytes, st, wc);
         if (e != cudaSuccess) return e;
         return mark(5);
     }
@@ -896,7 +925,7 @@ extern "C" int qmc_workspace_size(const qmc_system *sys, int n_walk, int precisi
     if (!sys || !bytes || n_walk < 0) return invalid("qmc_workspace_size: bad argument");
     if (precision < QMC_PREC_F64 || precision > QMC_PREC_F64_TCA4) return invalid("qmc_workspace_size: precision");
     const Plan p = make_plan(sys, precision, true);
-    *bytes = bytes_for(p, std::min(n_walk, 65535));
+    *bytes = bytes_wanted(p, std::min(n_walk, 65535));
     return QMC_OK;
 }
 
@@ -937,7 +966,7 @@ int eval_impl(const qmc_system *sys, int n_walk, const double *R, int precision,
         return invalid("qmc_walkers_eval: null required pointer");
     if (precision < QMC_PREC_F64 || precision > QMC_PREC_F64_TCA4) return invalid("qmc_walkers_eval: precision");
     const Plan p = make_plan(sys, precision, out->dinv == nullptr);
-    const int chunk = chunk_walkers(p, n_walk, ws_bytes);
+    const int chunk = chunk_walkers(p, make_plan(sys, precision, true), n_walk, ws_bytes);
     if (chunk < 1) {
         set_error("qmc_walkers_eval: workspace smaller than one walker");
         return QMC_ERR_CAPACITY;
@@ -1005,7 +1034,7 @@ int eval_impl(const qmc_system *sys, int n_walk, const double *R, int precision,
         if ((e = mark(2)) != cudaSuccess) return cuda_fail(e, "qmc_walkers_eval: event");
         if (p.cfree) {
             e = launch_vdrift(s, sys->mixed.ffb, sys->mixed, nw, Rc, c.masks, sys->mixed.mask_words, Dinv, c.vd, c.st,
-                              c.vdscr, st, wc);
+                              c.stage, c.stage_bytes, st, wc);
             if (e != cudaSuccess) return cuda_fail(e, "qmc_walkers_eval: C-free drift launch");
         }
         e = launch_drift_energy(s, nw, Rc, Dinv, cview(p, c), c.la, c.sg, c.st, *out, w0, st, sys->mixed.ffb.Q);
@@ -1062,7 +1091,7 @@ extern "C" int qmc_slater_matrices(const qmc_system *sys, int n_walk, const doub
     // all five matrices: the C-free variant's system computes them as the tensor-core mode does
     const Plan p = make_plan(sys, precision, false,
                              sys->tiles.c15_mode == QMC_C15_CFREE ? QMC_C15_TENSOR : sys->tiles.c15_mode);
-    const int chunk = chunk_walkers(p, n_walk, ws_bytes);
+    const int chunk = chunk_walkers(p, make_plan(sys, precision, true), n_walk, ws_bytes);
     if (chunk < 1) {
         set_error("qmc_slater_matrices: workspace smaller than one walker");
         return QMC_ERR_CAPACITY;
@@ -1340,7 +1369,8 @@ extern "C" int qmc_multidet_workspace_size(const qmc_system *const *dets, int n_
     if (rc) return rc;
     if (!bytes || n_walk < 0) return invalid("qmc_multidet_workspace_size: bad argument");
     size_t ev = 0;
-    for (int k = 0; k < n_det; ++k) ev = std::max(ev, bytes_for(make_plan(dets[k], precision, true), std::min(n_walk, 65535)));
+    for (int k = 0; k < n_det; ++k) 
+        ev = std::max(ev, bytes_wanted(make_plan(dets[k], precision, true), std::min(n_walk, 65535)));
     *bytes = md_own_bytes(n_det, n_walk, dets[0]->d.n_elec) + ev;
     return QMC_OK;
 }
@@ -1494,7 +1524,7 @@ extern "C" int qmc_dmc_workspace_size(const qmc_system *sys, int n_walk, int pre
     if (!sys || !bytes || n_walk < 0) return invalid("qmc_dmc_workspace_size: bad argument");
     if (precision < QMC_PREC_F64 || precision > QMC_PREC_F64_TCA4) return invalid("qmc_dmc_workspace_size: precision");
     const Plan p = make_plan(sys, precision, true);
-    *bytes = dmc_own_bytes(n_walk, sys->d.n_elec) + bytes_for(p, std::min(n_walk, 65535));
+    *bytes = dmc_own_bytes(n_walk, sys->d.n_elec) + bytes_wanted(p, std::min(n_walk, 65535));
     return QMC_OK;
 }
 
@@ -1584,10 +1614,10 @@ int check_segments(const qmc_segment *segs, int n_seg, int precision)
     return QMC_OK;
 }
 
-size_t seg_bytes(const qmc_segment &g, int precision)
+size_t seg_bytes(const qmc_segment &g, int precision, bool want)
 {
     const Plan p = make_plan(g.sys, precision, g.out.dinv == nullptr);
-    return al(bytes_for(p, std::max(g.n_walk, 1)));
+    return al(want ? bytes_wanted(p, std::max(g.n_walk, 1)) : bytes_for(p, std::max(g.n_walk, 1)));
 }
 
 }  // namespace
@@ -1598,7 +1628,7 @@ extern "C" int qmc_batch_workspace_size(const qmc_segment *segs, int n_seg, int 
     if (rc) return rc;
     if (!bytes) return invalid("qmc_batch_workspace_size: null bytes");
     size_t tot = 0;
-    for (int i = 0; i < n_seg; ++i) tot += seg_bytes(segs[i], precision);
+    for (int i = 0; i < n_seg; ++i) tot += seg_bytes(segs[i], precision, true);
     *bytes = tot;
     return QMC_OK;
 }
@@ -1608,8 +1638,12 @@ extern "C" int qmc_batch_eval(const qmc_segment *segs, int n_seg, int precision,
 {
     int rc = check_segments(segs, n_seg, precision);
     if (rc) return rc;
-    size_t need = 0;
-    for (int i = 0; i < n_seg; ++i) need += seg_bytes(segs[i], precision);
+    size_t need = 0, all = 0;
+    for (int i = 0; i < n_seg; ++i) {
+        need += seg_bytes(segs[i], precision, false);
+        all += seg_bytes(segs[i], precision, true);
+    }
+    const bool want = all <= ws_bytes;
     if (need > ws_bytes) {
         set_error("qmc_batch_eval: workspace smaller than qmc_batch_workspace_size");
         return QMC_ERR_CAPACITY;
@@ -1625,7 +1659,7 @@ extern "C" int qmc_batch_eval(const qmc_segment *segs, int n_seg, int precision,
             return cuda_fail(e, "qmc_batch_eval: fork wait");
     char *base = static_cast<char *>(ws);
     for (int i = 0; i < n_seg; ++i) {
-        const size_t b = seg_bytes(segs[i], precision);
+        const size_t b = seg_bytes(segs[i], precision, want);
         rc = eval_impl(segs[i].sys, segs[i].n_walk, segs[i].R, precision, &segs[i].out, base, b,
                        pool->st[i % kPoolStreams], nullptr);
         if (rc) return rc;

@@ -159,17 +159,20 @@ cudaError_t launch_c15_ff(const SysDev &s, const FfBasis &fb, int nw, const doub
                           int mw, const float2 *const *A, const int *ns32, const float *const *colmax,
                           double *X, double *L5, cudaStream_t st, int walkers_per_cta);
 bool c15tc_fits(const SysDev &s, int mw);
-size_t c15tc_bytes(const SysDev &s, int nw);
+// scratch of nw walkers: the least (want = false) or what lets one launch fill the card
+size_t c15tc_bytes(const SysDev &s, int nw, bool c1_only, bool want);
+size_t c15tc_tile_bytes(const SysDev &s, int nw);    // all 18 planes of full tiles: at least the least above
 cudaError_t launch_c15_tc(const SysDev &s, const FfBasis &fb, const MixedTables &mt, const TcTables &tt, int nw,
                           const double *R, const uint32_t *masks, int mw, double *X, double *L5, float *Cg,
-                          uint32_t *wstatus, void *scratch, cudaStream_t st, const WaitCfg &wc,
+                          uint32_t *wstatus, void *scratch, size_t scratch_bytes, cudaStream_t st, const WaitCfg &wc,
                           bool c1_only = false);
 // C-free variant: drift and Laplacian from v = D^-1 A^T (k_vdrift.cu)
 bool vdrift_fits(const SysDev &s);
-size_t vdrift_bytes(const SysDev &s, int nw);
+size_t vdrift_bytes(const SysDev &s, int nw, bool want);
+size_t vdrift_tile_bytes(const SysDev &s, int nw);   // full tiles: at least the least above
 cudaError_t launch_vdrift(const SysDev &s, const FfBasis &fb, const MixedTables &mt, int nw, const double *R,
                           const uint32_t *masks, int mw, const double *Dinv, double *vd, uint32_t *wstatus,
-                          void *scratch, cudaStream_t st, const WaitCfg &wc);
+                          void *scratch, size_t scratch_bytes, cudaStream_t st, const WaitCfg &wc);
 cudaError_t launch_tc_contract(const SysDev &s, int nw, const double *R, const uint32_t *masks, int mw,
                                const TcTables &tt, float *Cg, uint32_t *wstatus, cudaStream_t st, const WaitCfg &wc);
 cudaError_t launch_widen(const float *src, size_t spitch, double *dst, size_t dpitch, size_t width, int rows,
