@@ -33,9 +33,11 @@ METRIC = "walker-steps/s at 1056 e, mixed-prec vs FP64 GPU path, at <=1e-6 log|P
 
 
 def launches_per_step(q, prec, n_walk):
-    """Library kernels launched by one qmc_walkers_eval of a single walker chunk."""
+    """Library kernels launched by one qmc_walkers_eval of a single walker chunk: exact for the mixed
+    path from 8 walker tiles on (the default workload); with fewer tiles a workspace of the queried
+    size holds larger electron batches than counted here, and the FP64 path adds its drift kernel."""
     if prec == "f64":
-        return 3                      # contraction, Gauss-Jordan, energy
+        return 3                      # C1, Gauss-Jordan, energy
     t = q.tiles()
     n = 2                             # masks, energy
     if t["c15_mode"] in ("tensor", "cfree"):
@@ -221,7 +223,7 @@ def stage_roofline(q, prec, stage_mean, kbar, W, pk):
     fp32_inst_peak = 152 * 128 * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12      # T instructions/s
     t = q.tiles()
     if prec == "f64":
-        kern_ms = {"k_contract_f64": stage_mean[0], "k_gj": stage_mean[1], "k_drift_energy": stage_mean[2]}
+        kern_ms = {"k_c1_f64": stage_mean[0], "k_gj": stage_mean[1], "k_vd_f64+k_drift_energy": stage_mean[2]}
     else:
         a4_kern = {"float_float": "k_gj_ff+k_gj", "tensor": "k_gt_panel+k_gt_update+k_gj"}.get(t["a4_mode"], "k_gj")
         c15_kern = {"tensor": "k_c15_prep+k_c15_mma", "cfree": "k_c15_prep+k_c15_mma (C1)"}.get(t["c15_mode"],
@@ -235,9 +237,9 @@ def stage_roofline(q, prec, stage_mean, kbar, W, pk):
     if kern == "k_gj":
         roof = {"bound": "alu", "achieved": flop_a4 / ts / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
                 "peak_source": fp64_src, "work": "2 (N_up^3 + N_dn^3) flop per walker"}
-    elif kern == "k_contract_f64":
-        roof = {"bound": "alu", "achieved": flop_a3 / ts / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
-                "peak_source": fp64_src, "work": "10 sum_s N_s^2 Kbar flop per walker"}
+    elif kern in ("k_c1_f64", "k_vd_f64+k_drift_energy"):
+        roof = {"bound": "alu", "achieved": 2.0 * prod / ts / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
+                "peak_source": fp64_src, "work": "2 sum_s N_s^2 Kbar flop per walker (C1, or v = D^-1 A^T)"}
     elif kern == "k_gj_ff+k_gj":
         roof = {"bound": "alu", "achieved": flop_a4 / ts / 1e12, "peak": fp32_inst_peak / 6.0, "unit": "TFLOP/s",
                 "peak_source": "FP32 pipe (152 SMs x 128 lanes x sm_max_mhz) / 6: 12 FP32 instructions "

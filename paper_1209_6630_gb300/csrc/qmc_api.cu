@@ -717,6 +717,7 @@ struct Plan {
     size_t redo_bytes; // per chunk (float-float a4): list and state of the FP64 recomputation
     bool c15tc;        // C1/C5 on the tensor cores (staging buffer per chunk)
     bool cfree;        // C-free variant: C1 alone, drift and Laplacian from v = D^-1 A^T
+    bool vd64;         // FP64 path: C1 alone, drift and Laplacian from v = D^-1 A^T in FP64
     bool f64tc;        // FP64 path with the tensor-core a4 (QMC_PREC_F64_TCA4)
     double kappa_max;  // FP64 recomputation threshold of the float-pair a4
     bool dinv;
@@ -725,7 +726,8 @@ struct Plan {
 
 size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 
-// c15_override >= 0 replaces the system's c15_mode (qmc_slater_matrices needs all five matrices)
+// c15_override >= 0 replaces the system's c15_mode: qmc_slater_matrices needs all five matrices (in the
+// FP64 path too)
 Plan make_plan(const qmc_system *sys, int precision, bool need_dinv, int c15_override = -1)
 {
     Plan p;
@@ -743,6 +745,7 @@ Plan make_plan(const qmc_system *sys, int precision, bool need_dinv, int c15_ove
     p.kappa_max = p.f64tc ? sys->tiles.f64_kappa_max : sys->tiles.a4_kappa_max;
     p.redo_bytes = p.ffgj ? redo_scratch_bytes(std::max(sys->d.n_up, sys->d.n_dn)) : 0;
     p.c15tc = p.mixed && (c15 == QMC_C15_TENSOR || c15 == QMC_C15_CFREE);
+    p.vd64 = !p.mixed && c15_override < 0 && cfree_f64_fits(sys->d);
     p.sd = &sys->d;
     p.per_walker = p.msz * 8 + p.cd_bytes + (need_dinv ? p.msz * 8 : 0) + 36 + p.mask_bytes +
                    (p.ffgj ? p.msz * 8 + 2 : 0);
@@ -780,6 +783,7 @@ bool carve(const Plan &p, int nw, void *ws, size_t ws_bytes, Carve &c)
     } else {
         c.Cd = take(p.msz * 4 * 8 * nw);
         c.L5 = nullptr;
+        if (p.vd64) c.vd = static_cast<double *>(c.Cd);   // [nw][N][4] in the place of C2..C5 (N <= n_up^2 + n_dn^2)
     }
     c.D = p.dinv ? reinterpret_cast<double *>(take(p.msz * 8 * nw)) : nullptr;
     c.la = reinterpret_cast<double *>(take(16 * (size_t)nw));
@@ -880,6 +884,7 @@ cudaError_t run_products(const qmc_system *sys, int precision, int nw, const dou
                          cudaStream_t st, Mark mark, const WaitCfg &wc, const Plan &p)
 {
     const SysDev &s = sys->d;
+    if (p.vd64) return launch_c1_f64(s, nw, Rc, c.X, st);
     if (!p.mixed) return launch_contract_f64(s, nw, Rc, c.X, static_cast<double *>(c.Cd), st);
     const MixedTables &mt = sys->mixed;
     cudaError_t e = launch_shell_mask(s, mt, nw, Rc, mt.mask_words, c.masks, st);
@@ -1036,6 +1041,10 @@ int eval_impl(const qmc_system *sys, int n_walk, const double *R, int precision,
             e = launch_vdrift(s, sys->mixed.ffb, sys->mixed, nw, Rc, c.masks, sys->mixed.mask_words, Dinv, c.vd, c.st,
                               c.stage, c.stage_bytes, st, wc);
             if (e != cudaSuccess) return cuda_fail(e, "qmc_walkers_eval: C-free drift launch");
+        }
+        if (p.vd64) {
+            e = launch_vdrift_f64(s, nw, Rc, Dinv, c.vd, st);
+            if (e != cudaSuccess) return cuda_fail(e, "qmc_walkers_eval: FP64 drift launch");
         }
         e = launch_drift_energy(s, nw, Rc, Dinv, cview(p, c), c.la, c.sg, c.st, *out, w0, st, sys->mixed.ffb.Q);
         if (e != cudaSuccess) return cuda_fail(e, "qmc_walkers_eval: energy launch");

@@ -6,7 +6,7 @@
 
 namespace qmc {
 
-__device__ __forceinline__ int ncart(int L) { return (L + 1) * (L + 2) / 2; }
+__host__ __device__ __forceinline__ int ncart(int L) { return (L + 1) * (L + 2) / 2; }
 
 // Squared distance rounded exactly as ((dx*dx) + (dy*dy)) + (dz*dz), each
 // operation correctly rounded and never fused: the screening decision

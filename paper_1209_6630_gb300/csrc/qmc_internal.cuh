@@ -127,6 +127,11 @@ int cuda_fail(cudaError_t e, const char *where);
 // kernels (launchers); all return a cudaError_t from the launch
 cudaError_t launch_contract_f64(const SysDev &s, int nw, const double *R, double *X, double *Cd,
                                 cudaStream_t st);
+// FP64 path without C2..C5 (k_cfree_f64.cu)
+bool cfree_f64_fits(const SysDev &s);
+cudaError_t launch_c1_f64(const SysDev &s, int nw, const double *R, double *X, cudaStream_t st);
+cudaError_t launch_vdrift_f64(const SysDev &s, int nw, const double *R, const double *Dinv, double *vd,
+                              cudaStream_t st);
 cudaError_t launch_screen_ao(const SysDev &s, int nw, const double *R, int cap, int32_t *cnt,
                              int32_t *idx, double *B, cudaStream_t st);
 cudaError_t launch_gj(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb);
