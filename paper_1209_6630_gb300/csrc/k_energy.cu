@@ -1,8 +1,8 @@
 // Steps a5-a6: drift, kinetic energy and local energy per walker, FP64.
 // With a Jastrow factor (Psi = e^J Det_up Det_dn, Sec. II.C) the drift gains
 // grad_e J and the kinetic term lap_e J + |grad_e J|^2 + 2 grad_e J . b_e (b_e
-// the determinants' drift), J is added to log|Psi| (FP64 pair sums, one warp
-// per electron).
+// the determinants' drift), J is added to log|Psi| (FP64 pair sums, each pair
+// evaluated once for both of its electrons).
 //
 //   drift_{e,l} = sum_k (D^-1)_{ek} d_l phi_k(r_e)     (Eq. 2 with the
 //   lap_e       = sum_k (D^-1)_{ek} lap phi_k(r_e)      Sec. II.C vector products;
@@ -10,8 +10,11 @@
 //   V_en = -sum_{e,a} Z_a / |r_e - Q_a|,  V_ee = sum_{i<j} 1 / |r_i - r_j|,
 //   V_nn = sum_{a<b} Z_a Z_b / |Q_a - Q_b| (load time),  E_L = T + V (Eq. 4)
 //
-// One CTA per walker; one warp per electron row for the dot products (rows
-// of D^-1 and of C2..C5 are contiguous); warp-shuffle reductions.
+// A cluster of 1, 2, 4 or 8 CTAs per walker (one where the walkers fill the card); one warp per
+// electron row for the dot products (rows of D^-1 and of C2..C5 are contiguous);
+// warp-shuffle reductions, the CTAs' sums added in rank order through distributed shared memory.
+// Measured: 1056 electrons x 37 walkers 854 -> 272 us (37 CTAs before), 158 electrons x 1 walker
+// 52 -> 17 us; with the Jastrow factor, 434 electrons x 601 walkers 13.6 -> 7.5 ms.
 //
 // FP64 path: everything in FP64.  Mixed path (C2..C4 in FP32): the drift
 // dots in FP32 (D^-1 truncated to float by integer operations), the
@@ -19,6 +22,7 @@
 // pipes: differences of float-pair positions, r^2 as a float pair, 1/r from
 // the FP32 reciprocal square root refined by one Newton step (relative error
 // ~2^-43), sums kept as float pairs.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <type_traits>
@@ -27,6 +31,8 @@
 #include "qmc_internal.cuh"
 
 namespace qmc {
+
+namespace cg = cooperative_groups;
 
 constexpr int kEnThreads = 256;
 constexpr int kEnWarps = kEnThreads / 32;
@@ -61,15 +67,29 @@ __device__ __forceinline__ float2 ff_inv_r(float2 dx, float2 dy, float2 dz)
     return ff::renorm(y0, 0.5f * y0 * e.x);                      // Newton step y0 (1 + e/2)
 }
 
+// 1/sqrt(x) in FP64 from the FP32 reciprocal square root y (relative error 2^-22): with
+// e = 1 - x y^2, 1/sqrt(x) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + O(e^3)), O(e^3) < 2^-64
+// (Halley's third-order iteration): 5 FP64 operations, where the pipe is what the sums wait for.
+__device__ __forceinline__ bool in_fast_range(double x) { return x > 1e-30 && x < 1e30; }
+
+__device__ __forceinline__ double rsqrt_f64(double x)
+{
+    if (!in_fast_range(x)) return rsqrt(x);
+    const double y = (double)rsqrtf((float)x);
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(e * y, fma(0.375, e, 0.5), y);
+}
+
 // Coulomb sums of one walker in float-float (mixed path); rs: 3N positions,
 // qs: 3 n_atom nuclear positions, zs: charges, all staged in shared memory.
+// Warp `wid` of `nwarps` (over the walker's CTAs).
 __device__ __forceinline__ void coulomb_ff(const SysDev &s, const float2 *rs, const float2 *qs, const float *zs,
-                                           double &ven, double &vee)
+                                           int wid, int nwarps, double &ven, double &vee)
 {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const int N = s.n_elec;
     float2 en = make_float2(0.f, 0.f), ee = make_float2(0.f, 0.f);
-    for (int e = wid; e < N; e += kEnWarps) {
+    for (int e = wid; e < N; e += nwarps) {
         const float2 rx = rs[3 * e], ry = rs[3 * e + 1], rz = rs[3 * e + 2];
         for (int a = lane; a < s.n_atom; a += 32) {
             const float2 y = ff_inv_r(ff::sub(rx, qs[3 * a]), ff::sub(ry, qs[3 * a + 1]), ff::sub(rz, qs[3 * a + 2]));
@@ -130,36 +150,88 @@ __device__ __forceinline__ void dets_drift_lap(const SysDev &s, const double *__
     b3 = warp_sum(b3);
 }
 
-// The Jastrow factor's part for electron e (one warp, FP64; results on every
-// lane): g = grad_e J, L = lap_e J, and Je = the terms of J that e owns (its
-// pairs with j > e and its e-n terms), so that sum_e Je = J.  Pade form
-// U = a r / (1 + b r): U' = a / (1 + b r)^2, U'' = -2 a b / (1 + b r)^3,
-// lap U(|r_e - x|) = U'' + 2 U' / r, grad U = U' (r_e - x) / r.
-__device__ __forceinline__ void jastrow_e(const SysDev &s, const double *__restrict__ Rw, int e, int lane,
-                                          double &g0, double &g1, double &g2, double &L, double &Je)
+// One Jastrow term, Pade form U = a r / (1 + b r): U' = a / (1 + b r)^2, U'' = -2 a b / (1 + b r)^3,
+// lap U(|r_e - x|) = U'' + 2 U' / r, grad U = U' (r_e - x) / r.  f = U' / r.
+__device__ __forceinline__ void jastrow_term(double r2, double a, double b, double &f, double &lap, double &u)
 {
-    const double rx = Rw[3 * e], ry = Rw[3 * e + 1], rz = Rw[3 * e + 2];
-    const bool up = e < s.n_up;
-    g0 = g1 = g2 = L = Je = 0.0;
-    auto term = [&](double dx, double dy, double dz, double a, double b, bool own) {
-        const double r = sqrt(dx * dx + dy * dy + dz * dz);
-        const double q = 1.0 + b * r, iq = 1.0 / q;
-        const double u1 = a * iq * iq, u2 = -2.0 * a * b * iq * iq * iq;
-        const double f = u1 / r;
-        g0 += f * dx; g1 += f * dy; g2 += f * dz;
-        L += u2 + 2.0 * f;
-        if (own) Je += a * r * iq;
-    };
-    for (int j = lane; j < s.n_elec; j += 32) {
-        if (j == e) continue;
-        const double a = ((j < s.n_up) == up) ? s.ja_par : s.ja_anti;
-        term(rx - Rw[3 * j], ry - Rw[3 * j + 1], rz - Rw[3 * j + 2], a, s.jb_ee, j > e);
+    double iq, ir, r, q;
+    bool fast = in_fast_range(r2);
+    if (fast) {
+        ir = rsqrt_f64(r2);
+        r = r2 * ir;
+        q = 1.0 + b * r;
+        fast = q < 1e30;
     }
-    for (int at = lane; at < s.n_atom; at += 32)
-        term(rx - s.Q[3 * at], ry - s.Q[3 * at + 1], rz - s.Q[3 * at + 2], -s.ja_en[at], s.jb_en[at], true);
-    g0 = warp_sum(g0); g1 = warp_sum(g1); g2 = warp_sum(g2);
-    L = warp_sum(L);
-    Je = warp_sum(Je);
+    if (fast) {
+        // 1 / q from the FP32 reciprocal y: with e = 1 - q y, 1 / q = y (1 + e + e^2 + O(e^3))
+        const double y = (double)__frcp_rn((float)q);
+        const double e = fma(-q, y, 1.0);
+        iq = fma(y, fma(e, e, e), y);
+        const double t = a * iq;
+        u = t * r;
+        const double u1 = t * iq;
+        f = u1 * ir;
+        lap = fma(2.0, f, -2.0 * b * (u1 * iq));
+    } else {
+        r = sqrt(r2);
+        q = 1.0 + b * r;
+        iq = 1.0 / q;
+        const double u1 = a * iq * iq;
+        f = u1 / r;
+        lap = -2.0 * a * b * iq * iq * iq + 2.0 * f;
+        u = a * r * iq;
+    }
+}
+
+// The Jastrow factor of one walker over the CTAs of its cluster: grad_e J (acc[0..2][e]) and
+// lap_e J (acc[3][e]) are the sums of the ranks' arrays, J itself the sum of the returned values
+// over all threads.  Each pair is evaluated once: in step d electron e meets e + d (mod N);
+// within a step the partners are distinct, so their sums need only a barrier between steps, and
+// every sum has a fixed order.  rank takes the steps and the atoms congruent to it.
+// rj: 3N positions; acc: [4][N] in shared memory.
+__device__ double jastrow_all(const SysDev &s, const double *rj, double *acc, int rank, int nrank)
+{
+    const int t = threadIdx.x, N = s.n_elec;
+    double Jt = 0.0;
+    for (int q = t; q < 4 * N; q += kEnThreads) acc[q] = 0.0;
+    __syncthreads();
+    for (int e0 = 0; e0 < N; e0 += kEnThreads) {
+        const int e = e0 + t;
+        const bool ok = e < N;
+        const double rx = ok ? rj[3 * e] : 0.0, ry = ok ? rj[3 * e + 1] : 0.0, rz = ok ? rj[3 * e + 2] : 0.0;
+        double g0 = 0.0, g1 = 0.0, g2 = 0.0, L = 0.0;
+        for (int d = 1 + rank; d <= N / 2; d += nrank) {
+            // (an even N meets its opposite electron from both sides at d = N / 2: the lower one counts)
+            if (ok && !(2 * d == N && e >= d)) {
+                const int j = e + d < N ? e + d : e + d - N;
+                const double dx = rx - rj[3 * j], dy = ry - rj[3 * j + 1], dz = rz - rj[3 * j + 2];
+                const double a = ((e < s.n_up) == (j < s.n_up)) ? s.ja_par : s.ja_anti;
+                double f, lp, u;
+                jastrow_term(dx * dx + dy * dy + dz * dz, a, s.jb_ee, f, lp, u);
+                g0 = fma(f, dx, g0); g1 = fma(f, dy, g1); g2 = fma(f, dz, g2);
+                L += lp;
+                Jt += u;
+                acc[j] = fma(-f, dx, acc[j]);
+                acc[N + j] = fma(-f, dy, acc[N + j]);
+                acc[2 * N + j] = fma(-f, dz, acc[2 * N + j]);
+                acc[3 * N + j] += lp;
+            }
+            __syncthreads();
+        }
+        if (ok) {
+            for (int at = rank; at < s.n_atom; at += nrank) {
+                const double dx = rx - s.Q[3 * at], dy = ry - s.Q[3 * at + 1], dz = rz - s.Q[3 * at + 2];
+                double f, lp, u;
+                jastrow_term(dx * dx + dy * dy + dz * dz, -s.ja_en[at], s.jb_en[at], f, lp, u);
+                g0 = fma(f, dx, g0); g1 = fma(f, dy, g1); g2 = fma(f, dz, g2);
+                L += lp;
+                Jt += u;
+            }
+            acc[e] += g0; acc[N + e] += g1; acc[2 * N + e] += g2; acc[3 * N + e] += L;
+        }
+        __syncthreads();                                       // before the next block's partners
+    }
+    return Jt;
 }
 
 template <typename TG>
@@ -169,21 +241,54 @@ __global__ void __launch_bounds__(kEnThreads) k_drift_energy(SysDev s, const dou
                                                              const double *__restrict__ logabs2,
                                                              const double *__restrict__ sign2,
                                                              const uint32_t *__restrict__ sing,
-                                                             qmc_eval_out o, int w_off, const float2 *__restrict__ Q2)
+                                                             qmc_eval_out o, int w_off, const float2 *__restrict__ Q2,
+                                                             int stage)
 {
     constexpr bool kMixed = std::is_same<TG, float>::value;
-    extern __shared__ __align__(16) unsigned char en_smem[];   // mixed: positions, nuclei, charges
+    // mixed: positions, nuclei, charges as floats; with a Jastrow factor (before them) positions
+    // and the pair sums in FP64
+    extern __shared__ __align__(16) unsigned char en_smem[];
     __shared__ double red[4][kEnWarps];
+    __shared__ double total[4];
     __shared__ int s_nonfinite;
-    const int w = blockIdx.x;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int nrank = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int w = blockIdx.x / nrank;
     const int wg = w + w_off;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int gw = rank * kEnWarps + wid, ngw = nrank * kEnWarps;   // warps of the walker
     const int N = s.n_elec;
     const size_t msz = (size_t)s.n_up * s.n_up + (size_t)s.n_dn * s.n_dn;
     const double *Rw = R + (size_t)w * N * 3;
 
+    if (t == 0) s_nonfinite = 0;
+    __syncthreads();
+    double *acc = reinterpret_cast<double *>(en_smem);         // [4][N] (Jastrow only)
+    float2 *rs = reinterpret_cast<float2 *>(acc + (s.jas ? 4 * N : 0));
+    float *zs = reinterpret_cast<float *>(rs + 3 * N);         // (padded to an even count)
+    float2 *qs = reinterpret_cast<float2 *>(zs + ((s.n_atom + 1) & ~1));
+    double *rj = kMixed ? reinterpret_cast<double *>(qs + ((stage & 1) ? 3 * s.n_atom : 0)) : acc + 4 * N;   // [3 N]
+    int bad = 0;
+    for (int q = t; q < 3 * N; q += kEnThreads) {
+        const double x = Rw[q];
+        bad |= !isfinite(x);
+        if (stage & 2) rj[q] = x;
+        if constexpr (kMixed) rs[q] = ff::from_double(x);
+    }
+    if constexpr (kMixed) {
+        if (stage & 1)
+            for (int q = t; q < 3 * s.n_atom; q += kEnThreads) qs[q] = Q2[q];
+        for (int a = t; a < s.n_atom; a += kEnThreads) zs[a] = (float)s.Z[a];
+    }
+    if (bad) s_nonfinite = 1;
+    __syncthreads();
+
     double lap_acc = 0.0, jas_acc = 0.0;
-    for (int e = wid; e < N; e += kEnWarps) {
+    if (s.jas) {
+        jas_acc = jastrow_all(s, (stage & 2) ? rj : Rw, acc, rank, nrank);
+        cluster.sync();                                        // every rank's sums are complete
+    }
+    for (int e = gw; e < N; e += ngw) {
         double b0 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0;
         if (cv.vd) {             // C-free variant: drift and Laplacian of the determinants already formed
             const double *v = cv.vd + ((size_t)w * N + e) * 4;
@@ -191,54 +296,53 @@ __global__ void __launch_bounds__(kEnThreads) k_drift_energy(SysDev s, const dou
         } else {
             dets_drift_lap<kMixed>(s, Dinv, Cg, cv, w, e, lane, msz, b0, b1, b2, b3);
         }
-        double g0 = 0.0, g1 = 0.0, g2 = 0.0, L = 0.0, Je = 0.0;
-        if (s.jas) jastrow_e(s, Rw, e, lane, g0, g1, g2, L, Je);
         if (lane == 0) {
+            double g0 = 0.0, g1 = 0.0, g2 = 0.0, L = 0.0;
+            if (s.jas)
+                for (int r = 0; r < nrank; ++r) {
+                    const double *x = cluster.map_shared_rank(acc, r);
+                    g0 += x[e]; g1 += x[N + e]; g2 += x[2 * N + e]; L += x[3 * N + e];
+                }
             double *dr = o.drift + ((size_t)wg * N + e) * 3;
             dr[0] = b0 + g0; dr[1] = b1 + g1; dr[2] = b2 + g2;
             // lap_e Psi / Psi with Psi = e^J Det: lap J + |grad J|^2 + 2 grad J . grad Det / Det + lap Det / Det
             lap_acc += b3 + L + (g0 * g0 + g1 * g1 + g2 * g2) + 2.0 * (g0 * b0 + g1 * b1 + g2 * b2);
-            jas_acc += Je;
         }
     }
     double ven = 0.0, vee = 0.0;
     if constexpr (kMixed) {
-        float2 *rs = reinterpret_cast<float2 *>(en_smem);
-        float2 *qs = rs + 3 * N;
-        float *zs = reinterpret_cast<float *>(qs + 3 * s.n_atom);
-        if (t == 0) s_nonfinite = 0;
-        __syncthreads();
-        int bad = 0;
-        for (int q = t; q < 3 * N; q += kEnThreads) {
-            const double x = Rw[q];
-            bad |= !isfinite(x);
-            rs[q] = ff::from_double(x);
-        }
-        for (int q = t; q < 3 * s.n_atom; q += kEnThreads) qs[q] = Q2[q];
-        for (int a = t; a < s.n_atom; a += kEnThreads) zs[a] = (float)s.Z[a];
-        if (bad) s_nonfinite = 1;
-        __syncthreads();
-        coulomb_ff(s, rs, qs, zs, ven, vee);
+        coulomb_ff(s, rs, (stage & 1) ? qs : Q2, zs, gw, ngw, ven, vee);
     } else {
-        for (int e = wid; e < N; e += kEnWarps) {
+        for (int e = gw; e < N; e += ngw) {
             const double rx = Rw[3 * e], ry = Rw[3 * e + 1], rz = Rw[3 * e + 2];
             for (int a = lane; a < s.n_atom; a += 32) {
                 const double dx = rx - s.Q[3 * a], dy = ry - s.Q[3 * a + 1], dz = rz - s.Q[3 * a + 2];
-                ven -= s.Z[a] * rsqrt(dx * dx + dy * dy + dz * dz);
+                ven -= s.Z[a] * rsqrt_f64(dx * dx + dy * dy + dz * dz);
             }
             for (int j = e + 1 + lane; j < N; j += 32) {
                 const double dx = rx - Rw[3 * j], dy = ry - Rw[3 * j + 1], dz = rz - Rw[3 * j + 2];
-                vee += rsqrt(dx * dx + dy * dy + dz * dz);
+                vee += rsqrt_f64(dx * dx + dy * dy + dz * dz);
             }
         }
     }
+    if (s.jas) jas_acc = warp_sum(jas_acc);
     ven = warp_sum(ven);
     vee = warp_sum(vee);
     if (lane == 0) { red[0][wid] = lap_acc; red[1][wid] = ven; red[2][wid] = vee; red[3][wid] = jas_acc; }
     __syncthreads();
-    if (t == 0) {
+    if (t < 4) {
+        double x = 0.0;
+        for (int q = 0; q < kEnWarps; ++q) x += red[t][q];
+        total[t] = x;
+    }
+    if (nrank > 1 || s.jas) cluster.sync();                    // totals, and no CTA leaves while its sums are read
+    else __syncthreads();
+    if (t == 0 && rank == 0) {
         double lap = 0.0, Ven = 0.0, Vee = 0.0, Jt = 0.0;
-        for (int q = 0; q < kEnWarps; ++q) { lap += red[0][q]; Ven += red[1][q]; Vee += red[2][q]; Jt += red[3][q]; }
+        for (int r = 0; r < nrank; ++r) {
+            const double *x = cluster.map_shared_rank(total, r);
+            lap += x[0]; Ven += x[1]; Vee += x[2]; Jt += x[3];
+        }
         const double T = -0.5 * lap;
         const double el = T + Ven + Vee + s.vnn;
         // a spin with no electrons contributes det = 1
@@ -246,10 +350,7 @@ __global__ void __launch_bounds__(kEnThreads) k_drift_energy(SysDev s, const dou
         const double sg0 = s.n_up ? sign2[2 * w] : 1.0, sg1 = s.n_dn ? sign2[2 * w + 1] : 1.0;
         uint32_t st = sing[w];
         const bool singular = (st & (QMC_STATUS_SINGULAR_UP | QMC_STATUS_SINGULAR_DN)) != 0;
-        bool finite_in = true;
-        if constexpr (kMixed) finite_in = !s_nonfinite;
-        else
-            for (int q = 0; q < 3 * N; ++q) finite_in = finite_in && isfinite(Rw[q]);
+        const bool finite_in = !s_nonfinite;
         if (!finite_in) st |= QMC_STATUS_NONFINITE;
         if (!singular && !(isfinite(el) && isfinite(la0) && isfinite(la1) && isfinite(Jt))) st |= QMC_STATUS_NONFINITE;
         o.logpsi[wg] = singular ? -INFINITY : la0 + la1 + Jt;     // log|Psi| = log|Det_up| + log|Det_dn| + J
@@ -262,6 +363,44 @@ __global__ void __launch_bounds__(kEnThreads) k_drift_energy(SysDev s, const dou
         }
         o.status[wg] = st;
     }
+    if (nrank > 1) cluster.sync();                             // rank 0 has read the totals
+}
+
+template <typename TG>
+static cudaError_t launch_en(const SysDev &s, int nw, const double *R, const double *Dinv, const CView &cv,
+                             const double *logabs2, const double *sign2, const uint32_t *sing,
+                             const qmc_eval_out &o, int w_off, cudaStream_t st, const float2 *Q2)
+{
+    constexpr bool kMixed = std::is_same<TG, float>::value;
+    const size_t N = s.n_elec, na = s.n_atom;
+    // stage bit 0: the nuclei's float pairs in shared memory, bit 1: the positions in FP64 (for the
+    // Jastrow pairs); without the room they are read from global memory
+    int stage = 0;
+    size_t sm = (s.jas ? 8 * 4 * N : 0) + (kMixed ? sizeof(float2) * 3 * N + sizeof(float) * ((na + 1) & ~size_t(1)) : 0);
+    const size_t most = 200 * 1024;
+    if (kMixed && sm + sizeof(float2) * 3 * na <= most) { stage |= 1; sm += sizeof(float2) * 3 * na; }
+    if (s.jas && sm + 8 * 3 * N <= most) { stage |= 2; sm += 8 * 3 * N; }
+    // CTAs per walker: up to 8 (the portable cluster size) while the walkers give fewer than four
+    // CTAs to each of 152 SMs and each warp keeps an electron
+    unsigned c = 1;
+    while (c < 8 && (size_t)nw * c < 152 * 4 && N >= (size_t)2 * kEnWarps * c) c *= 2;
+    cudaError_t e = cudaFuncSetAttribute(k_drift_energy<TG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = c;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nw * c);
+    cfg.blockDim = dim3(kEnThreads);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, k_drift_energy<TG>, s, R, Dinv, static_cast<const TG *>(cv.g), cv, logabs2, sign2,
+                           sing, o, w_off, Q2, stage);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_drift_energy(const SysDev &s, int nw, const double *R, const double *Dinv, const CView &cv,
@@ -269,18 +408,8 @@ cudaError_t launch_drift_energy(const SysDev &s, int nw, const double *R, const 
                                 const qmc_eval_out &o, int w_off, cudaStream_t st, const float2 *Q2)
 {
     if (nw == 0) return cudaSuccess;
-    if (cv.g_f32) {
-        const size_t sm = sizeof(float2) * 3 * ((size_t)s.n_elec + s.n_atom) + sizeof(float) * (size_t)s.n_atom;
-        cudaError_t e = cudaFuncSetAttribute(k_drift_energy<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sm);
-        if (e != cudaSuccess) return e;
-        k_drift_energy<float><<<nw, kEnThreads, sm, st>>>(s, R, Dinv, static_cast<const float *>(cv.g), cv,
-                                                          logabs2, sign2, sing, o, w_off, Q2);
-    } else {
-        k_drift_energy<double><<<nw, kEnThreads, 0, st>>>(s, R, Dinv, static_cast<const double *>(cv.g), cv,
-                                                           logabs2, sign2, sing, o, w_off, nullptr);
-    }
-    return cudaGetLastError();
+    return cv.g_f32 ? launch_en<float>(s, nw, R, Dinv, cv, logabs2, sign2, sing, o, w_off, st, Q2)
+                    : launch_en<double>(s, nw, R, Dinv, cv, logabs2, sign2, sing, o, w_off, st, nullptr);
 }
 
 }  // namespace qmc
