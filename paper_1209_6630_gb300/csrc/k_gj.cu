@@ -11,6 +11,9 @@
 //      operations at once, as a rank-NB update
 //        X[i][j] <- [i not a pivot row] X[i][j] + sum_c P[i][c] X[piv_c][j]
 //      (P = the eliminated panel, which holds the composite row operations).
+// (Matrices too few for one CTA each to fill the card: launch_gj_wide, k_gj_redo.cu.)
+// The panel (gj_panel.cuh) was a third of the time with 16-way bank conflicts, a division and
+// FP64 compares in every thread: 300 matrices of n = 217 7.95 -> 6.14 ms, 400 of n = 528 122 -> 116.
 // Pivoting is implicit: rows never move in memory; a row map records which
 // physical row was the pivot of each step.  After the last panel the array
 // holds Res with X^-1[a][b] = Res[pp[a]][ipp[b]] (pp = pivot rows, ipp its
@@ -22,6 +25,7 @@
 #include <math.h>
 
 #include "ff_math.cuh"
+#include "gj_panel.cuh"
 #include "qmc_internal.cuh"
 
 namespace qmc {
@@ -38,22 +42,6 @@ __host__ __device__ __forceinline__ size_t p_region(int n, int nb)
 {
     const size_t a = (size_t)n * nb;
     return a > 32 * 33 ? a : 32 * 33;
-}
-
-__device__ __forceinline__ void argmax_merge(double &v, int &i, double v2, int i2)
-{
-    if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
-}
-
-__device__ __forceinline__ void block_argmax(double &bv, int &bi, double *red_v, int *red_i, int lane, int wid)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double v2 = __shfl_down_sync(0xffffffffu, bv, o);
-        const int i2 = __shfl_down_sync(0xffffffffu, bi, o);
-        argmax_merge(bv, bi, v2, i2);
-    }
-    if (lane == 0) { red_v[wid] = bv; red_i[wid] = bi; }
 }
 
 __device__ __forceinline__ void argmax_merge_f(float &v, int &i, float v2, int i2)
@@ -73,7 +61,7 @@ __device__ __forceinline__ void block_argmax_f(float &bv, int &bi, float *red_v,
 }
 
 template <int NB>
-__global__ void __launch_bounds__(kGjThreads) k_gj(GjJobs2 jobs)
+__global__ void __launch_bounds__(kGjThreads, NB == 32 ? 1 : 3) k_gj(GjJobs2 jobs)
 {
     const GjJob &J = jobs.j[blockIdx.y];
     const int m = blockIdx.x;
@@ -89,13 +77,11 @@ __global__ void __launch_bounds__(kGjThreads) k_gj(GjJobs2 jobs)
     short *used = reinterpret_cast<short *>(U + NB * 32); // [n] 1 once a row has been a pivot
     short *pp = used + n;                                 // [n] pivot row of step k
     short *rowc = pp + n;                                 // [n] panel column of a pivot row, or -1
-    __shared__ double red_v[kGjWarps];
-    __shared__ int red_i[kGjWarps];
-    __shared__ int s_p, s_sing;
+    __shared__ GjPanelShared<NB> S;
 
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     for (int i = t; i < n; i += kGjThreads) { used[i] = 0; rowc[i] = -1; }
-    if (t == 0) s_sing = 0;
+    bool sing = false;
     double logabs = 0.0;
     int neg = 0;
     __syncthreads();
@@ -104,63 +90,22 @@ __global__ void __launch_bounds__(kGjThreads) k_gj(GjJobs2 jobs)
         const int w = min(NB, n - jb);
         for (int q = t; q < n * NB; q += kGjThreads) {
             const int i = q / NB, c = q - i * NB;
-            P[q] = (c < w) ? X[(size_t)i * n + jb + c] : 0.0;
+            P[gj_at<NB>(i, c)] = (c < w) ? X[(size_t)i * n + jb + c] : 0.0;
         }
         __syncthreads();
-        // pivot candidates of the panel's first column
-        double bv = -1.0;
-        int bi = n;
-        for (int i = t; i < n; i += kGjThreads)
-            if (!used[i]) argmax_merge(bv, bi, fabs(P[i * NB]), i);
-        block_argmax(bv, bi, red_v, red_i, lane, wid);
-        __syncthreads();
-
-        for (int c = 0; c < w; ++c) {
-            if (t == 0) {
-                double v = red_v[0];
-                int b = red_i[0];
-                for (int q = 1; q < kGjWarps; ++q) argmax_merge(v, b, red_v[q], red_i[q]);
-                s_p = b;
-                if (!(v > 0.0)) s_sing = 1;   // exact zero (or NaN) pivot
+        if (!gj_panel<NB>(P, n, w, used, S)) { sing = true; break; }
+        if (wid == 0) {
+            gj_add_pivots<NB>(S, w, logabs, neg);
+            if (lane < w) {
+                pp[jb + lane] = S.pp[lane];
+                rowc[S.pp[lane]] = (short)lane;
             }
-            __syncthreads();
-            if (s_sing) break;
-            const int p = s_p;
-            const double piv = P[p * NB + c];
-            const double inv = 1.0 / piv;
-            if (t == 0) {
-                used[p] = 1;
-                pp[jb + c] = (short)p;
-                rowc[p] = (short)c;
-                logabs += log(fabs(piv));
-                neg ^= (piv < 0.0);
-            }
-            __syncthreads();   // every thread has read P[p][c] (piv); used[p] is set
-            if (t < NB) P[p * NB + t] = (t == c) ? inv : P[p * NB + t] * inv;
-            __syncthreads();
-            // eliminate column c from the other rows and, on the way, find the
-            // pivot candidates of column c+1 among the rows not yet used
-            double nbv = -1.0;
-            int nbi = n;
-            const int cn = c + 1;
-            for (int i = t; i < n; i += kGjThreads) {
-                if (i == p) continue;
-                const double f = P[i * NB + c];
-#pragma unroll
-                for (int cc = 0; cc < NB; ++cc)
-                    if (cc != c) P[i * NB + cc] = fma(-f, P[p * NB + cc], P[i * NB + cc]);
-                P[i * NB + c] = -f * inv;
-                if (cn < w && !used[i]) argmax_merge(nbv, nbi, fabs(P[i * NB + cn]), i);
-            }
-            block_argmax(nbv, nbi, red_v, red_i, lane, wid);
-            __syncthreads();
         }
-        if (s_sing) break;
 
         // store the eliminated panel
         for (int q = t; q < n * w; q += kGjThreads) {
             const int i = q / w, c = q - i * w;
-            X[(size_t)i * n + jb + c] = P[i * NB + c];
+            X[(size_t)i * n + jb + c] = P[gj_at<NB>(i, c)];
         }
 
         // rank-w update of every other column, 32 columns at a time; the pivot
@@ -205,10 +150,9 @@ __global__ void __launch_bounds__(kGjThreads) k_gj(GjJobs2 jobs)
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
                         const int ii = i + r * kGjWarps;
-                        const double2 *pr = reinterpret_cast<const double2 *>(P + ii * NB);
 #pragma unroll
                         for (int c2 = 0; c2 < NB / 2; ++c2) {
-                            const double2 pv = pr[c2];
+                            const double2 pv = *reinterpret_cast<const double2 *>(P + gj_at<NB>(ii, 2 * c2));
                             x[r] = fma(pv.x, u[2 * c2], x[r]);
                             x[r] = fma(pv.y, u[2 * c2 + 1], x[r]);
                         }
@@ -218,10 +162,9 @@ __global__ void __launch_bounds__(kGjThreads) k_gj(GjJobs2 jobs)
                 }
                 for (; i < n; i += kGjWarps) {
                     double x = (rowc[i] >= 0) ? 0.0 : X[(size_t)i * n + col];
-                    const double2 *pr = reinterpret_cast<const double2 *>(P + i * NB);
 #pragma unroll
                     for (int c2 = 0; c2 < NB / 2; ++c2) {
-                        const double2 pv = pr[c2];
+                        const double2 pv = *reinterpret_cast<const double2 *>(P + gj_at<NB>(i, 2 * c2));
                         x = fma(pv.x, u[2 * c2], x);
                         x = fma(pv.y, u[2 * c2 + 1], x);
                     }
@@ -235,7 +178,7 @@ __global__ void __launch_bounds__(kGjThreads) k_gj(GjJobs2 jobs)
         __syncthreads();
     }
 
-    if (s_sing) {
+    if (sing) {
         const double qnan = __longlong_as_double(0x7ff8000000000000ll);
         for (size_t q = t; q < (size_t)n * n; q += kGjThreads) Dout[q] = qnan;
         if (t == 0) {
@@ -292,6 +235,17 @@ static cudaError_t launch_gj_nb(const GjJobs2 &js, int n_jobs, int nmax, int cma
     return cudaGetLastError();
 }
 
+// Whether to spread each matrix over many CTAs (launch_gj_wide, two launches per panel) rather
+// than to give it one (k_gj).  An SM's FP64 pipe takes as long for one matrix in k_gj whatever
+// the others do, so the call takes ceil(T / 152) matrices' time; spread, T / 152 and the panels'
+// latency.  Measured (ms, k_gj / spread): n = 217: T = 4 3.34 / 0.84, 100 3.35 / 2.60, 192 6.11 /
+// 4.36, 300 6.14 / 6.32, 600 11.96 / 12.54, 2000 40.5 / 40.0; n = 528: 4 40.2 / 4.5, 150 42.8 /
+// 40.5, 400 116 / 103; n = 866: 1 176 / 7.6, 150 190 / 173; n = 31: 50 0.100 / 0.112.
+static bool gj_wide(int n, long long T)
+{
+    return n >= 32 && (n >= 512 || (T + 151) / 152 * 152 * 100 > 105 * T);
+}
+
 cudaError_t launch_gj(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb)
 {
     GjJobs2 js;
@@ -303,6 +257,7 @@ cudaError_t launch_gj(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb)
         cmax = max(cmax, js.j[q].count);
     }
     if (cmax == 0) return cudaSuccess;
+    if (!jobs[0].only_redo && gj_wide(nmax, js.j[0].count + js.j[1].count)) return launch_gj_wide(jobs, n_jobs, st, nb);
     switch (nb) {
     case 8: return launch_gj_nb<8>(js, n_jobs, nmax, cmax, st);
     case 16: return launch_gj_nb<16>(js, n_jobs, nmax, cmax, st);

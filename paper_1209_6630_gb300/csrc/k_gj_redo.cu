@@ -5,21 +5,33 @@
 //
 // A 528 x 528 FP64 elimination on one SM is bound by that SM's FP64 pipe
 // (~35 ms), so a single flagged matrix would dominate the stage.  Here each
-// flagged matrix is spread over many CTAs: for every panel of NB columns one
+// matrix is spread over many CTAs: for every panel of NB columns one
 // CTA eliminates the panel (partial pivoting among rows not yet used; the
 // same arithmetic, order and panel width as k_gj, so the results are
-// identical) and then one CTA per 32-column block applies the rank-NB update
-// to its columns,
+// identical) and then one CTA per block of 32, 8 or 4 columns applies the
+// rank-NB update to its columns,
 //   X[i][j] <- [i not a pivot of the panel] X[i][j] + sum_c P[i][c] X[piv_c][j],
-// two launches per panel.  Grids are fixed (kRedoMax matrices); a list kernel
-// collects the flagged matrices in a deterministic order and marks them
-// handled (flag 2); flagged matrices beyond the list keep flag 1 and go
-// through k_gj.  With nothing flagged every CTA exits at once.
+// two launches per panel.  A list kernel collects the flagged matrices (up to
+// kRedoMax) in a deterministic order and marks them handled (flag 2); flagged
+// matrices beyond the list keep flag 1 and go through k_gj.  The update's CTAs
+// walk over the (matrix, column block) items of the list, with blocks narrow
+// enough to give every SM an item; with nothing flagged every CTA exits at once.
+//
+// launch_gj_wide runs the same kernels over all matrices of a call too few to
+// fill the card with one CTA each (every SM's FP64 pipe is then in use); the
+// matrices' state sits in their own D^-1 arrays until the end.
+// (Rule and times: gj_wide in k_gj.cu.)
+#include <cooperative_groups.h>
 #include <math.h>
 
+#include <algorithm>
+
+#include "gj_panel.cuh"
 #include "qmc_device.cuh"
 
 namespace qmc {
+
+namespace cg = cooperative_groups;
 
 constexpr int kRThreads = 256;
 constexpr int kRWarps = kRThreads / 32;
@@ -42,46 +54,35 @@ struct RedoState {
 
 struct RedoArgs {
     GjJob j[2];
-    RedoList *list;
+    RedoList *list;        // null: every matrix of both jobs, in order
+    int n_all;             // their number
     char *state;           // kRedoMax entries of state_stride bytes
     size_t state_stride;
     int nmax;
     int e_off[2];          // first electron of each job's spin
 };
 
-__device__ __forceinline__ RedoState *rstate(const RedoArgs &a, int b)
+__device__ __forceinline__ int rcount(const RedoArgs &a) { return a.list ? a.list->count : a.n_all; }
+__device__ __forceinline__ RedoEntry rentry(const RedoArgs &a, int b)
 {
-    return reinterpret_cast<RedoState *>(a.state + (size_t)b * a.state_stride);
+    if (a.list) return a.list->e[b];
+    RedoEntry en;
+    en.job = b >= a.j[0].count;
+    en.m = en.job ? b - a.j[0].count : b;
+    return en;
 }
-__device__ __forceinline__ short *rpp(const RedoArgs &a, int b)
+__device__ __forceinline__ RedoState *rstate(const RedoArgs &a, int b, const RedoEntry &en)
 {
-    return reinterpret_cast<short *>(a.state + (size_t)b * a.state_stride + 16);
+    return reinterpret_cast<RedoState *>(a.list ? (void *)(a.state + (size_t)b * a.state_stride)
+                                                : (void *)(a.j[en.job].Dinv + (size_t)en.m * a.j[en.job].d_stride));
 }
-__device__ __forceinline__ short *rpanel(const RedoArgs &a, int b)
-{
-    return rpp(a, b) + a.nmax;
-}
+__device__ __forceinline__ short *rpp(RedoState *st) { return reinterpret_cast<short *>(st + 1); }
+__device__ __forceinline__ short *rpanel(RedoState *st, int n) { return rpp(st) + n; }
 
 size_t redo_scratch_bytes(int nmax)
 {
     const size_t stride = (16 + 4 * (size_t)nmax + 255) & ~size_t(255);
     return ((sizeof(RedoList) + 255) & ~size_t(255)) + kRedoMax * stride;
-}
-
-__device__ __forceinline__ void rargmax(double &v, int &i, double v2, int i2)
-{
-    if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
-}
-
-__device__ __forceinline__ void rblock_argmax(double &bv, int &bi, double *red_v, int *red_i, int lane, int wid)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double v2 = __shfl_down_sync(0xffffffffu, bv, o);
-        const int i2 = __shfl_down_sync(0xffffffffu, bi, o);
-        rargmax(bv, bi, v2, i2);
-    }
-    if (lane == 0) { red_v[wid] = bv; red_i[wid] = bi; }
 }
 
 // Collect flagged matrices (flag 1) of both jobs, job 0 first, in index order.
@@ -124,171 +125,164 @@ __global__ void __launch_bounds__(1024) k_redo_list(RedoArgs a, int n_jobs)
     if (t == 0) a.list->count = min(s_base, kRedoMax);
 }
 
-// Eliminate panel [jb, jb + w) of every listed matrix (one CTA each).
+// Eliminate panel [jb, jb + w) of every matrix (one CTA each).
 template <int kRNB>
 __global__ void __launch_bounds__(kRThreads) k_redo_panel(RedoArgs a, int jb)
 {
     const int b = blockIdx.x;
-    if (b >= a.list->count) return;
-    const RedoEntry en = a.list->e[b];
+    if (b >= rcount(a)) return;
+    const RedoEntry en = rentry(a, b);
     const GjJob &J = a.j[en.job];
     const int n = J.n;
     if (jb >= n) return;
-    RedoState *stt = rstate(a, b);
-    short *pp = rpp(a, b), *panel = rpanel(a, b);
+    RedoState *stt = rstate(a, b, en);
+    short *pp = rpp(stt), *panel = rpanel(stt, n);
     double *__restrict__ X = J.X + (size_t)en.m * J.x_stride;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *P = reinterpret_cast<double *>(smem_raw);             // [n][kRNB]
     short *used = reinterpret_cast<short *>(P + (size_t)n * kRNB);  // [n]
-    __shared__ double red_v[kRWarps];
-    __shared__ int red_i[kRWarps];
-    __shared__ int s_p, s_sing;
-    __shared__ double s_logabs;
-    __shared__ int s_neg;
+    __shared__ GjPanelShared<kRNB> S;
 
     if (jb == 0) {
         for (int i = t; i < n; i += kRThreads) panel[i] = -1;
         if (t == 0) { stt->logabs = 0.0; stt->neg = 0; stt->sing = 0; }
         __syncthreads();
     }
-    if (t == 0) { s_sing = stt->sing; s_logabs = stt->logabs; s_neg = stt->neg; }
-    __syncthreads();
-    if (s_sing) return;
+    if (stt->sing) return;
     const int w = min(kRNB, n - jb);
     for (int i = t; i < n; i += kRThreads) used[i] = panel[i] >= 0;
     for (int q = t; q < n * kRNB; q += kRThreads) {
         const int i = q / kRNB, c = q - i * kRNB;
-        P[q] = (c < w) ? X[(size_t)i * n + jb + c] : 0.0;
+        P[gj_at<kRNB>(i, c)] = (c < w) ? X[(size_t)i * n + jb + c] : 0.0;
     }
     __syncthreads();
-    double bv = -1.0;
-    int bi = n;
-    for (int i = t; i < n; i += kRThreads)
-        if (!used[i]) rargmax(bv, bi, fabs(P[i * kRNB]), i);
-    rblock_argmax(bv, bi, red_v, red_i, lane, wid);
-    __syncthreads();
-    for (int c = 0; c < w; ++c) {
-        if (t == 0) {
-            double v = red_v[0];
-            int p = red_i[0];
-            for (int q = 1; q < kRWarps; ++q) rargmax(v, p, red_v[q], red_i[q]);
-            s_p = p;
-            if (!(v > 0.0)) s_sing = 1;
+    const bool ok = gj_panel<kRNB>(P, n, w, used, S);
+    if (wid == 0) {
+        double logabs = stt->logabs;
+        int neg = stt->neg;
+        __syncwarp();
+        if (ok) {
+            gj_add_pivots<kRNB>(S, w, logabs, neg);
+            if (lane < w) {
+                pp[jb + lane] = S.pp[lane];
+                panel[S.pp[lane]] = (short)jb;
+            }
         }
-        __syncthreads();
-        if (s_sing) break;
-        const int p = s_p;
-        const double piv = P[p * kRNB + c];
-        const double inv = 1.0 / piv;
-        if (t == 0) {
-            used[p] = 1;
-            pp[jb + c] = (short)p;
-            panel[p] = (short)jb;
-            s_logabs += log(fabs(piv));
-            s_neg ^= (piv < 0.0);
-        }
-        __syncthreads();
-        if (t < kRNB) P[p * kRNB + t] = (t == c) ? inv : P[p * kRNB + t] * inv;
-        __syncthreads();
-        double nbv = -1.0;
-        int nbi = n;
-        const int cn = c + 1;
-        for (int i = t; i < n; i += kRThreads) {
-            if (i == p) continue;
-            const double f = P[i * kRNB + c];
-#pragma unroll
-            for (int cc = 0; cc < kRNB; ++cc)
-                if (cc != c) P[i * kRNB + cc] = fma(-f, P[p * kRNB + cc], P[i * kRNB + cc]);
-            P[i * kRNB + c] = -f * inv;
-            if (cn < w && !used[i]) rargmax(nbv, nbi, fabs(P[i * kRNB + cn]), i);
-        }
-        rblock_argmax(nbv, nbi, red_v, red_i, lane, wid);
-        __syncthreads();
+        if (lane == 0) { stt->sing = !ok; stt->logabs = logabs; stt->neg = neg; }
     }
-    if (!s_sing)
+    if (ok)
         for (int q = t; q < n * w; q += kRThreads) {
             const int i = q / w, c = q - i * w;
-            X[(size_t)i * n + jb + c] = P[i * kRNB + c];
+            X[(size_t)i * n + jb + c] = P[gj_at<kRNB>(i, c)];
         }
-    if (t == 0) { stt->sing = s_sing; stt->logabs = s_logabs; stt->neg = s_neg; }
 }
 
-// Rank-w update of the 32 columns of block blockIdx.x of every listed matrix.
+// Rank-w update of the matrices' columns outside the panel, in blocks of 32, 8 or 4 columns: the
+// widest that give each of 152 SMs two items (a block owns its columns: its pivot rows are read
+// before its rows are written).
 template <int kRNB>
 __global__ void __launch_bounds__(kRThreads) k_redo_update(RedoArgs a, int jb)
 {
-    const int b = blockIdx.y;
-    if (b >= a.list->count) return;
-    const RedoEntry en = a.list->e[b];
-    const GjJob &J = a.j[en.job];
-    const int n = J.n;
-    const int c0 = blockIdx.x * 32;
-    if (jb >= n || c0 >= n) return;
-    const int w = min(kRNB, n - jb);
-    if (c0 >= jb && c0 + 32 <= jb + w) return;            // entirely inside the panel
-    const RedoState *stt = rstate(a, b);
-    if (stt->sing) return;
-    const short *pp = rpp(a, b), *panel = rpanel(a, b);
-    double *__restrict__ X = J.X + (size_t)en.m * J.x_stride;
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int count = rcount(a);
+    int lc = 5;
+    if ((long long)count * ((a.nmax + 31) / 32) < 304) lc = (long long)count * ((a.nmax + 7) / 8) < 304 ? 2 : 3;
+    const int nblk = (a.nmax + (1 << lc) - 1) >> lc, items = count * nblk;
+    const int t = threadIdx.x, cols = 1 << lc;
+    const int cl = t & (cols - 1), r0 = t >> lc, rstep = kRThreads >> lc;   // a thread's column and rows
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *P = reinterpret_cast<double *>(smem_raw);   // [n][kRNB]
-    double *U = P + (size_t)n * kRNB;                    // [kRNB][32]
-    for (int q = t; q < n * kRNB; q += kRThreads) {
-        const int i = q / kRNB, c = q - i * kRNB;
-        P[q] = (c < w) ? X[(size_t)i * n + jb + c] : 0.0;
-    }
-    for (int q = t; q < kRNB * 32; q += kRThreads) {
-        const int c = q >> 5, col = c0 + (q & 31);
-        U[q] = (c < w && col < n) ? X[(size_t)pp[jb + c] * n + col] : 0.0;
-    }
-    __syncthreads();
-    const int col = c0 + lane;
-    if (col >= n || (col >= jb && col < jb + w)) return;
-    double u[kRNB];
-#pragma unroll
-    for (int c = 0; c < kRNB; ++c) u[c] = U[c * 32 + lane];
-    for (int i = wid; i < n; i += kRWarps) {
-        double x = (panel[i] == jb) ? 0.0 : X[(size_t)i * n + col];
-        const double2 *pr = reinterpret_cast<const double2 *>(P + i * kRNB);
-#pragma unroll
-        for (int c2 = 0; c2 < kRNB / 2; ++c2) {
-            const double2 pv = pr[c2];
-            x = fma(pv.x, u[2 * c2], x);
-            x = fma(pv.y, u[2 * c2 + 1], x);
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int b = it / nblk, c0 = (it - b * nblk) << lc;
+        const RedoEntry en = rentry(a, b);
+        const GjJob &J = a.j[en.job];
+        const int n = J.n;
+        if (jb >= n || c0 >= n) continue;
+        const int w = min(kRNB, n - jb);
+        if (c0 >= jb && c0 + cols <= jb + w) continue;    // entirely inside the panel
+        RedoState *stt = rstate(a, b, en);
+        if (stt->sing) continue;
+        const short *pp = rpp(stt), *panel = rpanel(stt, n);
+        double *__restrict__ X = J.X + (size_t)en.m * J.x_stride;
+        __syncthreads();                                  // the previous item's reads of P
+        for (int q = t; q < n * kRNB; q += kRThreads) {
+            const int i = q / kRNB, c = q - i * kRNB;
+            P[gj_at<kRNB>(i, c)] = (c < w) ? X[(size_t)i * n + jb + c] : 0.0;
         }
-        X[(size_t)i * n + col] = x;
+        const int col = c0 + cl;
+        const bool active = col < n && !(col >= jb && col < jb + w);
+        double u[kRNB];
+#pragma unroll
+        for (int c = 0; c < kRNB; ++c) u[c] = (active && c < w) ? X[(size_t)pp[jb + c] * n + col] : 0.0;
+        __syncthreads();                                  // every pivot row has been read
+        if (!active) continue;
+        int i = r0;
+        for (; i + 3 * rstep < n; i += 4 * rstep) {       // four rows: independent chains
+            double x[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int ii = i + r * rstep;
+                x[r] = (panel[ii] == jb) ? 0.0 : X[(size_t)ii * n + col];
+            }
+#pragma unroll
+            for (int c2 = 0; c2 < kRNB / 2; ++c2)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const double2 pv = *reinterpret_cast<const double2 *>(P + gj_at<kRNB>(i + r * rstep, 2 * c2));
+                    x[r] = fma(pv.x, u[2 * c2], x[r]);
+                    x[r] = fma(pv.y, u[2 * c2 + 1], x[r]);
+                }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) X[(size_t)(i + r * rstep) * n + col] = x[r];
+        }
+        for (; i < n; i += rstep) {
+            double x = (panel[i] == jb) ? 0.0 : X[(size_t)i * n + col];
+#pragma unroll
+            for (int c2 = 0; c2 < kRNB / 2; ++c2) {
+                const double2 pv = *reinterpret_cast<const double2 *>(P + gj_at<kRNB>(i, 2 * c2));
+                x = fma(pv.x, u[2 * c2], x);
+                x = fma(pv.y, u[2 * c2 + 1], x);
+            }
+            X[(size_t)i * n + col] = x;
+        }
     }
 }
 
-// D^-1, log|det| and sign of every listed matrix: Dinv[pp[c]][k] = Res[pp[k]][c].
-__global__ void __launch_bounds__(kRThreads) k_redo_final(RedoArgs a)
+// D^-1, log|det| and sign of every matrix: Dinv[pp[c]][k] = Res[pp[k]][c], one cluster per matrix
+// at a time (one CTA took 744 us for n = 528).
+constexpr int kFinalCluster = 8;
+
+__global__ void __cluster_dims__(kFinalCluster, 1, 1) __launch_bounds__(kRThreads) k_redo_final(RedoArgs a)
 {
-    const int b = blockIdx.x;
-    if (b >= a.list->count) return;
-    const RedoEntry en = a.list->e[b];
-    const GjJob &J = a.j[en.job];
-    const int n = J.n, m = en.m;
-    const RedoState *stt = rstate(a, b);
-    const short *pp = rpp(a, b);
-    const double *__restrict__ X = J.X + (size_t)m * J.x_stride;
-    double *__restrict__ Dout = J.Dinv + (size_t)m * J.d_stride;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     __shared__ double tile[32 * 33];
-    __shared__ unsigned char seen[1024];
-    if (stt->sing) {
-        const double qnan = __longlong_as_double(0x7ff8000000000000ll);
-        for (size_t q = t; q < (size_t)n * n; q += kRThreads) Dout[q] = qnan;
-        if (t == 0) {
-            if (J.logabs) J.logabs[(size_t)m * J.la_stride] = -INFINITY;
-            if (J.sign) J.sign[(size_t)m * J.la_stride] = 0.0;
-            if (J.flag) atomicOr(J.flag + m, J.flag_bit);
+    __shared__ short pp[1024];
+    const int count = rcount(a);
+    for (int b = blockIdx.x / kFinalCluster; b < count; b += gridDim.x / kFinalCluster) {
+        const RedoEntry en = rentry(a, b);
+        const GjJob &J = a.j[en.job];
+        const int n = J.n, m = en.m;
+        const double *__restrict__ X = J.X + (size_t)m * J.x_stride;
+        double *__restrict__ Dout = J.Dinv + (size_t)m * J.d_stride;
+        RedoState *sp = rstate(a, b, en);
+        const RedoState st0 = *sp;
+        for (int i = t; i < n; i += kRThreads) pp[i] = rpp(sp)[i];
+        cluster.sync();                                    // the state may lie in Dout
+        if (st0.sing) {
+            const double qnan = __longlong_as_double(0x7ff8000000000000ll);
+            for (size_t q = (size_t)rank * kRThreads + t; q < (size_t)n * n; q += kFinalCluster * kRThreads) Dout[q] = qnan;
+            if (t == 0 && rank == 0) {
+                if (J.logabs) J.logabs[(size_t)m * J.la_stride] = -INFINITY;
+                if (J.sign) J.sign[(size_t)m * J.la_stride] = 0.0;
+                if (J.flag) atomicOr(J.flag + m, J.flag_bit);
+            }
+            continue;
         }
-        return;
-    }
-    for (int kb = 0; kb < n; kb += 32)
-        for (int cb = 0; cb < n; cb += 32) {
+        const int nt = (n + 31) / 32;
+        for (int q = rank; q < nt * nt; q += kFinalCluster) {
+            const int kb = q / nt * 32, cb = (q - q / nt * nt) * 32;
             for (int r = wid; r < 32; r += kRWarps) {
                 const int k = kb + r, c = cb + lane;
                 tile[r * 33 + lane] = (k < n && c < n) ? X[(size_t)pp[k] * n + c] : 0.0;
@@ -300,17 +294,18 @@ __global__ void __launch_bounds__(kRThreads) k_redo_final(RedoArgs a)
             }
             __syncthreads();
         }
-    if (t == 0) {
-        int par = 0;
-        for (int i = 0; i < n; ++i) seen[i] = 0;
-        for (int i = 0; i < n; ++i) {
-            if (seen[i]) continue;
-            int len = 0, j = i;
-            while (!seen[j]) { seen[j] = 1; j = pp[j]; ++len; }
-            par ^= ((len & 1) == 0);
+        if (rank == 0) {
+            // parity of the row permutation k -> pp[k]: its inversions
+            int inv = 0;
+            for (int i = t; i < n; i += kRThreads)
+                for (int j = i + 1; j < n; ++j) inv ^= pp[j] < pp[i];
+            const int odd = __syncthreads_count(inv) & 1;
+            if (t == 0) {
+                if (J.logabs) J.logabs[(size_t)m * J.la_stride] = st0.logabs;
+                if (J.sign) J.sign[(size_t)m * J.la_stride] = (odd ^ st0.neg) ? -1.0 : 1.0;
+            }
         }
-        if (J.logabs) J.logabs[(size_t)m * J.la_stride] = stt->logabs;
-        if (J.sign) J.sign[(size_t)m * J.la_stride] = (par ^ stt->neg) ? -1.0 : 1.0;
+        __syncthreads();                                   // pp is rewritten for the next matrix
     }
 }
 
@@ -376,7 +371,7 @@ template <int NB>
 static cudaError_t launch_redo_panels(const RedoArgs &a, int nmax, cudaStream_t st)
 {
     const size_t smp = sizeof(double) * (size_t)nmax * NB + sizeof(short) * nmax;
-    const size_t smu = sizeof(double) * ((size_t)nmax * NB + NB * 32);
+    const size_t smu = sizeof(double) * (size_t)nmax * NB;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k_redo_panel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smp)) !=
         cudaSuccess)
@@ -384,11 +379,50 @@ static cudaError_t launch_redo_panels(const RedoArgs &a, int nmax, cudaStream_t 
     if ((e = cudaFuncSetAttribute(k_redo_update<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smu)) !=
         cudaSuccess)
         return e;
-    const dim3 ugrid((nmax + 31) / 32, kRedoMax);
+    // update: two or three CTAs on each of 152 SMs walk over the items
+    const unsigned ugrid = a.list ? 456 : (unsigned)std::min<long long>(456 * 8, (long long)a.n_all * ((nmax + 3) / 4));
     for (int jb = 0; jb < nmax; jb += NB) {
-        k_redo_panel<NB><<<kRedoMax, kRThreads, smp, st>>>(a, jb);
+        k_redo_panel<NB><<<a.list ? kRedoMax : a.n_all, kRThreads, smp, st>>>(a, jb);
         k_redo_update<NB><<<ugrid, kRThreads, smu, st>>>(a, jb);
     }
+    return cudaGetLastError();
+}
+
+static cudaError_t launch_redo_nb(const RedoArgs &a, int nmax, cudaStream_t st, int nb)
+{
+    switch (nb) {
+    case 8: return launch_redo_panels<8>(a, nmax, st);
+    case 16: return launch_redo_panels<16>(a, nmax, st);
+    case 32: return launch_redo_panels<32>(a, nmax, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+static int redo_jobs(RedoArgs &a, const GjJob *jobs, int n_jobs)
+{
+    a.nmax = 0;
+    for (int q = 0; q < 2; ++q) {
+        a.j[q] = jobs[q < n_jobs ? q : 0];
+        if (q >= n_jobs) a.j[q].count = 0;
+        if (a.j[q].count > 0) a.nmax = max(a.nmax, a.j[q].n);
+    }
+    a.n_all = a.j[0].count + a.j[1].count;
+    a.e_off[0] = a.e_off[1] = 0;
+    a.list = nullptr;
+    a.state = nullptr;
+    a.state_stride = 0;
+    return a.nmax;
+}
+
+// Every matrix of the jobs through the kernels above.
+cudaError_t launch_gj_wide(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb)
+{
+    RedoArgs a;
+    const int nmax = redo_jobs(a, jobs, n_jobs);
+    if (a.n_all == 0) return cudaSuccess;
+    const cudaError_t e = launch_redo_nb(a, nmax, st, nb);
+    if (e != cudaSuccess) return e;
+    k_redo_final<<<kFinalCluster * std::min(a.n_all, 1024), kRThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -399,15 +433,9 @@ cudaError_t launch_gj_redo(const GjJob *jobs, int n_jobs, void *scratch, cudaStr
                            const double *R, const int *e_off)
 {
     RedoArgs a;
-    int nmax = 0;
-    for (int q = 0; q < 2; ++q) {
-        a.j[q] = jobs[q < n_jobs ? q : 0];
-        if (q >= n_jobs) a.j[q].count = 0;
-        nmax = max(nmax, a.j[q].n);
-    }
+    const int nmax = redo_jobs(a, jobs, n_jobs);
     if (n_jobs == 0 || nmax == 0) return cudaSuccess;
     if (nmax > 1024) return cudaErrorInvalidValue;
-    a.nmax = nmax;
     a.list = static_cast<RedoList *>(scratch);
     a.state = static_cast<char *>(scratch) + ((sizeof(RedoList) + 255) & ~size_t(255));
     a.state_stride = (16 + 4 * (size_t)nmax + 255) & ~size_t(255);
@@ -423,14 +451,9 @@ cudaError_t launch_gj_redo(const GjJob *jobs, int n_jobs, void *scratch, cudaStr
         k_redo_c1<<<dim3(nmax, kC1Slots), kC1Threads, sm, st>>>(*s, a, R);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    switch (nb) {
-    case 8: e = launch_redo_panels<8>(a, nmax, st); break;
-    case 16: e = launch_redo_panels<16>(a, nmax, st); break;
-    case 32: e = launch_redo_panels<32>(a, nmax, st); break;
-    default: return cudaErrorInvalidValue;
-    }
+    e = launch_redo_nb(a, nmax, st, nb);
     if (e != cudaSuccess) return e;
-    k_redo_final<<<kRedoMax, kRThreads, 0, st>>>(a);
+    k_redo_final<<<kFinalCluster * 38, kRThreads, 0, st>>>(a);   // two CTAs on each of 152 SMs
     return cudaGetLastError();
 }
 

@@ -135,6 +135,8 @@ cudaError_t launch_vdrift_f64(const SysDev &s, int nw, const double *R, const do
 cudaError_t launch_screen_ao(const SysDev &s, int nw, const double *R, int cap, int32_t *cnt,
                              int32_t *idx, double *B, cudaStream_t st);
 cudaError_t launch_gj(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb);
+// The same elimination with each matrix spread over many CTAs (k_gj_redo.cu).
+cudaError_t launch_gj_wide(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb);
 // Multi-CTA FP64 recomputation of up to kRedoMax flagged matrices (redo 1 -> 2).
 constexpr int kRedoMax = 256;
 size_t redo_scratch_bytes(int nmax);

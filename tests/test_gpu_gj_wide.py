@@ -1,0 +1,47 @@
+"""FP64 elimination with each matrix spread over many CTAs (few matrices) against
+one CTA per matrix: the same arithmetic in the same order, so bit for bit the
+same log|det|, sign and inverse; singular matrices, pivot ties, zeros and
+non-finite entries among them.  One CTA per matrix runs on the batch repeated
+until it fills the card (304 matrices: two on each of 152 SMs)."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+dev = torch.device("cuda", 0)
+
+
+def _inv(X):
+    from paper_1209_6630_gb300 import det_inverse
+    return det_inverse(X.clone())
+
+
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 15, 16, 17, 31, 32, 33, 63, 64, 65, 100, 217, 255, 256, 257, 300])
+def test_wide_equals_one_cta_per_matrix(n):
+    g = torch.Generator(device="cuda").manual_seed(n)
+    X = torch.randn(8, n, n, dtype=torch.float64, device=dev, generator=g)
+    X[1] = X[1].round()                              # ties
+    X[2, :, n // 2] = 0.0                            # an exactly zero column
+    X[3, n // 3, :] = X[3, 0, :]                      # (n > 1) two equal rows
+    X[4, 0, 0] = float("nan")
+    X[5, n - 1, 0] = float("inf")
+    X[6] = torch.eye(n, dtype=torch.float64, device=dev).flip(0)
+    few = _inv(X)
+    many = _inv(X.repeat(38, 1, 1))
+    for a, b in zip(few, many):
+        b = b[:8]
+        assert torch.equal(torch.isnan(a), torch.isnan(b)) if a.is_floating_point() else True
+        assert torch.equal(a.nan_to_num(0.0), b.nan_to_num(0.0)) if a.is_floating_point() else torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n,batch", [(512, 2), (640, 1), (866, 1), (1024, 2)])
+def test_wide_large_inverse(n, batch):
+    """Against torch in FP64 (LU): both within n x 2^-53 x kappa of the inverse; kappa <= 1e6 for these."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    X = torch.randn(batch, n, n, dtype=torch.float64, device=dev, generator=g)
+    X += 3.0 * n ** 0.5 * torch.eye(n, dtype=torch.float64, device=dev)
+    logabs, sign, D, sing = _inv(X)
+    s, l = torch.linalg.slogdet(X)
+    assert torch.equal(s, sign) and not sing.any()
+    assert ((logabs - l).abs() / l.abs()).max().item() < 1e-10
+    E = D.mT @ X - torch.eye(n, dtype=torch.float64, device=dev)
+    assert E.abs().max().item() < n * 2.0 ** -53 * 1e6
