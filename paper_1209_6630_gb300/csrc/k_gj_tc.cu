@@ -41,17 +41,21 @@
 // result or an expired bounded wait are flagged, and the FP64 recomputation
 // (C1 from the positions and the FP64 elimination) replaces them, exactly as
 // for k_gj_ff.
+#include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
 
 #include <algorithm>
 
+#include "f64_bits.cuh"
 #include "ff_math.cuh"
 #include "qmc_internal.cuh"
 #include "slices.cuh"
 #include "umma.cuh"
 
 namespace qmc {
+
+namespace cg = cooperative_groups;
 
 constexpr int kGtB = 32;                             // panel width = K of the update
 constexpr int kGtThreads = 256;                      // init and final kernels
@@ -139,11 +143,17 @@ __device__ __forceinline__ void gt_block_argmax(float &bv, int &bi, float *red_v
     if (lane == 0) { red_v[wid] = bv; red_i[wid] = bi; }
 }
 
+// Float-pair copy of X and ||X||_inf; a cluster of CTAs shares a matrix's rows where the matrices
+// are few.  Both this kernel and k_gt_final only move data, but were bound by the FP64 pipe's
+// conversions; on the integer pipes (f64_bits.cuh), 4096 matrices of 528 rows: 8.5 -> 3.8 ms
+// (18.3 GB, 4.9 TB/s); 74 matrices, spread: 0.69 -> 0.11 ms.
 __global__ void __launch_bounds__(kGtThreads) k_gt_init(GtJobs js)
 {
+    cg::cluster_group cluster = cg::this_cluster();
+    const int nrank = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const GjJob &J = js.j[blockIdx.y];
-    const int m = blockIdx.x;
-    if (m >= J.count) return;
+    const int m = blockIdx.x / nrank;
+    if (m >= J.count) return;                            // (the same for a whole cluster)
     const int n = J.n;
     const GtLayout L = gt_layout(n);
     unsigned char *sc = js.scr[blockIdx.y] + (size_t)m * L.per;
@@ -152,36 +162,44 @@ __global__ void __launch_bounds__(kGtThreads) k_gt_init(GtJobs js)
     const int ld = gt_ld(n);
     short *used = reinterpret_cast<short *>(sc + L.used);
     unsigned char *piv = sc + L.piv;
-    GtState *st = reinterpret_cast<GtState *>(sc + L.state);
     __shared__ float red_f[kGtWarps];
+    __shared__ float s_max;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     float rmax = 0.f;
-    for (int i = wid; i < n; i += kGtWarps) {
+    for (int i = rank * kGtWarps + wid; i < n; i += nrank * kGtWarps) {
         float rs = 0.f;
+#pragma unroll 4
         for (int c = lane; c < n; c += 32) {
-            const double x = X[(size_t)i * n + c];
-            const float h = (float)x;
-            Wk[(size_t)i * ld + c] = make_float2(h, (float)(x - (double)h));
-            rs += fabsf(h);
+            const float2 v = split_f64(X[(size_t)i * n + c]);
+            Wk[(size_t)i * ld + c] = v;
+            rs += fabsf(v.x);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
         rmax = fmaxf(rmax, rs);
     }
     if (lane == 0) red_f[wid] = rmax;
-    for (int i = t; i < n; i += kGtThreads) {
-        used[i] = 0;
-        piv[i] = 0;
-    }
+    if (rank == 0)
+        for (int i = t; i < n; i += kGtThreads) {
+            used[i] = 0;
+            piv[i] = 0;
+        }
     __syncthreads();
     if (t == 0) {
         float xm = 0.f;
         for (int q = 0; q < kGtWarps; ++q) xm = fmaxf(xm, red_f[q]);
+        s_max = xm;
+    }
+    if (nrank > 1) cluster.sync();
+    if (t == 0 && rank == 0) {
+        float xm = s_max;
+        for (int r = 1; r < nrank; ++r) xm = fmaxf(xm, *cluster.map_shared_rank(&s_max, r));
         GtState s0;
         s0.mag_h = 1.f; s0.mag_l = 0.f; s0.mag_e = 0; s0.neg = 0; s0.sing = 0; s0.xnorm = xm;
         s0.pad[0] = s0.pad[1] = 0;
-        *st = s0;
+        *reinterpret_cast<GtState *>(sc + L.state) = s0;
     }
+    if (nrank > 1) cluster.sync();                       // no CTA leaves before its maximum is read
 }
 
 // Operand B of the update: the pivot rows before the update (zero in the panel's columns
@@ -904,74 +922,120 @@ __global__ void __launch_bounds__(kGtUpThreads, 1) k_gt_update(const __grid_cons
     (void)nst;
 }
 
+// ||X^-1||_inf (the rows of X^-1 are the rows of the result, columns permuted) and
+// D^-1 = X^-T in one pass over the result, 32 x 32 tiles; a cluster shares a matrix's row blocks
+// where the matrices are few.  4096 matrices of 528 rows: 7.3 -> 3.7 ms;
+// 74, spread: 1.12 -> 0.13 ms.
 __global__ void __launch_bounds__(kGtThreads) k_gt_final(GtJobs js, double kappa_max)
 {
+    cg::cluster_group cluster = cg::this_cluster();
+    const int nrank = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const GjJob &J = js.j[blockIdx.y];
-    const int m = blockIdx.x;
-    if (m >= J.count) return;
+    const int m = blockIdx.x / nrank;
+    if (m >= J.count) return;                            // (the same for a whole cluster)
     const int n = J.n;
     const GtLayout L = gt_layout(n);
     unsigned char *sc = js.scr[blockIdx.y] + (size_t)m * L.per;
     const GtState S = *reinterpret_cast<const GtState *>(sc + L.state);
     if (S.sing) {                                        // a zero pivot in the float pairs: FP64 decides
-        if (threadIdx.x == 0 && J.redo) J.redo[m * J.redo_stride] = 1;
+        if (threadIdx.x == 0 && rank == 0 && J.redo) J.redo[m * J.redo_stride] = 1;
         return;
     }
     const float2 *__restrict__ Wk = reinterpret_cast<const float2 *>(sc + L.w);
     const int ld = gt_ld(n);
     double *__restrict__ Dout = J.Dinv + (size_t)m * J.d_stride;
     const short *pp_g = reinterpret_cast<const short *>(sc + L.pp);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *tile = reinterpret_cast<float2 *>(smem_raw);        // [32][33]
-    short *pp = reinterpret_cast<short *>(tile + 32 * 33);
-    short *seen = pp + n;
+    __shared__ float2 tile[2][32 * 33];
+    __shared__ short pp[1024];
     __shared__ float red_f[kGtWarps];
+    __shared__ float s_max;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    for (int i = t; i < n; i += kGtThreads) {
-        pp[i] = pp_g[i];
-        seen[i] = 0;
-    }
-    // ||X^-1||_inf: the rows of X^-1 are the rows of the result (columns permuted)
+    constexpr int RW = 32 / kGtWarps;                    // rows of a tile per warp
+    for (int i = t; i < n; i += kGtThreads) pp[i] = pp_g[i];
+    __syncthreads();
     float imax = 0.f;
-    for (int i = wid; i < n; i += kGtWarps) {
-        float rs = 0.f;
-        for (int c = lane; c < n; c += 32) rs += fabsf(Wk[(size_t)i * ld + c].x);
+    int buf = 0;
+    for (int kb = 32 * rank; kb < n; kb += 32 * nrank) {
+        float rs[RW];
+        const float2 *row[RW];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
-        imax = fmaxf(imax, rs);
+        for (int r = 0; r < RW; ++r) {
+            const int k = kb + wid + r * kGtWarps;
+            rs[r] = 0.f;
+            row[r] = k < n ? Wk + (size_t)pp[k] * ld : nullptr;
+        }
+        // the tiles alternate between two buffers: one barrier each
+        for (int cb = 0; cb < n; cb += 32, buf ^= 1) {
+            const int c = cb + lane;
+            float2 v[RW];
+#pragma unroll
+            for (int r = 0; r < RW; ++r) v[r] = (row[r] && c < n) ? row[r][c] : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                tile[buf][(wid + r * kGtWarps) * 33 + lane] = v[r];
+                if (c < n) rs[r] += fabsf(v[r].x);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                const int cr = cb + wid + r * kGtWarps, k = kb + lane;
+                if (cr < n && k < n)
+                    Dout[(size_t)pp[cr] * n + k] = join_f64(tile[buf][lane * 33 + wid + r * kGtWarps]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rs[r] += __shfl_xor_sync(0xffffffffu, rs[r], o);
+            imax = fmaxf(imax, rs[r]);
+        }
     }
     if (lane == 0) red_f[wid] = imax;
     __syncthreads();
-    for (int kb = 0; kb < n; kb += 32) {
-        for (int cb = 0; cb < n; cb += 32) {
-            for (int r = wid; r < 32; r += kGtWarps) {
-                const int k = kb + r, c = cb + lane;
-                tile[r * 33 + lane] = (k < n && c < n) ? Wk[(size_t)pp[k] * ld + c] : make_float2(0.f, 0.f);
-            }
-            __syncthreads();
-            for (int r = wid; r < 32; r += kGtWarps) {
-                const int c = cb + r, k = kb + lane;
-                if (c < n && k < n) Dout[(size_t)pp[c] * n + k] = ff::val(tile[lane * 33 + r]);
-            }
-            __syncthreads();
-        }
-    }
     if (t == 0) {
         float im = 0.f;
         for (int q = 0; q < kGtWarps; ++q) im = fmaxf(im, red_f[q]);
-        const double kappa = (double)S.xnorm * (double)im;
-        int par = 0;
-        for (int i = 0; i < n; ++i) {
-            if (seen[i]) continue;
-            int len = 0, j = i;
-            while (!seen[j]) { seen[j] = 1; j = pp[j]; ++len; }
-            par ^= ((len & 1) == 0);
-        }
-        const double logabs = log((double)S.mag_h + (double)S.mag_l) + S.mag_e * 0.69314718055994530942;
-        if (J.logabs) J.logabs[(size_t)m * J.la_stride] = logabs;
-        if (J.sign) J.sign[(size_t)m * J.la_stride] = (par ^ S.neg) ? -1.0 : 1.0;
-        if (J.redo && !(kappa <= kappa_max && isfinite(logabs))) J.redo[m * J.redo_stride] = 1;
+        s_max = im;
     }
+    if (nrank > 1) cluster.sync();
+    if (rank == 0) {
+        // parity of the row permutation k -> pp[k]: its inversions
+        int inv = 0;
+        for (int i = t; i < n; i += kGtThreads)
+            for (int j = i + 1; j < n; ++j) inv ^= pp[j] < pp[i];
+        const int par = __syncthreads_count(inv) & 1;
+        if (t == 0) {
+            float im = s_max;
+            for (int r = 1; r < nrank; ++r) im = fmaxf(im, *cluster.map_shared_rank(&s_max, r));
+            const double kappa = (double)S.xnorm * (double)im;
+            const double logabs = log((double)S.mag_h + (double)S.mag_l) + S.mag_e * 0.69314718055994530942;
+            if (J.logabs) J.logabs[(size_t)m * J.la_stride] = logabs;
+            if (J.sign) J.sign[(size_t)m * J.la_stride] = (par ^ S.neg) ? -1.0 : 1.0;
+            if (J.redo && !(kappa <= kappa_max && isfinite(logabs))) J.redo[m * J.redo_stride] = 1;
+        }
+    }
+    if (nrank > 1) cluster.sync();                       // no CTA leaves before its maximum is read
+}
+
+// init and final: CTAs per matrix, up to 8 (the portable cluster size) while the matrices give
+// fewer than eight CTAs (what an SM holds) to each of 152 SMs
+template <typename... Args>
+static cudaError_t gt_clusters(void (*kern)(Args...), dim3 g1, int n_jobs, cudaStream_t st, Args... args)
+{
+    unsigned c = 1;
+    while (c < 8 && (size_t)g1.x * n_jobs * c < 152 * 8) c *= 2;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = c;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(g1.x * c, g1.y);
+    cfg.blockDim = dim3(kGtThreads);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 bool gjtc_fits(int nmax)
@@ -1033,7 +1097,6 @@ cudaError_t launch_gj_tc(const GjJob *jobs, int n_jobs, void *scratch, cudaStrea
     // column exponents: one CTA per SM
     const size_t sm_up = 1024 + kGtSl * (size_t)(kGtAPlane + kGtBs * kGtBPlane) + kGtXs * (size_t)kGtXStage +
                          8 * (size_t)((nmax + kGtN - 1) / kGtN * kGtN);
-    const size_t sm_fin = sizeof(float2) * 32 * 33 + sizeof(short) * 2 * (size_t)nmax;
     cudaError_t e;
     if ((e = gt_tensor_maps(js)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_gt_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_panel)) !=
@@ -1047,11 +1110,8 @@ cudaError_t launch_gj_tc(const GjJob *jobs, int n_jobs, void *scratch, cudaStrea
     if ((e = cudaFuncSetAttribute(k_gt_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_up)) !=
         cudaSuccess)
         return e;
-    if ((e = cudaFuncSetAttribute(k_gt_final, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_fin)) !=
-        cudaSuccess)
-        return e;
     const dim3 g1(cmax, n_jobs);
-    k_gt_init<<<g1, kGtThreads, 0, st>>>(js);
+    if ((e = gt_clusters(k_gt_init, g1, n_jobs, st, js)) != cudaSuccess) return e;
     const int nt = (nmax + 127) / 128;
     const int nz = cmax * n_jobs;
     for (int jb = 0; jb < nmax; jb += kGtB) {
@@ -1065,7 +1125,7 @@ cudaError_t launch_gj_tc(const GjJob *jobs, int n_jobs, void *scratch, cudaStrea
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    k_gt_final<<<g1, kGtThreads, sm_fin, st>>>(js, kappa_max);
+    if ((e = gt_clusters(k_gt_final, g1, n_jobs, st, js, kappa_max)) != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
