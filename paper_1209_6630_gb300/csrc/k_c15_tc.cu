@@ -73,6 +73,7 @@ struct C15TcArgs {
     int n_tiles;                   // walker tiles of 128
     int kmax_steps;                // staging capacity per (electron, tile), in K steps
     int prows;                     // rows of a staged operand plane: 128, or a single tile's walkers rounded up to 8
+    int group;                     // rows per producer CTA (a power of two)
     int planes_per_stage;          // 18 (C1, C5, gradients), or 6 (C1 alone)
     unsigned char *planes;         // [batch e][tile][kmax_steps][2][planes_per_stage][prows x 64 bytes]
     int *ao_list;                  // [batch e][tile][kmax_steps * 64]
@@ -199,11 +200,15 @@ __global__ void __launch_bounds__(kPrepThreads, kC1Only ? 3 : 2) k_c15_prep(C15T
     // thread -> (row, every n_slot-th chunk of 8 AOs): a warp's lanes hold different walkers at the
     // same AOs, so the shells' loops are uniform in a warp; a tile of few walkers (rp, the power
     // of two that holds its rows) spreads its AO chunks over the threads that have no row
+    // (row groups share a tile where the (electron, tile) pairs are few: each forms the
+    // whole tile's union list and produces its own rows)
     const int rv = min(TC_M, a.nw - tile * TC_M);
-    const int lrp = 32 - __clz(rv - 1), rp = 1 << lrp;          // rv = 1: __clz(0) = 32, rp = 1
-    const int t = threadIdx.x, row = t & (rp - 1), slot_c = t >> lrp, n_slot = kPrepThreads >> lrp;
+    const int r0 = (int)blockIdx.z * a.group, rvg = min(a.group, rv - r0);
+    if (rvg <= 0) return;
+    const int lrp = 32 - __clz(rvg - 1), rp = 1 << lrp;         // rvg = 1: __clz(0) = 32, rp = 1
+    const int t = threadIdx.x, row = r0 + (t & (rp - 1)), slot_c = t >> lrp, n_slot = kPrepThreads >> lrp;
     const int w = tile * TC_M + row;
-    const bool wvalid = row < rv;
+    const bool wvalid = row < r0 + rvg;
     const int mw = a.mw;
     const uint32_t pbytes = (uint32_t)a.prows * (SK * 2);        // bytes of a staged plane
     const size_t stage_bytes = (size_t)a.planes_per_stage * pbytes;
@@ -224,9 +229,11 @@ __global__ void __launch_bounds__(kPrepThreads, kC1Only ? 3 : 2) k_c15_prep(C15T
     const int nks = (K + TC_K - 1) / TC_K;
     for (int q = K + t; q < nks * TC_K; q += kPrepThreads) ao_s[q] = -1;
     __syncthreads();
-    int *lst = a.ao_list + slot * (size_t)a.kmax_steps * TC_K;
-    for (int q = t; q < nks * TC_K; q += kPrepThreads) lst[q] = ao_s[q];
-    if (t == 0) a.nks[slot] = nks;
+    if (blockIdx.z == 0) {
+        int *lst = a.ao_list + slot * (size_t)a.kmax_steps * TC_K;
+        for (int q = t; q < nks * TC_K; q += kPrepThreads) lst[q] = ao_s[q];
+        if (t == 0) a.nks[slot] = nks;
+    }
 
     const double *rw = a.R + ((size_t)(wvalid ? w : 0) * s.n_elec + e) * 3;
     const float2 r2[3] = {ff::from_double(rw[0]), ff::from_double(rw[1]), ff::from_double(rw[2])};
@@ -769,11 +776,19 @@ cudaError_t launch_c15_tc(const SysDev &s, const FfBasis &fb, const MixedTables 
         cudaSuccess)
         return e;
     const int mtiles = (nmax + TC_N - 1) / TC_N;
+    // row groups of the producer: down to 32 rows (a warp's lanes) while a launch has fewer than
+    // three CTAs for each of 152 SMs (158 electrons x 100 walkers, 158 pairs: 307 -> 166 us;
+    // Slater matrices of 434 electrons x 129: 2.76 -> 1.39 ms)
+    const int rows = std::min(nw, (int)TC_M);
+    a.group = TC_M;
+    while (a.group > 32 && std::min(nb, (size_t)s.n_elec) * a.n_tiles * ((rows + a.group - 1) / a.group) < 152 * 3)
+        a.group /= 2;
+    const int rg = (rows + a.group - 1) / a.group;
     for (int e0 = 0; e0 < s.n_elec; e0 += (int)nb) {
         const int ne = s.n_elec - e0 < (int)nb ? s.n_elec - e0 : (int)nb;
         a.e0 = e0;
-        if (c1_only) k_c15_prep<true><<<dim3(a.n_tiles, ne), kPrepThreads, sm_prep, st>>>(a);
-        else k_c15_prep<false><<<dim3(a.n_tiles, ne), kPrepThreads, sm_prep, st>>>(a);
+        if (c1_only) k_c15_prep<true><<<dim3(a.n_tiles, ne, rg), kPrepThreads, sm_prep, st>>>(a);
+        else k_c15_prep<false><<<dim3(a.n_tiles, ne, rg), kPrepThreads, sm_prep, st>>>(a);
         k_c15_mma<<<dim3(mtiles, a.n_tiles, (c1_only ? 1 : 3) * ne), kMmaThreads, sm_mma, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
