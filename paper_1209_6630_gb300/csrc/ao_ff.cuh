@@ -43,16 +43,46 @@ __device__ __forceinline__ void ff_radial(const SysDev &s, const FfBasis &fb, in
         const float2 gam = fb.pg[p0 + p];
         const float2 x = ff::mul(gam, d2);
         const float2 ce = ff::mul(fb.pc[p0 + p], ff::exp_neg(x, fb.expj));
-        g = ff::add(g, ce);
         const float2 gce = ff::mul(gam, ce);
-        gd = ff::add(gd, gce);
         const float2 t = ff::add(make_float2(4.f * x.x, 4.f * x.y), make_float2(-6.f, 0.f));
+        if (p == 0) {                                      // 0 + ce and so on leave the pair as it is
+            g = ce;
+            gd = gce;
+            gl = ff::mul(t, gce);
+            continue;
+        }
+        g = ff::add(g, ce);
+        gd = ff::add(gd, gce);
         gl = ff::fma2(gl, t, gce);
     }
     o.g = g;
     o.gd = gd;
     o.gl = gl;
 }
+
+// The axes of a monomial of degree 1 (b = -1) or 2 (a <= b).  Degrees 0, 1 and 2 -- all but a few
+// shells in practice -- are written out below: the general expressions multiply by exact ones and
+// add exact zeros there, which leaves a float pair unchanged, so the values are the same bit for
+// bit at about half the instructions (every lane of a warp is at the same AO).
+__device__ __forceinline__ void ao_axes(int pw, int &a, int &b)
+{
+    const int nx = pw & 255, ny = (pw >> 8) & 255, nz = (pw >> 16) & 255;
+    a = nx ? 0 : (ny ? 1 : 2);
+    b = nx + ny + nz < 2 ? -1 : (nz ? 2 : (ny ? 1 : 0));
+}
+
+template <typename T>
+__device__ __forceinline__ T pick3(int i, T x, T y, T z)
+{
+    return i == 0 ? x : (i == 1 ? y : z);
+}
+
+__device__ __forceinline__ float2 pick3(int i, float2 x, float2 y, float2 z)
+{
+    return make_float2(pick3(i, x.x, y.x, z.x), pick3(i, x.y, y.y, z.y));
+}
+
+__device__ __forceinline__ int ao_degree(int pw) { return (pw & 255) + ((pw >> 8) & 255) + ((pw >> 16) & 255); }
 
 __device__ __forceinline__ void ff_angular(const SysDev &s, const FfBasis &fb, int mu, const FfRadial &rd,
                                            float2 &val, float2 &lap)
@@ -64,6 +94,16 @@ __device__ __forceinline__ void ff_angular(const SysDev &s, const FfBasis &fb, i
     if (L == 0) {
         val = ff::mul(c, rd.g);
         lap = ff::mul(c, rd.gl);
+        return;
+    }
+    if (L <= 2) {
+        int xa, xb;
+        ao_axes(pw, xa, xb);
+        const float2 da = pick3(xa, rd.dx, rd.dy, rd.dz);
+        const float2 P = L == 1 ? da : ff::mul(da, pick3(xb, rd.dx, rd.dy, rd.dz));
+        val = ff::mul(c, ff::mul(P, rd.g));
+        const float2 q = ff::sub(rd.gl, ff::mulf(rd.gd, (float)(4 * L)));
+        lap = ff::mul(c, xa == xb ? ff::fma2(make_float2(2.f * rd.g.x, 2.f * rd.g.y), P, q) : ff::mul(P, q));
         return;
     }
     const float2 px = ff_ipow(rd.dx, nx), py = ff_ipow(rd.dy, ny), pz = ff_ipow(rd.dz, nz);
@@ -101,16 +141,28 @@ __device__ __forceinline__ void ff_radial_val(const SysDev &s, const FfBasis &fb
     const int p0 = s.sh_pstart[sh], np = s.sh_nprim[sh];
 #pragma unroll 1
     for (int p = 0; p < np; ++p)
-        g = ff::add(g, ff::mul(fb.pc[p0 + p], ff::exp_neg(ff::mul(fb.pg[p0 + p], d2), fb.expj)));
+    {
+        const float2 ce = ff::mul(fb.pc[p0 + p], ff::exp_neg(ff::mul(fb.pg[p0 + p], d2), fb.expj));
+        g = p == 0 ? ce : ff::add(g, ce);
+    }
     o.g = g;
 }
 
 __device__ __forceinline__ float2 ff_angular_val(const SysDev &s, const FfBasis &fb, int mu, const FfRadial &rd)
 {
-    const int pw = s.ao_pow[mu];
+    const int pw = s.ao_pow[mu], L = ao_degree(pw);
+    const float2 c = fb.sc[mu];
+    if (L == 0) return ff::mul(c, rd.g);
+    if (L <= 2) {
+        int xa, xb;
+        ao_axes(pw, xa, xb);
+        float2 P = pick3(xa, rd.dx, rd.dy, rd.dz);
+        if (L == 2) P = ff::mul(P, pick3(xb, rd.dx, rd.dy, rd.dz));
+        return ff::mul(c, ff::mul(P, rd.g));
+    }
     const int nx = pw & 255, ny = (pw >> 8) & 255, nz = (pw >> 16) & 255;
     const float2 P = ff::mul(ff_ipow(rd.dx, nx), ff::mul(ff_ipow(rd.dy, ny), ff_ipow(rd.dz, nz)));
-    return ff::mul(fb.sc[mu], ff::mul(P, rd.g));
+    return ff::mul(c, ff::mul(P, rd.g));
 }
 
 // Ordered list of the AOs of the shells set in `bits` for a block of any

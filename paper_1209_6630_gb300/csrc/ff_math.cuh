@@ -50,6 +50,15 @@ __device__ __forceinline__ float2 add(float2 a, float2 b)
     return renorm(s, e);
 }
 
+// a + b where |a.x| >= |b.x| (or a.x = 0): the same value in three operations fewer
+__device__ __forceinline__ float2 add_ordered(float2 a, float2 b)
+{
+    float s, e;
+    fast_two_sum(a.x, b.x, s, e);
+    e = __fadd_rn(e, __fadd_rn(a.y, b.y));
+    return renorm(s, e);
+}
+
 __device__ __forceinline__ float2 neg(float2 x) { return make_float2(-x.x, -x.y); }
 __device__ __forceinline__ float2 sub(float2 a, float2 b) { return add(a, neg(b)); }
 
@@ -126,9 +135,9 @@ __device__ __forceinline__ float2 exp_neg(float2 x, const float2 *__restrict__ T
     const float s = sh;
     const float tail = s * s * s * (-1.0f / 6.0f + s * (1.0f / 24.0f + s * (-1.0f / 120.0f + s * (1.0f / 720.0f))));
     const float2 s2 = mul(sv, sv);
-    float2 p = add(make_float2(1.0f, 0.f), neg(sv));
-    p = add(p, make_float2(0.5f * s2.x, 0.5f * s2.y));
-    p = add(p, make_float2(tail, 0.f));
+    float2 p = add_ordered(make_float2(1.0f, 0.f), neg(sv));      // |s| <= 1/64
+    p = add_ordered(p, make_float2(0.5f * s2.x, 0.5f * s2.y));
+    p = add_ordered(p, make_float2(tail, 0.f));
     const float2 e = mul(p, T[(int)jf + 12]);
     const float scale = __int_as_float((127 - (int)kf) << 23);   // 2^-k, k in [0, 126]: a normal float
     return make_float2(__fmul_rn(e.x, scale), __fmul_rn(e.y, scale));

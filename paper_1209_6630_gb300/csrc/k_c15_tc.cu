@@ -456,7 +456,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) k_c15_mma(C15TcArgs a)
         const size_t stage_bytes = (size_t)a.planes_per_stage * pbytes;
         const unsigned char *Ag = a.planes + slot * (size_t)a.kmax_steps * 2 * stage_bytes +
                                   (size_t)o * kC15Slices * pbytes;           // o = 2: the gradient planes
-        const int nbplanes = grad ? 2 : kC15Slices;
         const uint16_t *__restrict__ Bsl = a.slice[spin];
         const size_t slice_stride = (size_t)s.n_ao * nspad;
         for (int sg = 0; sg < nst; ++sg) {
@@ -472,15 +471,24 @@ __global__ void __launch_bounds__(kMmaThreads, 1) k_c15_mma(C15TcArgs a)
                         bulk_g2s(smem_u32(Ab + j * kSPlaneBytes), Ag + (size_t)sg * stage_bytes + (size_t)j * pbytes,
                                  pbytes, FULL(buf));
             }
-            for (int q = cl; q < nbplanes * SK * (TC_N / 8); q += 32 * kMmaCpWarps) {
-                const int j = q / (SK * (TC_N / 8));
-                const int rem = q - j * (SK * (TC_N / 8));
-                const int r = rem / (TC_N / 8), c = rem - r * (TC_N / 8);
+            // rows cl / 16 + 8 i, chunk cl % 16 of each plane
+            constexpr int kRowStep = 32 * kMmaCpWarps / (TC_N / 8);
+            const int c = cl % (TC_N / 8);
+#pragma unroll
+            for (int i = 0; i < SK / kRowStep; ++i) {
+                const int r = cl / (TC_N / 8) + i * kRowStep;
                 const int mu = ao_s[sg * SK + r];
                 const bool v = mu >= 0 && 8 * c < ncols;
-                const uint16_t *bsrc = grad ? (j ? a.tt.lo[spin] : a.tt.hi[spin]) : Bsl + j * slice_stride;
-                const uint16_t *src = bsrc + (size_t)(v ? mu : 0) * nspad + k0 + (v ? 8 * c : 0);
-                cp_async16(smem_u32(Bb + j * kSBPlaneBytes + b_off(r, 8 * c)), src, v);
+                const size_t off = (size_t)(v ? mu : 0) * nspad + k0 + (v ? 8 * c : 0);
+                const uint32_t dst = smem_u32(Bb + b_off(r, 8 * c));
+                if (grad) {
+                    cp_async16(dst, a.tt.hi[spin] + off, v);
+                    cp_async16(dst + kSBPlaneBytes, a.tt.lo[spin] + off, v);
+                } else {
+                    const uint16_t *src = Bsl + off;
+#pragma unroll
+                    for (int j = 0; j < kC15Slices; ++j) cp_async16(dst + j * kSBPlaneBytes, src + j * slice_stride, v);
+                }
             }
             asm volatile("cp.async.wait_all;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

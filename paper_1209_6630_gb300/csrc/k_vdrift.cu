@@ -46,6 +46,7 @@ constexpr uint32_t kVdPlane = TC_M * kVdK * 2;                // A: [128 rows][3
 constexpr uint32_t kVdBPlane = kVdN * kVdK * 2;               // B: [64 rows][32 K]: 4 KB
 constexpr uint32_t kVdBuf = kC15Slices * (kVdPlane + kVdBPlane);   // 6 A planes + 6 B planes: 72 KB
 constexpr int kVdAcc = 4;
+static_assert(kVdThreads == kVdN * 4, "one 16-byte chunk of a B plane per thread");
 
 struct VdArgs {
     SysDev s;
@@ -108,6 +109,62 @@ __device__ __forceinline__ void vd_sums(uint32_t tmem_lanes, int c0, float2 *out
         ff::two_sum(s2, __uint_as_float(v3[q]), s, e2);
         out[q * ld] = ff::renorm(s, __fadd_rn(e, e2));
     }
+}
+
+// Laplacian (float-float) and gradient (FP32) of one AO from its shell's radial part; the degrees
+// 0, 1 and 2 written out (ao_ff.cuh), the same values as the general expressions below.
+__device__ __forceinline__ void vd_derivs(const SysDev &s, const VdArgs &a, int mu, const FfRadial &rd, float2 &lp,
+                                          float &g1, float &g2, float &g3)
+{
+    const int pw2 = s.ao_pow[mu], L = ao_degree(pw2);
+    const float dx = rd.dx.x + rd.dx.y, dy = rd.dy.x + rd.dy.y, dz = rd.dz.x + rd.dz.y;
+    const float g = rd.g.x + rd.g.y, m2gd = -2.f * (rd.gd.x + rd.gd.y);
+    const float c = a.scf[mu];
+    if (L <= 2) {
+        const float2 cf = a.fb.sc[mu];
+        if (L == 0) {
+            lp = ff::mul(cf, rd.gl);
+            g1 = c * (m2gd * dx);
+            g2 = c * (m2gd * dy);
+            g3 = c * (m2gd * dz);
+            return;
+        }
+        int xa, xb;
+        ao_axes(pw2, xa, xb);
+        const float2 fa = pick3(xa, rd.dx, rd.dy, rd.dz);
+        const float2 q = ff::sub(rd.gl, ff::mulf(rd.gd, (float)(4 * L)));
+        const float da = pick3(xa, dx, dy, dz);
+        float P = da, xA = 1.f, xB = 0.f;                  // d P / d axis a, d P / d axis b
+        float2 fP = fa;
+        if (L == 2) {
+            const float db = pick3(xb, dx, dy, dz);
+            P = da * db;
+            xA = xa == xb ? 2.f * da : db;
+            xB = da;
+            fP = ff::mul(fa, pick3(xb, rd.dx, rd.dy, rd.dz));
+        }
+        lp = ff::mul(cf, xa == xb ? ff::fma2(make_float2(2.f * rd.g.x, 2.f * rd.g.y), fP, q) : ff::mul(fP, q));
+        const float X0 = xa == 0 ? xA : 0.f;               // (axis b is never 0 unless a is)
+        const float X1 = xa == 1 ? xA : (xb == 1 ? xB : 0.f);
+        const float X2 = xa == 2 ? xA : (xb == 2 ? xB : 0.f);
+        g1 = c * fmaf(__fmul_rn(m2gd, dx), P, __fmul_rn(X0, g));
+        g2 = c * fmaf(__fmul_rn(m2gd, dy), P, __fmul_rn(X1, g));
+        g3 = c * fmaf(__fmul_rn(m2gd, dz), P, __fmul_rn(X2, g));
+        return;
+    }
+    float2 val;
+    ff_angular(s, a.fb, mu, rd, val, lp);
+    const int nx = pw2 & 255, ny = (pw2 >> 8) & 255, nz = (pw2 >> 16) & 255;
+    auto ip = [](float x, int n) {
+        float y = 1.f;
+        for (int i = 0; i < n; ++i) y *= x;
+        return y;
+    };
+    const float px = ip(dx, nx), py = ip(dy, ny), pz = ip(dz, nz);
+    const float P = px * py * pz;
+    g1 = c * ((nx ? nx * ip(dx, nx - 1) : 0.f) * py * pz * g + m2gd * dx * P);
+    g2 = c * (px * (ny ? ny * ip(dy, ny - 1) : 0.f) * pz * g + m2gd * dy * P);
+    g3 = c * (px * py * (nz ? nz * ip(dz, nz - 1) : 0.f) * g + m2gd * dz * P);
 }
 
 // Two CTAs per SM (256 threads, N = 64 AOs per tile, one operand stage of
@@ -229,6 +286,10 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
     unsigned char *Ab = base;
     unsigned char *Bb = base + kC15Slices * kVdPlane;
     for (int at = 0; at < nat && ok; ++at) {
+        // this thread's chunk of a B row in every slice plane and stage of the tile
+        const int bmu = ao_s[at * kVdN + (t >> 2)];
+        const uint16_t *bsrc = Bsl + (size_t)max(bmu, 0) * nspad + 8 * (t & 3);
+        const uint32_t bdst = smem_u32(Bb + a_off64(t >> 2, t & 3));
         for (int sg = 0; sg < nst; ++sg) {
             // the stage buffer: A (the staged D^-1 slices) and B (the rows of A of this AO tile)
             const int k0 = sg * kVdK;
@@ -240,14 +301,9 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
                     for (int j = 0; j < kC15Slices; ++j)
                         bulk_g2s(smem_u32(Ab + j * kVdPlane), As + (size_t)j * pbytes, pbytes, cb);
             }
-            for (int q = t; q < kC15Slices * kVdN * 4; q += kVdThreads) {
-                const int j = q / (kVdN * 4), rem = q - j * (kVdN * 4);
-                const int r = rem >> 2, c = rem & 3;
-                const int mu = ao_s[at * kVdN + r];
-                const bool v = mu >= 0;
-                const uint16_t *src = Bsl + j * bstride + (size_t)(v ? mu : 0) * nspad + k0 + 8 * c;
-                cp_async16(smem_u32(Bb + j * kVdBPlane + a_off64(r, c)), src, v);
-            }
+#pragma unroll
+            for (int j = 0; j < kC15Slices; ++j)
+                cp_async16(bdst + j * kVdBPlane, bsrc + j * bstride + k0, bmu >= 0);
             asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 0;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -289,6 +345,7 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
         // epilogue: v for 32 AOs of this walker row, then the AO derivatives at r_e
         FfRadial rd;
         int last_sh = -1;
+        bool on = false;                                   // last_sh is active for this walker
         // the stage buffer is idle here: [16][256] of the threads' own columns, or [64][64 rows]
         float2 *vbuf = reinterpret_cast<float2 *>(base);
         const int vld = small ? TC_M / 2 : kVdThreads;
@@ -311,33 +368,21 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
                 const int mu = ao_s[at * kVdN + c0 + q];
                 if (mu < 0) break;
                 const int sh = s.ao_shell[mu];
-                if (!((my_mask[sh >> 5] >> (sh & 31)) & 1u)) continue;
+                if (sh != last_sh) {
+                    last_sh = sh;
+                    on = (my_mask[sh >> 5] >> (sh & 31)) & 1u;
+                    if (on) ff_radial(s, a.fb, sh, r2, rd);
+                }
+                if (!on) continue;
                 const int ex = Ee + a.gexp[spin][mu];
                 const float2 vr = vcol[q * vld];
                 const float2 vmu = make_float2(scale_pow2(vr.x, ex), scale_pow2(vr.y, ex));   // exact scaling
-                if (sh != last_sh) {
-                    last_sh = sh;
-                    ff_radial(s, a.fb, sh, r2, rd);
-                }
                 // Laplacian in float-float (the kinetic term cancels against the potential: an FP32
                 // Laplacian left E_L at 2e-5 relative on 2048 walkers of 1056 electrons), the
-                // gradient in FP32 from the same radial part; products with v and sums in FP64
-                float2 val, lp;
-                ff_angular(s, a.fb, mu, rd, val, lp);
-                const int pw2 = s.ao_pow[mu];
-                const int nx = pw2 & 255, ny = (pw2 >> 8) & 255, nz = (pw2 >> 16) & 255;
-                const float dx = rd.dx.x + rd.dx.y, dy = rd.dy.x + rd.dy.y, dz = rd.dz.x + rd.dz.y;
-                auto ip = [](float x, int n) {
-                    float y = 1.f;
-                    for (int i = 0; i < n; ++i) y *= x;
-                    return y;
-                };
-                const float px = ip(dx, nx), py = ip(dy, ny), pz = ip(dz, nz);
-                const float P = px * py * pz, g = rd.g.x + rd.g.y, m2gd = -2.f * (rd.gd.x + rd.gd.y);
-                const float c = a.scf[mu];
-                const float g1 = c * ((nx ? nx * ip(dx, nx - 1) : 0.f) * py * pz * g + m2gd * dx * P);
-                const float g2 = c * (px * (ny ? ny * ip(dy, ny - 1) : 0.f) * pz * g + m2gd * dy * P);
-                const float g3 = c * (px * py * (nz ? nz * ip(dz, nz - 1) : 0.f) * g + m2gd * dz * P);
+                // gradient in FP32 from the same radial part; products with v as float pairs
+                float2 lp;
+                float g1, g2, g3;
+                vd_derivs(s, a, mu, rd, lp, g1, g2, g3);
                 b0 = ff::fma2(b0, vmu, make_float2(g1, 0.f));
                 b1 = ff::fma2(b1, vmu, make_float2(g2, 0.f));
                 b2 = ff::fma2(b2, vmu, make_float2(g3, 0.f));

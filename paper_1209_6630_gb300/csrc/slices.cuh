@@ -17,24 +17,10 @@ __device__ __forceinline__ int exp_bound(float x)   // 2^E > 1.001 x (x >= 0)
     return ((__float_as_int(y) >> 23) & 0xff) - 126;
 }
 
-// Slices of the float pair x with |x| < 2^E: s_j = rint(r 2^(7(j+1))) 2^(-7(j+1)),
-// r the remainder, computed exactly in float pairs.
-__device__ __forceinline__ void slice6(float2 x, int E, float (&s)[kC15Slices])
-{
-    E = min(max(E, -125), 126);
-    const float sc = __int_as_float((127 - E) << 23);
-    float2 r = make_float2(x.x * sc, x.y * sc);
-#pragma unroll
-    for (int j = 0; j < kC15Slices; ++j) {
-        const int sh = kC15SliceBits * (j + 1);
-        const float q = rintf(r.x * __int_as_float((127 + sh) << 23));
-        const float sj = q * __int_as_float((127 - sh) << 23);
-        s[j] = sj;
-        r = ff::sub(r, make_float2(sj, 0.f));
-    }
-}
-
-// The same with S slices (S = 7: 49 bits, the Gauss-Jordan updates).
+// S slices of the float pair x with |x| < 2^E: s_j = rint(r 2^(7(j+1))) 2^(-7(j+1)),
+// r the remainder, exactly in float pairs: s_j is r.x rounded to its unit, so r.x - s_j is exact
+// in FP32 and the remainder is that plus r.y, renormalised (S = 6: 42 bits, the products; S = 7:
+// 49 bits, the Gauss-Jordan updates).
 template <int S>
 __device__ __forceinline__ void slice_n(float2 x, int E, float (&s)[S])
 {
@@ -47,9 +33,11 @@ __device__ __forceinline__ void slice_n(float2 x, int E, float (&s)[S])
         const float q = rintf(r.x * __int_as_float((127 + sh) << 23));
         const float sj = q * __int_as_float((127 - sh) << 23);
         s[j] = sj;
-        r = ff::sub(r, make_float2(sj, 0.f));
+        r = ff::renorm(__fsub_rn(r.x, sj), r.y);
     }
 }
+
+__device__ __forceinline__ void slice6(float2 x, int E, float (&s)[kC15Slices]) { slice_n<kC15Slices>(x, E, s); }
 
 // x * 2^e exactly (barring underflow or overflow of the result) for |e| <= 250,
 // as two multiplications by powers of two that are normal FP32 numbers
