@@ -24,6 +24,7 @@
 // (three CTAs per SM); NB = 8 halves it at the cost of twice the panel sweeps.
 #include <math.h>
 
+#include "f64_bits.cuh"
 #include "ff_math.cuh"
 #include "gj_panel.cuh"
 #include "qmc_internal.cuh"
@@ -44,20 +45,17 @@ __host__ __device__ __forceinline__ size_t p_region(int n, int nb)
     return a > 32 * 33 ? a : 32 * 33;
 }
 
-__device__ __forceinline__ void argmax_merge_f(float &v, int &i, float v2, int i2)
+// bytes of the float-float panel as row pairs (at the end two 32 x 33 transpose tiles lie there)
+__host__ __device__ __forceinline__ size_t gjff_p_bytes(int n, int nb)
 {
-    if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
+    const size_t a = (size_t)((n + 1) / 2) * nb * 16;
+    return a > 2 * 32 * 33 * 8 ? a : 2 * 32 * 33 * 8;
 }
 
-__device__ __forceinline__ void block_argmax_f(float &bv, int &bi, float *red_v, int *red_i, int lane, int wid)
+// ... with the pivot rows' tile [NB][32], the pivot map and the panel's row flags
+__host__ __device__ __forceinline__ size_t gjff_fixed_bytes(int n, int nb)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float v2 = __shfl_down_sync(0xffffffffu, bv, o);
-        const int i2 = __shfl_down_sync(0xffffffffu, bi, o);
-        argmax_merge_f(bv, bi, v2, i2);
-    }
-    if (lane == 0) { red_v[wid] = bv; red_i[wid] = bi; }
+    return (gjff_p_bytes(n, nb) + sizeof(float2) * nb * 32 + sizeof(short) * (2 * (size_t)n + 2) + 15) / 16 * 16;
 }
 
 template <int NB>
@@ -278,84 +276,160 @@ cudaError_t launch_gj(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb)
 // recomputes the flagged matrices with the FP64 k_gj, which skips the others.
 // (float-float helpers: ff_math.cuh)
 
-template <int NB>
-__global__ void __launch_bounds__(kGjThreads, NB == 8 ? 4 : (NB == 16 ? 3 : 1)) k_gj_ff(GjJobs2 jobs, double kappa_max)
+// The panel holds one row per thread in registers (two where n > 512): a column step is
+// two barriers, an integer REDUX search for the pivot, the pivot row scaled by its owner's warp,
+// and NB float-float multiply-adds per row into registers rotated by one, so that the step's
+// column is always the first and the loop needs no unrolling.  The trailing update pairs two rows
+// (packed FP32 instructions: two results per issue slot, the same roundings), the eliminated
+// panel lying in shared memory as row pairs {h, h', l, l'}.  Bound by the FP32 pipe: n^3 multiply-adds
+// of 12 operations.  Measured (16 lanes per row of the panel and scalar updates before): 8192
+// matrices of 217 rows 63.4 -> 52.1 ms, 200 of 79 rows 285 -> 223 us, 2 of 79 rows 232 -> 152 us.
+
+// |x| as an integer that orders like it; 0 for NaN (never a pivot) and 0
+__device__ __forceinline__ unsigned gjff_key(float x)
 {
+    const unsigned b = __float_as_uint(x) & 0x7fffffffu;
+    return b > 0x7f800000u ? 0u : b;
+}
+
+// The largest key of a warp and the smallest index that has it, in every lane.
+__device__ __forceinline__ void gjff_warp_max(unsigned &k, int &i)
+{
+    const unsigned m = __reduce_max_sync(0xffffffffu, k);
+    i = (int)__reduce_min_sync(0xffffffffu, k == m ? (unsigned)i : 0x7fffffffu);
+    k = m;
+}
+
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// (xh, xl) += (ph, pl) (uh, ul) for two rows: the product's error by FMA, TwoSum into the high
+// parts, the low parts plain
+__device__ __forceinline__ void gjff_step2(float2 &xh, float2 &xl, float2 ph, float2 pl, float2 uh, float2 ul)
+{
+    const float2 p = __fmul2_rn(ph, uh);
+    float2 pe = __ffma2_rn(ph, uh, neg2(p));
+    pe = __ffma2_rn(ph, ul, pe);
+    pe = __ffma2_rn(pl, uh, pe);
+    const float2 s = __fadd2_rn(xh, p), bb = __fadd2_rn(s, neg2(xh));
+    const float2 e = __fadd2_rn(__fadd2_rn(xh, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(p, neg2(bb)));
+    xh = s;
+    xl = __fadd2_rn(xl, __fadd2_rn(pe, e));
+}
+
+// MIN: CTAs per SM that the registers leave room for; kSmem: the work matrix lies in shared memory.
+template <int NB, int THREADS, int RPT, int MIN, bool kSmem>
+__global__ void __launch_bounds__(THREADS, MIN) k_gj_ff(GjJobs2 jobs, double kappa_max)
+{
+    constexpr int WARPS = THREADS / 32;
     const GjJob &J = jobs.j[blockIdx.y];
     const int m = blockIdx.x;
     if (m >= J.count) return;
     const int n = J.n;
     const double *__restrict__ X = J.X + (size_t)m * J.x_stride;
-    float2 *__restrict__ Wk = J.work + (size_t)m * J.x_stride;
     double *__restrict__ Dout = J.Dinv + (size_t)m * J.d_stride;
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *P = reinterpret_cast<float2 *>(smem_raw);   // [n][NB], later a [32][33] tile
-    float2 *U = P + p_region(n, NB);                      // [NB][32]
-    short *used = reinterpret_cast<short *>(U + NB * 32);
-    short *pp = used + n;
-    short *rowc = pp + n;
-    __shared__ int red_i[kGjWarps];
-    __shared__ float red_f[kGjWarps];
+    float2 *Wk;                                               // the float-pair work matrix, row stride ld
+    const int ld = kSmem ? n | 1 : n;                         // (odd: a thread per row meets all banks)
+    if constexpr (kSmem) Wk = reinterpret_cast<float2 *>(smem_raw + gjff_fixed_bytes(n, NB));
+    else Wk = J.work + (size_t)m * J.x_stride;
+    const int np = (n + 1) >> 1;                              // row pairs
+    float4 *P = reinterpret_cast<float4 *>(smem_raw);         // [np][NB]
+    float2 *U = reinterpret_cast<float2 *>(smem_raw + gjff_p_bytes(n, NB));   // [NB][32]
+    short *pp = reinterpret_cast<short *>(U + NB * 32);
+    short *rowc = pp + n;                                     // [2 np] 1 where the row is a pivot of the panel
+    __shared__ unsigned red_k[WARPS];
+    __shared__ int red_i[WARPS];
+    __shared__ float red_f[WARPS];
+    __shared__ float2 raw_s[NB], prow_s[NB];
     __shared__ float s_xnorm;
 
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     // float-pair copy of X and ||X||_inf (max row sum of |x|, one warp per row)
     float rmax = 0.f;
-    for (int i = wid; i < n; i += kGjWarps) {
+    for (int i = wid; i < n; i += WARPS) {
         float rs = 0.f;
+#pragma unroll 4
         for (int c = lane; c < n; c += 32) {
-            const double x = X[(size_t)i * n + c];
-            const float h = (float)x;
-            Wk[(size_t)i * n + c] = make_float2(h, (float)(x - (double)h));
-            rs += fabsf(h);
+            const float2 v = split_f64(X[(size_t)i * n + c]);
+            Wk[(size_t)i * ld + c] = v;
+            rs += fabsf(v.x);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
         rmax = fmaxf(rmax, rs);
     }
     if (lane == 0) red_f[wid] = rmax;
-    for (int i = t; i < n; i += kGjThreads) { used[i] = 0; rowc[i] = -1; }
+    for (int i = t; i < 2 * np; i += THREADS) rowc[i] = 0;
     __syncthreads();
     if (t == 0) {
         float xm = 0.f;
-        for (int q = 0; q < kGjWarps; ++q) xm = fmaxf(xm, red_f[q]);
+        for (int q = 0; q < WARPS; ++q) xm = fmaxf(xm, red_f[q]);
         s_xnorm = xm;
     }
-    // |det| = (mag_h + mag_l) 2^mag_e, kept by every thread (the pivots are
-    // the same in all threads); the sign from the parity of negative pivots
+    // |det| = (mag_h + mag_l) 2^mag_e, kept by the last warp (the one with the fewest rows); the sign
+    // from the parity of negative pivots
     float mag_h = 1.f, mag_l = 0.f;
     int mag_e = 0, neg = 0;
     bool sing = false;
+    bool used[RPT];                                           // this thread's rows t + THREADS r
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) used[r] = t + THREADS * r >= n;
     __syncthreads();
 
     for (int jb = 0; jb < n; jb += NB) {
         const int w = min(NB, n - jb);
-        for (int q = t; q < n * NB; q += kGjThreads) {
-            const int i = q / NB, c = q - i * NB;
-            P[q] = (c < w) ? Wk[(size_t)i * n + jb + c] : make_float2(0.f, 0.f);
+        float2 x[RPT][NB];
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            const int i = t + THREADS * r;
+            const float2 *src = Wk + (size_t)min(i, n - 1) * ld + jb;
+#pragma unroll
+            for (int q = 0; q < NB; ++q) x[r][q] = (i < n && q < w) ? src[q] : make_float2(0.f, 0.f);
+        }
+        {
+            unsigned k = 0;
+            int bi = n;
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                const unsigned kr = used[r] ? 0u : gjff_key(x[r][0].x);
+                if (kr > k) { k = kr; bi = t + THREADS * r; }
+            }
+            gjff_warp_max(k, bi);
+            if (lane == 0) { red_k[wid] = k; red_i[wid] = bi; }
         }
         __syncthreads();
-        float bv = -1.f;
-        int bi = n;
-        for (int i = t; i < n; i += kGjThreads)
-            if (!used[i]) argmax_merge_f(bv, bi, fabsf(P[i * NB].x), i);
-        block_argmax_f(bv, bi, red_f, red_i, lane, wid);
-        __syncthreads();
-
-        // NB consecutive lanes share a row, one panel column each: the
-        // accesses of a warp are contiguous (no bank conflicts)
-        const int cc = t & (NB - 1);
-        for (int c = 0; c < w; ++c) {
-            // every thread merges the warps' candidates in the same order
-            float v = red_f[0];
-            int p = red_i[0];
-            for (int q = 1; q < kGjWarps; ++q) argmax_merge_f(v, p, red_f[q], red_i[q]);
-            if (!(v > 0.f)) { sing = true; break; }
-            const float2 piv = P[p * NB + c];
-            const float2 pinv = ff::inv(piv);
-            const float2 prow = (cc == c) ? pinv : ff::mul(P[p * NB + cc], pinv);
-            {
+        for (int c = 0; c < NB; ++c) {
+            if (c >= w) {                                     // a short last panel: back into column order
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) {
+                    const float2 x0 = x[r][0];
+#pragma unroll
+                    for (int q = 0; q + 1 < NB; ++q) x[r][q] = x[r][q + 1];
+                    x[r][NB - 1] = x0;
+                }
+                continue;
+            }
+            unsigned k = lane < WARPS ? red_k[lane] : 0u;
+            int p = lane < WARPS ? red_i[lane] : n;
+            gjff_warp_max(k, p);
+            if (k == 0u) { sing = true; break; }              // every warp sees the same candidates
+            if (wid == (p & (THREADS - 1)) >> 5) {
+                // the pivot row, from its owner through shared memory, scaled a column per lane
+#pragma unroll
+                for (int r = 0; r < RPT; ++r)
+                    if (t + THREADS * r == p) {
+#pragma unroll
+                        for (int q = 0; q < NB; ++q) raw_s[q] = x[r][q];
+                        used[r] = true;
+                    }
+                __syncwarp();
+                const float2 pinv = ff::inv(raw_s[0]);
+                if (lane < NB) prow_s[lane] = lane ? ff::mul(raw_s[lane], pinv) : pinv;
+            }
+            __syncthreads();
+            if (wid == WARPS - 1) {
+                const float2 piv = raw_s[0];
                 const float2 a = piv.x < 0.f ? ff::neg(piv) : piv;
                 const float2 mg = ff::mul(make_float2(mag_h, mag_l), a);
                 int ex;
@@ -364,127 +438,125 @@ __global__ void __launch_bounds__(kGjThreads, NB == 8 ? 4 : (NB == 16 ? 3 : 1)) 
                 mag_l = ldexpf(mg.y, -ex);
                 mag_e += ex;
                 neg ^= piv.x < 0.f;
-            }
-            if (t == 0) {
-                used[p] = 1;
-                pp[jb + c] = (short)p;
-                rowc[p] = (short)c;
-            }
-            __syncthreads();                               // the candidates and row p have been read
-            if (t < NB) P[p * NB + t] = prow;              // t < NB: column cc == t
-            float nbv = -1.f;
-            int nbi = n;
-            const int cn = c + 1;
-            for (int base = (t & ~31) / NB; base < n; base += kGjThreads / NB) {
-                const int i = base + lane / NB;
-                const bool live = i < n && i != p;
-                const float2 mf = live ? ff::neg(P[i * NB + c]) : make_float2(0.f, 0.f);
-                __syncwarp();                              // every lane has read P[i][c]
-                if (live) {
-                    const float2 x = (cc != c) ? ff::fma2(P[i * NB + cc], mf, prow) : ff::mul(mf, pinv);
-                    P[i * NB + cc] = x;
-                    if (cc == cn && cn < w && !used[i]) argmax_merge_f(nbv, nbi, fabsf(x.x), i);
+                if (lane == 0) {
+                    pp[jb + c] = (short)p;
+                    rowc[p] = 1;
                 }
             }
-            block_argmax_f(nbv, nbi, red_f, red_i, lane, wid);
+            const float2 pinv = prow_s[0];
+            k = 0;
+            int bi = n;
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                const int i = t + THREADS * r;
+                if (i - lane >= n) break;                     // a warp without rows
+                if (i == p) {
+#pragma unroll
+                    for (int q = 0; q + 1 < NB; ++q) x[r][q] = prow_s[q + 1];
+                    x[r][NB - 1] = pinv;
+                } else {
+                    const float2 mf = ff::neg(x[r][0]);
+#pragma unroll
+                    for (int q = 0; q + 1 < NB; ++q) x[r][q] = ff::fma2(x[r][q + 1], mf, prow_s[q + 1]);
+                    x[r][NB - 1] = ff::mul(mf, pinv);
+                }
+                const unsigned kr = (used[r] || c + 1 >= w) ? 0u : gjff_key(x[r][0].x);
+                if (kr > k) { k = kr; bi = i; }
+            }
+            gjff_warp_max(k, bi);
+            if (lane == 0) { red_k[wid] = k; red_i[wid] = bi; }
             __syncthreads();
         }
         if (sing) break;
 
-        for (int q = t; q < n * w; q += kGjThreads) {
-            const int i = q / w, c = q - i * w;
-            Wk[(size_t)i * n + jb + c] = P[i * NB + c];
+        // the eliminated panel: part of the result, and the update's operand as row pairs
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            const int i = t + THREADS * r;
+            float *dst = reinterpret_cast<float *>(P + (size_t)(i >> 1) * NB) + (i & 1);
+            if (i < n) {
+#pragma unroll
+                for (int q = 0; q < NB; ++q) {
+                    if (q < w) Wk[(size_t)i * ld + jb + q] = x[r][q];
+                    dst[4 * q] = x[r][q].x;
+                    dst[4 * q + 2] = x[r][q].y;
+                }
+            } else if (i < 2 * np) {
+#pragma unroll
+                for (int q = 0; q < NB; ++q) dst[4 * q] = dst[4 * q + 2] = 0.f;
+            }
         }
 
         int c0 = 0;
         auto skip = [&](int cc0) { return cc0 >= jb && cc0 + 32 <= jb + w; };
         while (c0 < n && skip(c0)) c0 += 32;
-        constexpr int UPT = NB * 32 / kGjThreads;
+        constexpr int UPT = NB * 32 / THREADS > 0 ? NB * 32 / THREADS : 1;
         float2 upre[UPT];
         __syncthreads();
+        auto load_u = [&](int cc0) {
 #pragma unroll
-        for (int r = 0; r < UPT; ++r) {
-            const int q = t + r * kGjThreads, c = q >> 5, col = c0 + (q & 31);
-            upre[r] = (c0 < n && c < w && col < n) ? Wk[(size_t)pp[jb + c] * n + col] : make_float2(0.f, 0.f);
-        }
+            for (int r = 0; r < UPT; ++r) {
+                const int q = t + r * THREADS, c = q >> 5, col = cc0 + (q & 31);
+                upre[r] = (cc0 < n && c < w && col < n) ? Wk[(size_t)pp[jb + c] * ld + col] : make_float2(0.f, 0.f);
+            }
+        };
+        load_u(c0);
         while (c0 < n) {
             __syncthreads();
 #pragma unroll
-            for (int r = 0; r < UPT; ++r) U[t + r * kGjThreads] = upre[r];
+            for (int r = 0; r < UPT; ++r)
+                if (t + r * THREADS < NB * 32) U[t + r * THREADS] = upre[r];
             __syncthreads();
             int c1 = c0 + 32;
             while (c1 < n && skip(c1)) c1 += 32;
-#pragma unroll
-            for (int r = 0; r < UPT; ++r) {
-                const int q = t + r * kGjThreads, c = q >> 5, col = c1 + (q & 31);
-                upre[r] = (c1 < n && c < w && col < n) ? Wk[(size_t)pp[jb + c] * n + col] : make_float2(0.f, 0.f);
-            }
+            load_u(c1);
             const int col = c0 + lane;
             const bool active = col < n && !(col >= jb && col < jb + w);
             float2 u[NB];
 #pragma unroll
             for (int c = 0; c < NB; ++c) u[c] = U[c * 32 + lane];
             if (active) {
-                // rows (i, i + 8) two iterations ahead are loaded while the
-                // current pair is updated
-                auto load_pair = [&](int i, float2 &a, float2 &b) {
-                    const int i2 = i + kGjWarps;
-                    a = (i < n && rowc[i] < 0) ? Wk[(size_t)i * n + col] : make_float2(0.f, 0.f);
-                    b = (i2 < n && rowc[i2] < 0) ? Wk[(size_t)i2 * n + col] : make_float2(0.f, 0.f);
+                auto load_pair = [&](int r, float2 &h, float2 &l) {      // rows 2 r, 2 r + 1 (0 for pivots)
+                    const int i = 2 * r;
+                    const float2 a = (r < np && !rowc[i]) ? Wk[(size_t)i * ld + col] : make_float2(0.f, 0.f);
+                    const float2 b = (i + 1 < n && !rowc[i + 1]) ? Wk[(size_t)(i + 1) * ld + col] : make_float2(0.f, 0.f);
+                    h = make_float2(a.x, b.x);
+                    l = make_float2(a.y, b.y);
                 };
-                float2 nx0, nx1, mx0, mx1;                 // two row pairs ahead
-                load_pair(wid, nx0, nx1);
-                load_pair(wid + 2 * kGjWarps, mx0, mx1);
-#pragma unroll 2
-                for (int i = wid; i < n; i += 2 * kGjWarps) {
-                    // two rows at a time; products of a row summed with TwoSum
-                    // into the hi part and plain FP32 into the lo part, one
-                    // renormalisation per row at the end
-                    const int i2 = i + kGjWarps;
-                    const bool has2 = i2 < n;
-                    float2 x0 = nx0, x1 = nx1;
-                    nx0 = mx0;
-                    nx1 = mx1;
-                    load_pair(i + 4 * kGjWarps, mx0, mx1);
-                    const float4 *pr0 = reinterpret_cast<const float4 *>(P + i * NB);
-                    const float4 *pr1 = reinterpret_cast<const float4 *>(P + (has2 ? i2 : i) * NB);
-#pragma unroll
-                    for (int c2 = 0; c2 < NB / 2; ++c2) {
-                        const float4 a0 = pr0[c2], a1 = pr1[c2];
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const float2 uv = u[2 * c2 + h];
-                            const float ph0 = h ? a0.z : a0.x, pl0 = h ? a0.w : a0.y;
-                            const float ph1 = h ? a1.z : a1.x, pl1 = h ? a1.w : a1.y;
-                            float p = __fmul_rn(ph0, uv.x), pe = fmaf(ph0, uv.x, -p);
-                            pe = fmaf(ph0, uv.y, pe);
-                            pe = fmaf(pl0, uv.x, pe);
-                            float s, e;
-                            ff::two_sum(x0.x, p, s, e);
-                            x0.x = s;
-                            x0.y = __fadd_rn(x0.y, __fadd_rn(pe, e));
-                            p = __fmul_rn(ph1, uv.x);
-                            pe = fmaf(ph1, uv.x, -p);
-                            pe = fmaf(ph1, uv.y, pe);
-                            pe = fmaf(pl1, uv.x, pe);
-                            ff::two_sum(x1.x, p, s, e);
-                            x1.x = s;
-                            x1.y = __fadd_rn(x1.y, __fadd_rn(pe, e));
-                        }
+                auto store_pair = [&](int r, float2 h, float2 l) {
+                    float sh, sl;
+                    ff::fast_two_sum(h.x, l.x, sh, sl);
+                    Wk[(size_t)(2 * r) * ld + col] = make_float2(sh, sl);
+                    if (2 * r + 1 < n) {
+                        ff::fast_two_sum(h.y, l.y, sh, sl);
+                        Wk[(size_t)(2 * r + 1) * ld + col] = make_float2(sh, sl);
                     }
-                    float h0, l0;
-                    ff::fast_two_sum(x0.x, x0.y, h0, l0);
-                    Wk[(size_t)i * n + col] = make_float2(h0, l0);
-                    if (has2) {
-                        ff::fast_two_sum(x1.x, x1.y, h0, l0);
-                        Wk[(size_t)i2 * n + col] = make_float2(h0, l0);
+                };
+                // two row pairs at a time, the next two loaded meanwhile
+                float2 nh0, nl0, nh1, nl1;
+                load_pair(wid, nh0, nl0);
+                load_pair(wid + WARPS, nh1, nl1);
+                for (int r = wid; r < np; r += 2 * WARPS) {
+                    const int r1 = r + WARPS;
+                    float2 xh0 = nh0, xl0 = nl0, xh1 = nh1, xl1 = nl1;
+                    load_pair(r + 2 * WARPS, nh0, nl0);
+                    load_pair(r1 + 2 * WARPS, nh1, nl1);
+                    const float4 *p0 = P + (size_t)r * NB, *p1 = P + (size_t)(r1 < np ? r1 : r) * NB;
+#pragma unroll
+                    for (int c = 0; c < NB; ++c) {
+                        const float4 a0 = p0[c], a1 = p1[c];
+                        const float2 uh = make_float2(u[c].x, u[c].x), ul = make_float2(u[c].y, u[c].y);
+                        gjff_step2(xh0, xl0, make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), uh, ul);
+                        gjff_step2(xh1, xl1, make_float2(a1.x, a1.y), make_float2(a1.z, a1.w), uh, ul);
                     }
+                    store_pair(r, xh0, xl0);
+                    if (r1 < np) store_pair(r1, xh1, xl1);
                 }
             }
             c0 = c1;
         }
         __syncthreads();
-        for (int c = t; c < w; c += kGjThreads) rowc[pp[jb + c]] = -1;
+        for (int c = t; c < w; c += THREADS) rowc[pp[jb + c]] = 0;
         __syncthreads();
     }
 
@@ -495,45 +567,56 @@ __global__ void __launch_bounds__(kGjThreads, NB == 8 ? 4 : (NB == 16 ? 3 : 1)) 
     }
     __syncthreads();
 
-    // ||X^-1||_inf: the rows of X^-1 are the rows of the result (columns permuted)
+    // ||X^-1||_inf (the rows of X^-1 are the rows of the result, columns permuted) and D^-1 = X^-T
+    // in one pass, 32 x 32 tiles alternating between two buffers: one barrier each
+    constexpr int RW = 32 / WARPS;
+    float2 *tile = reinterpret_cast<float2 *>(smem_raw);      // [2][32][33] (P and U are done with)
     float imax = 0.f;
-    for (int i = wid; i < n; i += kGjWarps) {
-        float rs = 0.f;
-        for (int c = lane; c < n; c += 32) rs += fabsf(Wk[(size_t)i * n + c].x);
+    int buf = 0;
+    for (int kb = 0; kb < n; kb += 32) {
+        float rs[RW];
+        const float2 *row[RW];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
-        imax = fmaxf(imax, rs);
+        for (int r = 0; r < RW; ++r) {
+            const int k = kb + wid + r * WARPS;
+            rs[r] = 0.f;
+            row[r] = k < n ? Wk + (size_t)pp[k] * ld : nullptr;
+        }
+        for (int cb = 0; cb < n; cb += 32, buf ^= 32 * 33) {
+            const int c = cb + lane;
+            float2 v[RW];
+#pragma unroll
+            for (int r = 0; r < RW; ++r) v[r] = (row[r] && c < n) ? row[r][c] : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                tile[buf + (wid + r * WARPS) * 33 + lane] = v[r];
+                if (c < n) rs[r] += fabsf(v[r].x);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                const int cr = cb + wid + r * WARPS, k = kb + lane;
+                if (cr < n && k < n) Dout[(size_t)pp[cr] * n + k] = join_f64(tile[buf + lane * 33 + wid + r * WARPS]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rs[r] += __shfl_xor_sync(0xffffffffu, rs[r], o);
+            imax = fmaxf(imax, rs[r]);
+        }
     }
     if (lane == 0) red_f[wid] = imax;
 
-    float2 *tile = P;   // [32][33]
-    for (int kb = 0; kb < n; kb += 32) {
-        for (int cb = 0; cb < n; cb += 32) {
-            for (int r = wid; r < 32; r += kGjWarps) {
-                const int k = kb + r, c = cb + lane;
-                tile[r * 33 + lane] = (k < n && c < n) ? Wk[(size_t)pp[k] * n + c] : make_float2(0.f, 0.f);
-            }
-            __syncthreads();
-            for (int r = wid; r < 32; r += kGjWarps) {
-                const int c = cb + r, k = kb + lane;
-                if (c < n && k < n) Dout[(size_t)pp[c] * n + k] = ff::val(tile[lane * 33 + r]);
-            }
-            __syncthreads();
-        }
-    }
-
-    if (t == 0) {
+    // parity of the row permutation k -> pp[k]: its inversions
+    int inv = 0;
+    for (int i = t; i < n; i += THREADS)
+        for (int j = i + 1; j < n; ++j) inv ^= pp[j] < pp[i];
+    const int par = __syncthreads_count(inv) & 1;
+    if (t == THREADS - 32) {
         float im = 0.f;
-        for (int q = 0; q < kGjWarps; ++q) im = fmaxf(im, red_f[q]);
+        for (int q = 0; q < WARPS; ++q) im = fmaxf(im, red_f[q]);
         const double kappa = (double)s_xnorm * (double)im;
-        int par = 0;
-        for (int i = 0; i < n; ++i) used[i] = 0;
-        for (int i = 0; i < n; ++i) {
-            if (used[i]) continue;
-            int len = 0, j = i;
-            while (!used[j]) { used[j] = 1; j = pp[j]; ++len; }
-            par ^= ((len & 1) == 0);
-        }
         const double logabs = log((double)mag_h + (double)mag_l) + mag_e * 0.69314718055994530942;
         if (J.logabs) J.logabs[(size_t)m * J.la_stride] = logabs;
         if (J.sign) J.sign[(size_t)m * J.la_stride] = (par ^ neg) ? -1.0 : 1.0;
@@ -541,18 +624,41 @@ __global__ void __launch_bounds__(kGjThreads, NB == 8 ? 4 : (NB == 16 ? 3 : 1)) 
     }
 }
 
+template <int NB, int THREADS, int RPT, int MIN, bool kSmem>
+static cudaError_t launch_gj_ff_k(const GjJobs2 &js, int n_jobs, int nmax, int cmax, double kappa_max,
+                                  cudaStream_t st)
+{
+    const size_t sm = gjff_fixed_bytes(nmax, NB) + (kSmem ? sizeof(float2) * nmax * (size_t)(nmax | 1) : 0);
+    auto kern = k_gj_ff<NB, THREADS, RPT, MIN, kSmem>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    dim3 grid(cmax, n_jobs);
+    kern<<<grid, THREADS, sm, st>>>(js, kappa_max);
+    return cudaGetLastError();
+}
+
+// One row per thread while the rows fit a block of 256 or 512, else two.  Blocks of 256: the work
+// matrix in shared memory where that leaves room for the matrices' CTAs (three on each of 152 SMs,
+// or as many as there are: 2 matrices of 79 rows 164 -> 152 us); else with registers for two CTAs
+// per SM where two hold every matrix, for three beyond (8192 matrices of 217 rows: 54.5 -> 52.0 ms;
+// 2 of 79 rows: 164 -> 177 us).
 template <int NB>
 static cudaError_t launch_gj_ff_nb(const GjJobs2 &js, int n_jobs, int nmax, int cmax, double kappa_max,
                                    cudaStream_t st)
 {
-    const size_t sm = sizeof(float2) * (p_region(nmax, NB) + NB * 32) + sizeof(short) * 3 * (size_t)nmax;
-    cudaError_t e = cudaFuncSetAttribute(k_gj_ff<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_gj_ff<NB>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    dim3 grid(cmax, n_jobs);
-    k_gj_ff<NB><<<grid, kGjThreads, sm, st>>>(js, kappa_max);
-    return cudaGetLastError();
+    constexpr int M2 = NB <= 16 ? 2 : 1, M3 = NB <= 16 ? 3 : 1;
+    if (nmax <= 256) {
+        const long long T = (long long)cmax * n_jobs;
+        const size_t sm = gjff_fixed_bytes(nmax, NB) + sizeof(float2) * nmax * (size_t)(nmax | 1);
+        if (sm <= 72 * 1024 || (T <= 304 && sm <= 108 * 1024) || (T <= 152 && sm <= 220 * 1024))
+            return launch_gj_ff_k<NB, 256, 1, M2, true>(js, n_jobs, nmax, cmax, kappa_max, st);
+        if (T <= 304) return launch_gj_ff_k<NB, 256, 1, M2, false>(js, n_jobs, nmax, cmax, kappa_max, st);
+        return launch_gj_ff_k<NB, 256, 1, M3, false>(js, n_jobs, nmax, cmax, kappa_max, st);
+    }
+    if (nmax <= 512) return launch_gj_ff_k<NB, 512, 1, 1, false>(js, n_jobs, nmax, cmax, kappa_max, st);
+    return launch_gj_ff_k<NB, 512, 2, 1, false>(js, n_jobs, nmax, cmax, kappa_max, st);
 }
 
 cudaError_t launch_gj_ff(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb, double kappa_max)

@@ -45,3 +45,33 @@ def test_wide_large_inverse(n, batch):
     assert ((logabs - l).abs() / l.abs()).max().item() < 1e-10
     E = D.mT @ X - torch.eye(n, dtype=torch.float64, device=dev)
     assert E.abs().max().item() < n * 2.0 ** -53 * 1e6
+
+
+@pytest.mark.parametrize("key,W", [("tiny", 3), ("119e", 1), ("119e", 200), ("158e", 1), ("158e", 160), ("300e", 2),
+                                   ("434e", 3), ("434e", 160), ("700e", 2), ("1056e", 2)])
+@pytest.mark.parametrize("panel", [8, 16, 32])
+def test_float_float_inverse(key, W, panel):
+    """The float-float elimination in its forms (work matrix in shared memory or not, one or two rows per
+    thread, short last panels, odd sizes) against the FP64 one on the same C1 (qmc_slater_matrices):
+    log|det| within the mixed path's 1e-6 and the inverse's residual max|D^T C1 - 1| within 1e-6
+    (float pairs and a mixed C1, ~2^-44 x kappa <= 1e7; near-node matrices are recomputed in FP64)."""
+    from paper_1209_6630_gb300 import QmcSystem, det_inverse
+    from synth import config_system, make_system, make_walkers, tiny_system
+    s = {"tiny": lambda: tiny_system("h2o_like"), "119e": lambda: make_system(9, 3, 3, 20, seed=21),
+         "300e": lambda: make_system(22, 6, 8, 62, seed=31), "700e": lambda: make_system(53, 15, 16, 149, seed=32)}.get(
+             key, lambda: config_system(key))()
+    q = QmcSystem(s, 0)
+    q.set_tiles(a4_mode="float_float", gj_panel=panel, a4_kappa_max=1e7, c15_mode="tensor")
+    R = torch.from_numpy(make_walkers(s, W, first=91000)).to(dev)
+    out = q.eval(R, precision="mixed", want_dinv=True)
+    assert (out["status"] == 0).all()
+    sample = torch.unique(torch.linspace(0, W - 1, min(W, 6)).long())
+    for sp, C in enumerate(q.slater(R, precision="mixed")):
+        n = C.shape[-1]
+        off = s.n_up ** 2 if sp else 0
+        C1 = C[sample.to(dev), 0].contiguous()
+        D = out["dinv"][sample.to(dev), off: off + n * n].reshape(-1, n, n)
+        logabs = det_inverse(C1.clone())[0]
+        assert (out["logabs"][sample.to(dev), sp] - logabs).abs().max().item() < 1e-6
+        E = D.mT @ C1 - torch.eye(n, dtype=torch.float64, device=dev)
+        assert E.abs().max().item() < 1e-6
