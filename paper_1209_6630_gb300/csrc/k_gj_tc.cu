@@ -9,15 +9,14 @@
 //
 //   k_gt_init    float-pair copy of X (rows padded to an even length) and ||X||_inf
 //   per panel jb:
-//   k_gt_panel_t one CTA per matrix eliminates the n x 32 panel in shared
-//   (k_gt_panel) memory (pivot = the first row with the largest |entry| among
+//   k_gt_panel   one CTA per matrix eliminates the n x 32 panel, one thread per
+//                row (pivot = the first row with the largest |entry| among
 //                the rows not used yet: the pivots of LU with partial
-//                pivoting) -- one thread per row, in sub-panels of 8 with
-//                rank-8 updates between them, up to 544 rows, else one warp
-//                per row -- and writes the operands of the panel's update in
-//                exact BF16 slices: the panel P [n][32] (row i scaled by
-//                2^-E_i) and the pivot rows U [32][n] as they were before the
-//                update (column j scaled by 2^-F_j), seven slices of 7 bits
+//                pivoting), in sub-panels of 8 held in registers, and writes
+//                the operands of the panel's update in exact BF16 slices: the
+//                panel P [n][32] (row i scaled by 2^-E_i) and the pivot rows
+//                U [32][n] as they were before the update (column j scaled
+//                by 2^-F_j), seven slices of 7 bits
 //                each (the scheme of the C1/C5 products, one slice more)
 //   k_gt_update  X[i][j] <- [i is not a pivot row of the panel] X[i][j]
 //                           + sum_c P[i][c] U[c][j]
@@ -60,8 +59,6 @@ namespace cg = cooperative_groups;
 constexpr int kGtB = 32;                             // panel width = K of the update
 constexpr int kGtThreads = 256;                      // init and final kernels
 constexpr int kGtWarps = kGtThreads / 32;
-constexpr int kGpThreads = 512;                      // panel kernel: one warp per row, 16 rows at a time
-constexpr int kGpWarps = kGpThreads / 32;
 constexpr int kGtEpWarps = 16;                       // update kernel: 4 lane quadrants x 4 groups of 8 columns,
 constexpr int kGtUpThreads = 32 * (kGtEpWarps + 3);  // plus the X, B and MMA warps
 constexpr int kGtN = 32;                             // columns per update tile (= the panel width)
@@ -127,22 +124,6 @@ struct GtJobs {
     CUtensorMap tmw[2];                              // the work matrices of job q as [matrix][row][column]
 };
 
-__device__ __forceinline__ void gt_argmax_merge(float &v, int &i, float v2, int i2)
-{
-    if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
-}
-
-__device__ __forceinline__ void gt_block_argmax(float &bv, int &bi, float *red_v, int *red_i, int lane, int wid)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float v2 = __shfl_down_sync(0xffffffffu, bv, o);
-        const int i2 = __shfl_down_sync(0xffffffffu, bi, o);
-        gt_argmax_merge(bv, bi, v2, i2);
-    }
-    if (lane == 0) { red_v[wid] = bv; red_i[wid] = bi; }
-}
-
 // Float-pair copy of X and ||X||_inf; a cluster of CTAs shares a matrix's rows where the matrices
 // are few.  Both this kernel and k_gt_final only move data, but were bound by the FP64 pipe's
 // conversions; on the integer pipes (f64_bits.cuh), 4096 matrices of 528 rows: 8.5 -> 3.8 ms
@@ -202,8 +183,9 @@ __global__ void __launch_bounds__(kGtThreads) k_gt_init(GtJobs js)
     if (nrank > 1) cluster.sync();                       // no CTA leaves before its maximum is read
 }
 
-// Operand B of the update: the pivot rows before the update (zero in the panel's columns
-// and for c >= w), scaled per column; one thread per column, its 32 values loaded at once.
+// Operand B of the update: the pivot rows before the update (zero in the panel's columns and for
+// c >= w), scaled per column: first the column exponents (one thread per column, its 32 values
+// loaded at once), then the slices (8 columns of one pivot row per thread, 16-byte stores).
 __device__ __forceinline__ void gt_operand_b(unsigned char *sc, const GtLayout &L, int n, int jb, int w,
                                              const short *ppS)
 {
@@ -213,196 +195,94 @@ __device__ __forceinline__ void gt_operand_b(unsigned char *sc, const GtLayout &
     unsigned char *Bpl = sc + L.b;
     for (int col = threadIdx.x; col < n; col += blockDim.x) {
         const bool vcol = !(col >= jb && col < jb + w);
-        float2 u[kGtB];
         float mx = 0.f;
 #pragma unroll
-        for (int c = 0; c < kGtB; ++c) {
-            u[c] = (vcol && c < w) ? Wk[(size_t)ppS[c] * ld + col] : make_float2(0.f, 0.f);
-            mx = fmaxf(mx, fabsf(u[c].x));
-        }
-        const int F = exp_bound(mx);
-        Fcol[col] = F;
-        const int cl = col % kGtN;
-        unsigned char *base = Bpl + (size_t)(col / kGtN) * kGtSl * kGtBPlane + (cl & 7) * 2;
-#pragma unroll
-        for (int c = 0; c < kGtB; ++c) {
-            float s7[kGtSl];
-            slice_n<kGtSl>(u[c], F, s7);
-            unsigned char *b = base + b_off32c(c, cl & ~7);
-#pragma unroll
-            for (int j = 0; j < kGtSl; ++j)
-                *reinterpret_cast<__nv_bfloat16 *>(b + (size_t)j * kGtBPlane) = __float2bfloat16_rn(s7[j]);
-        }
+        for (int c = 0; c < kGtB; ++c) mx = fmaxf(mx, (vcol && c < w) ? fabsf(Wk[(size_t)ppS[c] * ld + col].x) : 0.f);
+        Fcol[col] = exp_bound(mx);
     }
-}
-
-__global__ void __launch_bounds__(kGpThreads, 1) k_gt_panel(GtJobs js)
-{
-    const GjJob &J = js.j[blockIdx.y];
-    const int m = blockIdx.x;
-    const int n = J.n, jb = js.jb;
-    if (m >= J.count || jb >= n) return;
-    const GtLayout L = gt_layout(n);
-    unsigned char *sc = js.scr[blockIdx.y] + (size_t)m * L.per;
-    GtState *st = reinterpret_cast<GtState *>(sc + L.state);
-    if (st->sing) return;
-    float2 *__restrict__ Wk = reinterpret_cast<float2 *>(sc + L.w);
-    const int ld = gt_ld(n);
-    short *pp_g = reinterpret_cast<short *>(sc + L.pp);
-    short *used_g = reinterpret_cast<short *>(sc + L.used);
-    unsigned char *piv_g = sc + L.piv;
-    int *Erow = reinterpret_cast<int *>(sc + L.e);
-    unsigned char *Apl = sc + L.a;
-
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *P = reinterpret_cast<float2 *>(smem_raw);           // [n][32]
-    short *used = reinterpret_cast<short *>(P + (size_t)n * kGtB);
-    __shared__ short ppS[kGtB];
-    __shared__ int red_i[kGpWarps];
-    __shared__ float red_f[kGpWarps];
-
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    const int w = min(kGtB, n - jb);
-    // the previous panel's pivots stop being pivots of the current panel
-    if (jb > 0 && t < kGtB) piv_g[pp_g[jb - kGtB + t]] = 0;
-    for (int i = t; i < n; i += kGpThreads) used[i] = used_g[i];
-    // the panel: one row of 32 per warp and step, four rows' loads in flight
-    for (int i0 = wid; i0 < n; i0 += 4 * kGpWarps) {
-        float2 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = i0 + u * kGpWarps;
-            v[u] = (i < n && lane < w) ? Wk[(size_t)i * ld + jb + lane] : make_float2(0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = i0 + u * kGpWarps;
-            if (i < n) P[i * kGtB + lane] = v[u];
-        }
-    }
-    GtState S = *st;
-    bool sing = false;
     __syncthreads();
-    float bv = -1.f;
-    int bi = n;
-    for (int i = t; i < n; i += kGpThreads)
-        if (!used[i]) gt_argmax_merge(bv, bi, fabsf(P[i * kGtB].x), i);
-    gt_block_argmax(bv, bi, red_f, red_i, lane, wid);
-    __syncthreads();
-
-    // one warp per row, lane = panel column: contiguous shared-memory accesses
-    const int cc = lane;
-    for (int c = 0; c < w; ++c) {
-        float v = red_f[0];
-        int p = red_i[0];
-        for (int q = 1; q < kGpWarps; ++q) gt_argmax_merge(v, p, red_f[q], red_i[q]);
-        if (!(v > 0.f)) {   // every thread sees the same candidates: all leave together
-            sing = true;
-            break;
-        }
-        const float2 pv = P[p * kGtB + c];
-        const float2 pinv = ff::inv(pv);
-        const float2 prow = (cc == c) ? pinv : ff::mul(P[p * kGtB + cc], pinv);
-        {
-            const float2 a = pv.x < 0.f ? ff::neg(pv) : pv;
-            const float2 mg = ff::mul(make_float2(S.mag_h, S.mag_l), a);
-            int ex;
-            frexpf(mg.x, &ex);
-            S.mag_h = ldexpf(mg.x, -ex);
-            S.mag_l = ldexpf(mg.y, -ex);
-            S.mag_e += ex;
-            S.neg ^= pv.x < 0.f;
-        }
-        if (t == 0) {
-            used[p] = 1;
-            ppS[c] = (short)p;
-        }
-        __syncthreads();                                  // the candidates and row p have been read
-        if (t < kGtB) P[p * kGtB + t] = prow;
-        float nbv = -1.f;
-        int nbi = n;
-        const int cn = c + 1;
-        // four rows per step (independent chains in flight)
-        constexpr int RU = 4;
-        for (int i0 = wid; i0 < n; i0 += RU * kGpWarps) {
-            float2 mf[RU], a[RU];
-            bool live[RU];
+    const int nch = (n + 7) / 8;
+    for (int it = threadIdx.x; it < kGtB * nch; it += blockDim.x) {
+        const int c = it / nch, col0 = (it - c * nch) * 8;
+        uint32_t o[kGtSl][4];
 #pragma unroll
-            for (int u = 0; u < RU; ++u) {
-                const int i = i0 + u * kGpWarps;
-                live[u] = i < n && i != p;
-                mf[u] = live[u] ? ff::neg(P[i * kGtB + c]) : make_float2(0.f, 0.f);
-                // lane c: 0 + m * pinv (its prow is pinv), the same expression as the other lanes
-                a[u] = (live[u] && cc != c) ? P[i * kGtB + cc] : make_float2(0.f, 0.f);
+        for (int q = 0; q < 4; ++q) {
+            float s7[2][kGtSl];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int col = col0 + 2 * q + h;
+                const bool v = c < w && col < n && !(col >= jb && col < jb + w);
+                slice_n<kGtSl>(v ? Wk[(size_t)ppS[c] * ld + col] : make_float2(0.f, 0.f), col < n ? Fcol[col] : 0, s7[h]);
             }
-            __syncwarp();                                 // every lane has read the rows' column c
 #pragma unroll
-            for (int u = 0; u < RU; ++u) {
-                const int i = i0 + u * kGpWarps;
-                if (!live[u]) continue;
-                const float2 x = ff::fma2(a[u], mf[u], prow);
-                P[i * kGtB + cc] = x;
-                if (cc == cn && cn < w && !used[i]) gt_argmax_merge(nbv, nbi, fabsf(x.x), i);
-            }
+            for (int j = 0; j < kGtSl; ++j) o[j][q] = bf16_pair(s7[0][j], s7[1][j]);
         }
-        gt_block_argmax(nbv, nbi, red_f, red_i, lane, wid);
-        __syncthreads();
-    }
-    if (sing) {
-        if (t == 0) st->sing = 1;
-        return;
-    }
-    // the eliminated panel is part of the result; bookkeeping of the pivots
-    for (int i = wid; i < n; i += kGpWarps)
-        if (lane < w) Wk[(size_t)i * ld + jb + lane] = P[i * kGtB + lane];
-    if (t < w) {
-        const int p = ppS[t];
-        pp_g[jb + t] = (short)p;
-        used_g[p] = 1;
-        piv_g[p] = 1;
-    }
-    if (t == 0) {
-        GtState o = *st;
-        o.mag_h = S.mag_h; o.mag_l = S.mag_l; o.mag_e = S.mag_e; o.neg = S.neg;
-        *st = o;
-    }
-
-    // operand A: the panel's rows, scaled per row, six slices, [row tile][slice] planes
-    for (int i = wid; i < n; i += kGpWarps) {
-        const float2 x = P[i * kGtB + lane];
-        float mx = fabsf(x.x);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        const int E = exp_bound(mx);
-        float s7[kGtSl];
-        slice_n<kGtSl>(x, E, s7);
-        unsigned char *base = Apl + (size_t)(i >> 7) * kGtSl * kGtAPlane + a_off64(i & 127, lane >> 3) +
-                              (lane & 7) * 2;
+        unsigned char *b = Bpl + (size_t)(col0 / kGtN) * kGtSl * kGtBPlane + b_off32c(c, col0 % kGtN);
 #pragma unroll
         for (int j = 0; j < kGtSl; ++j)
-            *reinterpret_cast<__nv_bfloat16 *>(base + (size_t)j * kGtAPlane) = __float2bfloat16_rn(s7[j]);
-        if (lane == 0) Erow[i] = E;
+            *reinterpret_cast<uint4 *>(b + (size_t)j * kGtBPlane) = make_uint4(o[j][0], o[j][1], o[j][2], o[j][3]);
     }
-    gt_operand_b(sc, L, n, jb, w, ppS);
 }
 
-// The panel kernel with one thread per row (n <= kGpRowMax): thread i owns row i of the
-// n x 32 panel (shared memory, rows padded to 33 float pairs: conflict-free).  The 32 columns
-// are eliminated in four sub-panels of 8, whose columns sit in the thread's registers: each
-// pivot step updates only those 8 columns (the pivot column becomes the column of the step's
-// Gauss-Jordan transformation, as in k_gt_panel); after the sub-panel its composed
-// transformation T = I + W S (W: the 8 transformation columns, S: the 8 pivot rows) is
-// applied to the other 24 panel columns as one rank-8 float-float update,
-//   X[i][j] <- [i not a pivot of the sub-panel] X[i][j] + sum_k W[i][k] X[p_k][j],
-// with the pivot rows' values from before the sub-panel.  The pivot rule (largest |entry|
-// among the rows not used yet, the first on ties) and the arithmetic per multiply-add are
-// those of the column-by-column elimination; the sums over a sub-panel's pivots are taken in
-// pivot order.  ~3x fewer instructions than k_gt_panel.
-constexpr int kGpRowMax = 544;
-constexpr int kGpSub = 8;
-constexpr int kGpRowLd = kGtB + 1;                       // float pairs per shared-memory row
+// |x| as an integer that orders like it; 0 for NaN (never a pivot) and 0
+__device__ __forceinline__ unsigned gt_key(float x)
+{
+    const unsigned b = __float_as_uint(x) & 0x7fffffffu;
+    return b > 0x7f800000u ? 0u : b;
+}
 
-__global__ void __launch_bounds__(kGpRowMax, 1) k_gt_panel_t(GtJobs js)
+// The largest key of a warp and the smallest index that has it, in every lane.
+__device__ __forceinline__ void gt_warp_max(unsigned &k, int &i)
+{
+    const unsigned m = __reduce_max_sync(0xffffffffu, k);
+    i = (int)__reduce_min_sync(0xffffffffu, k == m ? (unsigned)i : 0x7fffffffu);
+    k = m;
+}
+
+__device__ __forceinline__ float2 gt_neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// ff::fma2 for two values at once (packed FP32, the same roundings): (ah, al) + (xh, xl) (yh, yl)
+__device__ __forceinline__ void gt_fma2x2(float2 &ah, float2 &al, float2 xh, float2 xl, float2 yh, float2 yl)
+{
+    const float2 p = __fmul2_rn(xh, yh);
+    float2 pe = __ffma2_rn(xh, yh, gt_neg2(p));
+    pe = __ffma2_rn(xh, yl, pe);
+    pe = __ffma2_rn(xl, yh, pe);
+    const float2 s = __fadd2_rn(ah, p), bb = __fadd2_rn(s, gt_neg2(ah));
+    float2 se = __fadd2_rn(__fadd2_rn(ah, gt_neg2(__fadd2_rn(s, gt_neg2(bb)))), __fadd2_rn(p, gt_neg2(bb)));
+    se = __fadd2_rn(se, __fadd2_rn(al, pe));
+    ah = __fadd2_rn(s, se);
+    al = __fadd2_rn(se, gt_neg2(__fadd2_rn(ah, gt_neg2(s))));
+}
+
+__device__ __forceinline__ float2 gt_dup(float x) { return make_float2(x, x); }
+
+// The panel kernel: one thread per row.  The 32 columns are eliminated in four sub-panels of 8,
+// whose columns sit in the thread's registers: each pivot step updates only those 8 columns (the
+// pivot column becomes the column of the step's Gauss-Jordan transformation); the other 24 lie
+// in shared memory (pairs of columns {h, h', l, l'}, rows of 13 x 16 bytes: conflict-free) and take
+// the sub-panel's 8 pivots afterwards, two column pairs at a time in packed FP32; then the
+// registers change places with the next sub-panel's columns.
+//
+// kSeq = false (up to kGtSeqMin - 1 rows): the sub-panel's composed transformation T = I + W S (W:
+// the 8 transformation columns, S: the 8 pivot rows from before the sub-panel) as one rank-8 update,
+//   X[i][j] <- [i not a pivot of the sub-panel] X[i][j] + sum_k W[i][k] X[p_k][j].
+// kSeq = true: the 8 steps one after the other, X[i][j] <- X[i][j] - X[i][p_k's column] prow_k[j] with
+// the multipliers of each step kept in registers and the scaled pivot rows prow_k formed by 24
+// threads in step order: the roundings of a column-by-column elimination.  (The two differ in their
+// last bits, which an ill-conditioned matrix amplifies; each size keeps the one that it has had.)
+//
+// What bounds it is the FP32 pipe (15 operations per float-float multiply-add) and the chain of a
+// step: a REDUX search for the pivot (first of the rows not used yet with the largest |entry|), two
+// barriers, the pivot row scaled by its owner's warp.  Measured, one CTA per SM: 4096 matrices of
+// 528 rows, 17 panels, 54.0 -> 47.6 ms; 1024 of 866 rows, 28 panels (a warp per row before), 55.5 ->
+// 35.9 ms.
+constexpr int kGtSeqMin = 545;
+constexpr int kGpSub = 8;
+constexpr int kGpLd = 13;                                // float4 per shared-memory row
+
+template <int kMaxT, bool kSeq>
+__global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
 {
     const GjJob &J = js.j[blockIdx.y];
     const int m = blockIdx.x;
@@ -417,81 +297,87 @@ __global__ void __launch_bounds__(kGpRowMax, 1) k_gt_panel_t(GtJobs js)
     short *pp_g = reinterpret_cast<short *>(sc + L.pp);
     short *used_g = reinterpret_cast<short *>(sc + L.used);
     unsigned char *piv_g = sc + L.piv;
-    int *Erow = reinterpret_cast<int *>(sc + L.e);
-    unsigned char *Apl = sc + L.a;
 
     extern __shared__ __align__(16) unsigned char gp_smem[];
-    float2 *P = reinterpret_cast<float2 *>(gp_smem);     // [blockDim.x][kGpRowLd]
-    __shared__ __align__(16) float2 U_s[kGpSub][kGtB];    // the sub-panel's pivot rows, before it
-    __shared__ float2 prow_s[kGpSub + 1];                 // the step's pivot row on the sub-panel, scaled; 1 / pivot
+    __shared__ float4 U_s[kGpSub][12];                    // pivot rows of the sub-panel, other columns
+    __shared__ float2 raw_s[kGpSub], prow_s[kGpSub];      // the step's pivot row on the sub-panel: raw, scaled
+    __shared__ float2 pinv_s[kGpSub], mul_s[kGpSub][kGpSub];   // kSeq: 1 / pivot, multipliers of the pivot rows
     __shared__ short ppS[kGtB];
-    __shared__ int red_i[kGpRowMax / 32];
-    __shared__ float red_f[kGpRowMax / 32];
+    __shared__ unsigned red_k[kMaxT / 32];
+    __shared__ int red_i[kMaxT / 32];
 
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nwarps = blockDim.x >> 5;
     const int w = min(kGtB, n - jb);
     const int i = t;                                      // this thread's row
     const bool row_ok = i < n;
-    float2 *row = P + (size_t)t * kGpRowLd;
+    float4 *P = reinterpret_cast<float4 *>(gp_smem), *row = P + (size_t)t * kGpLd;
     // the previous panel's pivots stop being pivots of the current panel
     if (jb > 0 && t < kGtB) piv_g[pp_g[jb - kGtB + t]] = 0;
-    if (row_ok && w == kGtB) {
-        const float4 *src = reinterpret_cast<const float4 *>(Wk + (size_t)i * ld + jb);
+    float2 xh[4], xl[4];                                  // the sub-panel's columns 2 q, 2 q + 1 of this row
+    {
+        const float2 *src = Wk + (size_t)(row_ok ? i : 0) * ld + jb;
 #pragma unroll
         for (int q = 0; q < kGtB / 2; ++q) {
-            const float4 v = src[q];
-            row[2 * q] = make_float2(v.x, v.y);
-            row[2 * q + 1] = make_float2(v.z, v.w);
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row_ok && w == kGtB) v = *reinterpret_cast<const float4 *>(src + 2 * q);
+            else if (row_ok) {
+                if (2 * q < w) { v.x = src[2 * q].x; v.y = src[2 * q].y; }
+                if (2 * q + 1 < w) { v.z = src[2 * q + 1].x; v.w = src[2 * q + 1].y; }
+            }
+            if (q < 4) {
+                xh[q] = make_float2(v.x, v.z);
+                xl[q] = make_float2(v.y, v.w);
+            } else {
+                row[q - 4] = make_float4(v.x, v.z, v.y, v.w);
+            }
         }
-    } else {
-        for (int j = 0; j < kGtB; ++j) row[j] = (row_ok && j < w) ? Wk[(size_t)i * ld + jb + j] : make_float2(0.f, 0.f);
     }
     bool used = !row_ok || used_g[i] != 0;
     GtState S = *st;
     bool sing = false;
+    auto elem = [&](int c) { return (c & 1) ? make_float2(xh[c >> 1].y, xl[c >> 1].y) : make_float2(xh[c >> 1].x, xl[c >> 1].x); };
 
+#pragma unroll 1
     for (int sb = 0; sb < kGtB / kGpSub && sb * kGpSub < w; ++sb) {
         const int c0 = sb * kGpSub;
-        float2 xs[kGpSub];                                // the sub-panel's columns of this row
-#pragma unroll
-        for (int q = 0; q < kGpSub; ++q) xs[q] = row[c0 + q];
-        int nk = 0;                                       // pivots of this sub-panel
-        bool sub_piv = false;                             // this row is one of them
+        const int nk = min(kGpSub, w - c0);               // pivots of this sub-panel
+        int my_k = -1;                                    // this row's step, if it is one of them
+        float2 mf[kSeq ? kGpSub : 1];                     // kSeq: the row's multiplier of each step
 #pragma unroll
         for (int cc = 0; cc < kGpSub; ++cc) {
-            if (c0 + cc >= w) break;
+            if (cc >= nk) break;
             // block-wide argmax of |x[c]| over the rows not used yet
-            float bv = used ? -1.f : fabsf(xs[cc].x);
-            int bi = used ? n : i;
-            gt_block_argmax(bv, bi, red_f, red_i, lane, wid);
+            const float2 xc = elem(cc);
+            unsigned k = used ? 0u : gt_key(xc.x);
+            int p = used ? n : i;
+            gt_warp_max(k, p);
+            if (lane == 0) { red_k[wid] = k; red_i[wid] = p; }
             __syncthreads();
-            // every warp merges the warps' candidates by shuffles (the same merge rule, any order)
-            float v = lane < nwarps ? red_f[lane] : -1.f;
-            int p = lane < nwarps ? red_i[lane] : n;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float v2 = __shfl_xor_sync(0xffffffffu, v, o);
-                const int p2 = __shfl_xor_sync(0xffffffffu, p, o);
-                gt_argmax_merge(v, p, v2, p2);
-            }
-            if (!(v > 0.f)) {                             // every thread sees the same candidates
+            k = lane < nwarps ? red_k[lane] : 0u;
+            p = lane < nwarps ? red_i[lane] : n;
+            gt_warp_max(k, p);
+            if (k == 0u) {                                // every warp sees the same candidates
                 sing = true;
                 break;
             }
-            if (i == p) {                                 // publish the pivot row (all 32 columns) and,
-                for (int j = 0; j < kGtB; ++j) U_s[cc][j] = row[j];   // scaled by 1 / pivot, its
-#pragma unroll                                            // sub-panel part
-                for (int q = 0; q < kGpSub; ++q) U_s[cc][c0 + q] = xs[q];
-                const float2 pinv_o = ff::inv(xs[cc]);
+            if (wid == p >> 5) {                          // the pivot row, scaled a column per lane
+                if (i == p) {
 #pragma unroll
-                for (int q = 0; q < kGpSub; ++q) prow_s[q] = (q == cc) ? pinv_o : ff::mul(xs[q], pinv_o);
-                prow_s[kGpSub] = pinv_o;
-                used = true;
-                sub_piv = true;
+                    for (int q = 0; q < kGpSub; ++q) raw_s[q] = elem(q);
+                    used = true;
+                    my_k = cc;
+                }
+                __syncwarp();
+                const float2 pinv = ff::inv(raw_s[cc]);
+                if (lane < kGpSub) prow_s[lane] = lane == cc ? pinv : ff::mul(raw_s[lane], pinv);
+                if (lane == 0) {
+                    ppS[c0 + cc] = (short)p;
+                    if (kSeq) pinv_s[cc] = pinv;
+                }
             }
             __syncthreads();
-            const float2 pv = U_s[cc][c0 + cc];
-            if (t == 0) {
+            if (wid == nwarps - 1) {                      // (the last warp has the fewest rows)
+                const float2 pv = raw_s[cc];
                 const float2 a = pv.x < 0.f ? ff::neg(pv) : pv;
                 const float2 mg = ff::mul(make_float2(S.mag_h, S.mag_l), a);
                 int ex;
@@ -500,82 +386,147 @@ __global__ void __launch_bounds__(kGpRowMax, 1) k_gt_panel_t(GtJobs js)
                 S.mag_l = ldexpf(mg.y, -ex);
                 S.mag_e += ex;
                 S.neg ^= pv.x < 0.f;
-                ppS[c0 + cc] = (short)p;
             }
-            // the step on the sub-panel's 8 columns (the same expressions as k_gt_panel)
-            const float2 mf = ff::neg(xs[cc]);
+            // the step on the sub-panel's 8 columns: the pivot column starts from zero
+            const float2 f = ff::neg(xc);
+            if constexpr (kSeq) mf[cc] = f;
 #pragma unroll
-            for (int q = 0; q < kGpSub; ++q) {
-                const float2 prow = prow_s[q];
-                if (i == p) xs[q] = prow;
-                else xs[q] = ff::fma2(q == cc ? make_float2(0.f, 0.f) : xs[q], mf, prow);
+            for (int q = 0; q < 4; ++q) {
+                const float2 y0 = prow_s[2 * q], y1 = prow_s[2 * q + 1];
+                const float2 yh = make_float2(y0.x, y1.x), yl = make_float2(y0.y, y1.y);
+                if (i == p) {
+                    xh[q] = yh;
+                    xl[q] = yl;
+                } else {
+                    if (2 * q == cc) xh[q].x = xl[q].x = 0.f;
+                    if (2 * q + 1 == cc) xh[q].y = xl[q].y = 0.f;
+                    gt_fma2x2(xh[q], xl[q], gt_dup(f.x), gt_dup(f.y), yh, yl);
+                }
             }
-            ++nk;
         }
         if (sing) break;
+        // the pivot rows' other columns, from before the sub-panel
+        for (int q = t; q < nk * 12; q += blockDim.x) U_s[q / 12][q % 12] = P[(size_t)ppS[c0 + q / 12] * kGpLd + q % 12];
+        if constexpr (kSeq)
+            if (my_k >= 0)
 #pragma unroll
-        for (int q = 0; q < kGpSub; ++q) row[c0 + q] = xs[q];
-        // the sub-panel's transformation on the other 24 columns, pivot rows from before it
-        // (two columns per pass: two independent chains, U_s read 16 bytes at a time)
-        for (int j = 0; j < kGtB; j += 2) {
-            if (j >= c0 && j < c0 + kGpSub) continue;
-            float2 a0 = sub_piv ? make_float2(0.f, 0.f) : row[j];
-            float2 a1 = sub_piv ? make_float2(0.f, 0.f) : row[j + 1];
+                for (int c = 0; c < kGpSub; ++c) mul_s[my_k][c] = mf[c];
+        __syncthreads();
+        if constexpr (kSeq) {
+            // prow_k of the other columns, in step order: one thread per column
+            if (t < 24) {
+                float *u = reinterpret_cast<float *>(&U_s[0][t >> 1]) + (t & 1);
+                float2 pr[kGpSub];
 #pragma unroll
-            for (int k = 0; k < kGpSub; ++k)
-                if (k < nk) {
-                    const float4 u = *reinterpret_cast<const float4 *>(&U_s[k][j]);
-                    a0 = ff::fma2(a0, xs[k], make_float2(u.x, u.y));
-                    a1 = ff::fma2(a1, xs[k], make_float2(u.z, u.w));
+                for (int k = 0; k < kGpSub; ++k) {
+                    if (k >= nk) break;
+                    float2 v = make_float2(u[k * 48], u[k * 48 + 2]);
+#pragma unroll
+                    for (int c = 0; c < k; ++c) v = ff::fma2(v, mul_s[k][c], pr[c]);
+                    pr[k] = ff::mul(v, pinv_s[k]);
+                    u[k * 48] = pr[k].x;
+                    u[k * 48 + 2] = pr[k].y;
                 }
-            row[j] = a0;
-            row[j + 1] = a1;
+            }
+            __syncthreads();
         }
-        __syncthreads();                                  // U_s is rewritten by the next sub-panel
+        // the sub-panel's pivots on the other 24 columns of this row
+        const bool any_piv = __any_sync(0xffffffffu, my_k >= 0);
+#pragma unroll 1
+        for (int j = 0; j < 12; j += 2) {
+            float4 a0 = row[j], a1 = row[j + 1];
+            if (!kSeq && my_k >= 0) a0 = a1 = make_float4(0.f, 0.f, 0.f, 0.f);
+            float2 h0 = make_float2(a0.x, a0.y), l0 = make_float2(a0.z, a0.w);
+            float2 h1 = make_float2(a1.x, a1.y), l1 = make_float2(a1.z, a1.w);
+#pragma unroll
+            for (int k = 0; k < kGpSub; ++k) {
+                if (k >= nk) break;
+                const float4 u0 = U_s[k][j], u1 = U_s[k][j + 1];
+                const float2 f = kSeq ? mf[kSeq ? k : 0] : elem(k);
+                gt_fma2x2(h0, l0, gt_dup(f.x), gt_dup(f.y), make_float2(u0.x, u0.y), make_float2(u0.z, u0.w));
+                gt_fma2x2(h1, l1, gt_dup(f.x), gt_dup(f.y), make_float2(u1.x, u1.y), make_float2(u1.z, u1.w));
+                if (kSeq && any_piv && my_k == k) {       // the pivot row of step k becomes prow_k
+                    h0 = make_float2(u0.x, u0.y); l0 = make_float2(u0.z, u0.w);
+                    h1 = make_float2(u1.x, u1.y); l1 = make_float2(u1.z, u1.w);
+                }
+            }
+            row[j] = make_float4(h0.x, h0.y, l0.x, l0.y);
+            row[j + 1] = make_float4(h1.x, h1.y, l1.x, l1.y);
+        }
+        // the registers change places with the next sub-panel's columns: area sb of the row (4 column
+        // pairs) then holds this one's
+        if (sb < kGtB / kGpSub - 1) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 v = row[4 * sb + q];
+                row[4 * sb + q] = make_float4(xh[q].x, xh[q].y, xl[q].x, xl[q].y);
+                xh[q] = make_float2(v.x, v.y);
+                xl[q] = make_float2(v.z, v.w);
+            }
+        }
     }
     if (sing) {
         if (t == 0) st->sing = 1;
         return;
     }
-    // the eliminated panel is part of the result; bookkeeping of the pivots
+    // a short last panel leaves the loop early: the areas from its last sub-panel on still hold
+    // the columns after it, in order; those columns are all zero and not stored
+    const int last = min((w + kGpSub - 1) / kGpSub, kGtB / kGpSub) - 1;      // last sub-panel eliminated
+    const int swaps = min(last + 1, kGtB / kGpSub - 1);
+    // column pair q of the panel: area q / 4 before the swaps' end, the registers after
+    auto pair_at = [&](int q) {
+        const int g = q >> 2;
+        if (g < swaps) return row[q];
+        if (g == swaps) return make_float4(xh[q & 3].x, xh[q & 3].y, xl[q & 3].x, xl[q & 3].y);
+        return row[q - 4];
+    };
+    // the eliminated panel is part of the result; operand A: the row scaled by its exponent, seven
+    // slices, [row tile][slice] planes, 16-byte chunks of 8 columns
     if (row_ok) {
-        if (w == kGtB) {
-            float4 *dst = reinterpret_cast<float4 *>(Wk + (size_t)i * ld + jb);
+        float mx = 0.f;
+        float2 *dst = Wk + (size_t)i * ld + jb;
 #pragma unroll
-            for (int q = 0; q < kGtB / 2; ++q)
-                dst[q] = make_float4(row[2 * q].x, row[2 * q].y, row[2 * q + 1].x, row[2 * q + 1].y);
-        } else {
-            for (int j = 0; j < w; ++j) Wk[(size_t)i * ld + jb + j] = row[j];
+        for (int q = 0; q < kGtB / 2; ++q) {
+            const float4 v = pair_at(q);
+            mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
+            if (w == kGtB) *reinterpret_cast<float4 *>(dst + 2 * q) = make_float4(v.x, v.z, v.y, v.w);
+            else {
+                if (2 * q < w) dst[2 * q] = make_float2(v.x, v.z);
+                if (2 * q + 1 < w) dst[2 * q + 1] = make_float2(v.y, v.w);
+            }
+        }
+        const int E = exp_bound(mx);
+        reinterpret_cast<int *>(sc + L.e)[i] = E;
+        unsigned char *base = sc + L.a + (size_t)(i >> 7) * kGtSl * kGtAPlane;
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+            uint32_t o[kGtSl][4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 v = pair_at(4 * ch + q);
+                float s0[kGtSl], s1[kGtSl];
+                slice_n<kGtSl>(make_float2(v.x, v.z), E, s0);
+                slice_n<kGtSl>(make_float2(v.y, v.w), E, s1);
+#pragma unroll
+                for (int j = 0; j < kGtSl; ++j) o[j][q] = bf16_pair(s0[j], s1[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < kGtSl; ++j)
+                *reinterpret_cast<uint4 *>(base + (size_t)j * kGtAPlane + a_off64(i & 127, ch)) =
+                    make_uint4(o[j][0], o[j][1], o[j][2], o[j][3]);
         }
     }
+    // bookkeeping of the pivots
     if (t < w) {
         const int p = ppS[t];
         pp_g[jb + t] = (short)p;
         used_g[p] = 1;
         piv_g[p] = 1;
     }
-    if (t == 0) {
+    if (t == (int)blockDim.x - 32) {
         GtState o = *st;
         o.mag_h = S.mag_h; o.mag_l = S.mag_l; o.mag_e = S.mag_e; o.neg = S.neg;
         *st = o;
-    }
-    __syncthreads();
-    // operand A: the panel's rows, scaled per row, seven slices, [row tile][slice] planes
-    // (a warp per row, lane = column)
-    for (int r = wid; r < n; r += nwarps) {
-        const float2 xr = P[(size_t)r * kGpRowLd + lane];
-        float mx = fabsf(xr.x);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        const int E = exp_bound(mx);
-        float s7[kGtSl];
-        slice_n<kGtSl>(xr, E, s7);
-        unsigned char *base = Apl + (size_t)(r >> 7) * kGtSl * kGtAPlane + a_off64(r & 127, lane >> 3) +
-                              (lane & 7) * 2;
-#pragma unroll
-        for (int j = 0; j < kGtSl; ++j)
-            *reinterpret_cast<__nv_bfloat16 *>(base + (size_t)j * kGtAPlane) = __float2bfloat16_rn(s7[j]);
-        if (lane == 0) Erow[r] = E;
     }
     gt_operand_b(sc, L, n, jb, w, ppS);
 }
@@ -1092,20 +1043,17 @@ cudaError_t launch_gj_tc(const GjJob *jobs, int n_jobs, void *scratch, cudaStrea
     js.expire_m = (wc.expire_kernels & QMC_EXPIRE_A4) ? wc.expire_w : -1;
     if (cmax == 0 || n_jobs == 0) return cudaSuccess;
     if (!gjtc_fits(nmax)) return cudaErrorInvalidConfiguration;
-    const size_t sm_panel = sizeof(float2) * (size_t)nmax * kGtB + sizeof(short) * (size_t)nmax;
     // 56 KB of panel slices, 3 x 14 KB of pivot-row slices, 3 x 32 KB of old values, the
     // column exponents: one CTA per SM
     const size_t sm_up = 1024 + kGtSl * (size_t)(kGtAPlane + kGtBs * kGtBPlane) + kGtXs * (size_t)kGtXStage +
                          8 * (size_t)((nmax + kGtN - 1) / kGtN * kGtN);
     cudaError_t e;
     if ((e = gt_tensor_maps(js)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_gt_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_panel)) !=
-        cudaSuccess)
-        return e;
-    const int nthr_t = (nmax + 31) / 32 * 32;
-    const size_t sm_t = sizeof(float2) * (size_t)nthr_t * kGpRowLd;
-    if (nmax <= kGpRowMax &&
-        (e = cudaFuncSetAttribute(k_gt_panel_t, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_t)) != cudaSuccess)
+    const int nthr = (nmax + 31) / 32 * 32;
+    const size_t sm_panel = sizeof(float4) * (size_t)nthr * kGpLd;
+    // one thread per row; the register budget follows the block
+    auto panel = nmax < kGtSeqMin ? k_gt_panel<544, false> : (nthr <= 896 ? k_gt_panel<896, true> : k_gt_panel<1024, true>);
+    if ((e = cudaFuncSetAttribute(panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_panel)) != cudaSuccess)
         return e;
     if ((e = cudaFuncSetAttribute(k_gt_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_up)) !=
         cudaSuccess)
@@ -1116,9 +1064,7 @@ cudaError_t launch_gj_tc(const GjJob *jobs, int n_jobs, void *scratch, cudaStrea
     const int nz = cmax * n_jobs;
     for (int jb = 0; jb < nmax; jb += kGtB) {
         js.jb = jb;
-        // one thread per row where the rows fit one CTA, else the panel in shared memory
-        if (nmax <= kGpRowMax) k_gt_panel_t<<<g1, nthr_t, sm_t, st>>>(js);
-        else k_gt_panel<<<g1, kGpThreads, sm_panel, st>>>(js);
+        panel<<<g1, nthr, sm_panel, st>>>(js);
         for (int z0 = 0; z0 < nz; z0 += 65535) {
             const int zn = nz - z0 < 65535 ? nz - z0 : 65535;
             k_gt_update<<<dim3(nt, 1, zn), kGtUpThreads, sm_up, st>>>(js, z0);

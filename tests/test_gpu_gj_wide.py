@@ -75,3 +75,30 @@ def test_float_float_inverse(key, W, panel):
         assert (out["logabs"][sample.to(dev), sp] - logabs).abs().max().item() < 1e-6
         E = D.mT @ C1 - torch.eye(n, dtype=torch.float64, device=dev)
         assert E.abs().max().item() < 1e-6
+
+
+@pytest.mark.parametrize("n_up_plus", [31, 32, 33, 63, 65, 127, 129, 160, 543, 545, 577, 865])
+def test_tensor_panel_sizes(n_up_plus):
+    """The panel kernel of the tensor-core elimination at the edges of its sub-panels (short last
+    panels), of its warps and of its two arithmetics (544 / 545 rows): log|det| against the FP64 path
+    within 1e-6 and the inverse's residual within 1e-6 on every walker."""
+    from paper_1209_6630_gb300 import QmcSystem, det_inverse
+    from synth import make_system, make_walkers
+    n = n_up_plus
+    heavy = max(2, (2 * n) // 9)
+    s = make_system(heavy, 0, 0, 2 * n - 6 * heavy, seed=100 + n)      # 2 n electrons
+    assert s.n_up == n
+    q = QmcSystem(s, 0)
+    q.set_tiles(a4_mode="tensor", c15_mode="tensor")
+    R = torch.from_numpy(make_walkers(s, 3, first=95000)).to(dev)
+    out = q.eval(R, precision="mixed", want_dinv=True)
+    assert (out["status"] == 0).all()
+    for sp, C in enumerate(q.slater(R, precision="mixed")):
+        m = C.shape[-1]
+        off = s.n_up ** 2 if sp else 0
+        D = out["dinv"][:, off: off + m * m].reshape(-1, m, m)
+        C1 = C[:, 0].contiguous()
+        logabs = det_inverse(C1.clone())[0]
+        assert (out["logabs"][:, sp] - logabs).abs().max().item() < 1e-6
+        E = D.mT @ C1 - torch.eye(m, dtype=torch.float64, device=dev)
+        assert E.abs().max().item() < 1e-6
