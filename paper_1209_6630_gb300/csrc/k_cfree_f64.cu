@@ -22,175 +22,26 @@
 // (158 electrons x 100: 4.6 -> 1.1 + 1.4 ms)
 #include <algorithm>
 
-#include "qmc_device.cuh"
+#include "c1_f64.cuh"
 
 namespace qmc {
 
 namespace {
 
-constexpr int kCfThreads = 128;
-constexpr int kCfShells = kCfThreads;                  // shells per chunk, one per thread
-
-// Shared memory of a CTA: the active shells (for the whole electron), then one chunk's tables.
-struct CfSmem {
-    unsigned short *sh;            // [n_shell] active shells, ascending
-    double *ex;                    // [kCfShells * kMaxPrim] exp(-gamma_p d2), by shell, in order
-    double *d2;                    // [kCfShells]
-    double *last;                  // [max AOs of a chunk] values (k_c1_f64), or [n_s] a row of D^-1 (k_vd_f64)
-    int *ao;                       // [max AOs of a chunk] AO indices
-    unsigned char *p_sh, *a_sh;    // chunk-local shell of each primitive / AO
-};
-
-__host__ __device__ inline int cf_max_ao(const SysDev &s) { return min(kCfShells * ncart(kMaxL), s.n_ao); }
-
-__host__ __device__ inline size_t cf_smem(const SysDev &s)
-{
-    const size_t na = cf_max_ao(s);
-    const size_t b = 8 * ((size_t)kCfShells * kMaxPrim + kCfShells) + 4 * na + 2 * (size_t)s.n_shell +
-                     (size_t)kCfShells * kMaxPrim + na;
-    return (b + 15) / 16 * 16;                           // (the doubles of `last` follow)
-}
-
-__device__ inline CfSmem cf_carve(const SysDev &s, unsigned char *base)
-{
-    const int na = cf_max_ao(s);
-    CfSmem c;
-    c.ex = reinterpret_cast<double *>(base);
-    c.d2 = c.ex + kCfShells * kMaxPrim;
-    c.ao = reinterpret_cast<int *>(c.d2 + kCfShells);
-    c.sh = reinterpret_cast<unsigned short *>(c.ao + na);
-    c.p_sh = reinterpret_cast<unsigned char *>(c.sh + s.n_shell);
-    c.a_sh = c.p_sh + kCfShells * kMaxPrim;
-    c.last = reinterpret_cast<double *>(base + cf_smem(s));
-    return c;
-}
-
-// The active shells of an electron at r, ascending, into sh (the decisions of screen_electron).
-__device__ int cf_screen(const SysDev &s, double rx, double ry, double rz, unsigned short *sh_s, int *warp_s)
-{
-    const int t = threadIdx.x;
-    const int per = (s.n_shell + kCfThreads - 1) / kCfThreads;   // <= 64, checked at load
-    const int sh0 = min(t * per, s.n_shell), sh1 = min(sh0 + per, s.n_shell);
-    unsigned long long mask = 0ull;
-    int last_a = -1;
-    bool atom_in = false;
-    double d2 = 0.0;
-    for (int sh = sh0; sh < sh1; ++sh) {
-        const int a = s.sh_atom[sh];
-        if (a != last_a) {
-            last_a = a;
-            d2 = sqdist_rn(rx, ry, rz, s.Q + 3 * a);
-            atom_in = d2 < s.atom_R2[a];
-        }
-        if (atom_in && d2 < s.sh_R2[sh]) mask |= 1ull << (sh - sh0);
-    }
-    int total;
-    int off = block_excl_scan<kCfThreads>(__popcll(mask), warp_s, &total);
-    for (; mask; mask &= mask - 1) sh_s[off++] = (unsigned short)(sh0 + __ffsll((long long)mask) - 1);
-    __syncthreads();
-    return total;
-}
-
-// Tables of the chunk of shells from q0: returns its AO count; this thread's shell in `my` (-1:
-// none), its first primitive of ex in `pofs`.  ex holds the primitives' exponentials on return.
-__device__ int cf_chunk(const SysDev &s, const CfSmem &c, int q0, int n_act, double rx, double ry, double rz,
-                        int *warp_s, int &my, int &pofs)
-{
-    const int t = threadIdx.x;
-    my = q0 + t < n_act ? c.sh[q0 + t] : -1;
-    int nc = 0, np = 0, p0 = 0;
-    if (my >= 0) {
-        nc = ncart(s.sh_L[my]);
-        np = s.sh_nprim[my];
-        p0 = s.sh_pstart[my];
-        const double *q = s.Q + 3 * s.sh_atom[my];
-        c.d2[t] = sqdist_rn(rx, ry, rz, q);
-    }
-    int total;                                           // AOs in the low half, primitives in the high half
-    const int off = block_excl_scan<kCfThreads>(nc | np << 16, warp_s, &total);
-    pofs = off >> 16;
-    for (int i = 0; i < nc; ++i) {
-        c.ao[(off & 0xffff) + i] = s.sh_ao0[my] + i;
-        c.a_sh[(off & 0xffff) + i] = (unsigned char)t;
-    }
-    for (int i = 0; i < np; ++i) {
-        c.p_sh[pofs + i] = (unsigned char)t;
-        reinterpret_cast<int *>(c.ex + pofs + i)[0] = p0 + i;    // the primitive, until its exponential replaces it
-    }
-    __syncthreads();
-    const int ntp = total >> 16;
-    for (int i = t; i < ntp; i += kCfThreads) {
-        const int p = reinterpret_cast<const int *>(c.ex + i)[0];
-        c.ex[i] = exp(-s.pg[p] * c.d2[c.p_sh[i]]);
-    }
-    __syncthreads();
-    return total & 0xffff;
-}
-
 template <int NJ>
 __global__ void __launch_bounds__(kCfThreads) k_c1_f64(SysDev s, const double *__restrict__ R, double *__restrict__ X)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const CfSmem c = cf_carve(s, smem_raw);
     __shared__ int warp_s[kCfThreads / 32];
     __shared__ double g_s[kCfShells];
-
-    const int e = blockIdx.x, w = blockIdx.y, t = threadIdx.x;
+    const int e = blockIdx.x, w = blockIdx.y;
     const int spin = e >= s.n_up;
     const int ei = spin ? e - s.n_up : e;
     const int ns = spin ? s.n_dn : s.n_up;
-    const double *__restrict__ A = s.A64[spin];
     const double *r = R + ((size_t)w * s.n_elec + e) * 3;
-    const double rx = r[0], ry = r[1], rz = r[2];
-    const int n_act = cf_screen(s, rx, ry, rz, c.sh, warp_s);
-
-    double acc[NJ];
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) acc[j] = 0.0;
-    const int kwarp = t & ~31;
-    for (int q0 = 0; q0 < n_act; q0 += kCfShells) {
-        int my, pofs;
-        const int nao = cf_chunk(s, c, q0, n_act, rx, ry, rz, warp_s, my, pofs);
-        if (my >= 0) {
-            double g = 0.0;
-            const int np = s.sh_nprim[my], p0 = s.sh_pstart[my];
-            for (int p = 0; p < np; ++p) g = __dadd_rn(g, __dmul_rn(s.pc[p0 + p], c.ex[pofs + p]));
-            g_s[t] = g;
-        }
-        __syncthreads();
-        for (int m = t; m < nao; m += kCfThreads) {
-            const int mu = c.ao[m], sl = c.a_sh[m];
-            const double *q = s.Q + 3 * s.sh_atom[c.sh[q0 + sl]];
-            const int pw = s.ao_pow[mu];
-            const double P = ipow_small(rx - q[0], pw & 255) * ipow_small(ry - q[1], (pw >> 8) & 255) *
-                             ipow_small(rz - q[2], (pw >> 16) & 255);
-            c.last[m] = s.ao_scale[mu] * P * g_s[sl];
-        }
-        __syncthreads();
-        // MO slots j whose whole warp lies beyond ns are skipped (warp-uniform)
-#pragma unroll 4
-        for (int m = 0; m < nao; ++m) {
-            const double *__restrict__ arow = A + (size_t)c.ao[m] * ns;
-            const double b = c.last[m];
-            double a[NJ];
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int k = t + kCfThreads * j;
-                a[j] = (k < ns) ? __ldg(arow + k) : 0.0;
-            }
-#pragma unroll
-            for (int j = 0; j < NJ; ++j)
-                if (kwarp + kCfThreads * j < ns) acc[j] = fma(a[j], b, acc[j]);
-        }
-        __syncthreads();
-    }
     const size_t msz = (size_t)s.n_up * s.n_up + (size_t)s.n_dn * s.n_dn;
-    double *xrow = X + (size_t)w * msz + (spin ? (size_t)s.n_up * s.n_up : 0) + (size_t)ei * ns;
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-        const int k = t + kCfThreads * j;
-        if (k < ns) xrow[k] = acc[j];
-    }
+    c1_row_f64<NJ, false>(s, cf_carve(s, smem_raw), g_s, warp_s, spin, r[0], r[1], r[2],
+                          X + (size_t)w * msz + (spin ? (size_t)s.n_up * s.n_up : 0) + (size_t)ei * ns);
 }
 
 // Eight lanes' eight partial sums each: lane l of the group of 8 is left the total of sum l.
@@ -311,8 +162,6 @@ __global__ void __launch_bounds__(kCfThreads) k_vd_f64(SysDev s, const double *_
     __syncthreads();
     if (t < 4) vd[((size_t)w * s.n_elec + e) * 4 + t] = ((red[0][t] + red[1][t]) + red[2][t]) + red[3][t];
 }
-
-size_t c1_smem(const SysDev &s) { return cf_smem(s) + 8 * (size_t)cf_max_ao(s); }
 
 size_t vd_smem(const SysDev &s) { return cf_smem(s) + 8 * (size_t)(s.n_up > s.n_dn ? s.n_up : s.n_dn); }
 

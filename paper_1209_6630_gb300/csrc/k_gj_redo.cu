@@ -26,6 +26,7 @@
 
 #include <algorithm>
 
+#include "c1_f64.cuh"
 #include "gj_panel.cuh"
 #include "qmc_device.cuh"
 
@@ -312,59 +313,52 @@ __global__ void __cluster_dims__(kFinalCluster, 1, 1) __launch_bounds__(kRThread
 // C1 rows of every listed matrix recomputed in FP64 (exact screening, FP64 AO
 // values and products): near a nodal surface the mixed-precision C1 (~2^-40
 // normwise) perturbs log|det| by up to kappa times that.  Each CTA computes
-// one row (blockIdx.x) of every 32nd listed matrix; thread t owns MO columns
-// t, t + 128, ...
-constexpr int kC1Threads = 128;
-constexpr int kC1Chunk = 512;
+// one row (blockIdx.x) of every 32nd listed matrix.
+// (c1_f64.cuh: at 434 electrons x 4096 walkers, ~230 listed matrices, 8.5 -> 2.2 ms; before, every AO
+// evaluated its own exponentials, a core shell's eight among the others' one to three.)
+constexpr int kC1Slots = 32;   // CTAs per row; each loops over the listed matrices
 
-__device__ __forceinline__ void redo_c1_row(const SysDev &s, const RedoArgs &a, const double *__restrict__ R, int b)
+template <int NJ>
+__global__ void __launch_bounds__(kCfThreads) k_redo_c1(SysDev s, RedoArgs a, const double *__restrict__ R)
 {
-    const RedoEntry en = a.list->e[b];
-    const GjJob &J = a.j[en.job];
-    const int n = J.n, i = blockIdx.x;
-    if (i >= n) return;
-    const int e = a.e_off[en.job] + i;
-    const int spin = e >= s.n_up;
-    const double *__restrict__ A = s.A64[spin];
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *b_s = reinterpret_cast<double *>(smem_raw);             // [kC1Chunk]
-    int *idx_s = reinterpret_cast<int *>(b_s + kC1Chunk);            // [n_ao]
-    __shared__ int warp_s[kC1Threads / 32];
-    const double *r = R + ((size_t)en.m * s.n_elec + e) * 3;
-    const double rx = r[0], ry = r[1], rz = r[2];
-    const int K = screen_electron<kC1Threads>(s, rx, ry, rz, idx_s, s.n_ao, warp_s);
-    double *__restrict__ Xrow = J.X + (size_t)en.m * J.x_stride + (size_t)i * n;
-    constexpr int kMaxCols = 1024 / kC1Threads;
-    double acc[kMaxCols];
-#pragma unroll
-    for (int j = 0; j < kMaxCols; ++j) acc[j] = 0.0;
-    for (int k0 = 0; k0 < K; k0 += kC1Chunk) {
-        const int kc = min(kC1Chunk, K - k0);
-        for (int q = threadIdx.x; q < kc; q += kC1Threads) b_s[q] = ao_value_f64(s, idx_s[k0 + q], rx, ry, rz);
-        __syncthreads();
-        for (int q = 0; q < kc; ++q) {
-            const double bv = b_s[q];
-            const double *Arow = A + (size_t)idx_s[k0 + q] * n;
-#pragma unroll
-            for (int j = 0; j < kMaxCols; ++j) {
-                const int k = threadIdx.x + kC1Threads * j;
-                if (k < n) acc[j] = fma(bv, Arow[k], acc[j]);
-            }
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < kMaxCols; ++j) {
-        const int k = threadIdx.x + kC1Threads * j;
-        if (k < n) Xrow[k] = acc[j];
+    __shared__ int warp_s[kCfThreads / 32];
+    __shared__ double g_s[kCfShells];
+    for (int b = blockIdx.y; b < a.list->count; b += kC1Slots) {
+        const RedoEntry en = a.list->e[b];
+        const GjJob &J = a.j[en.job];
+        const int n = J.n, i = blockIdx.x;
+        if (i >= n) continue;
+        const int e = a.e_off[en.job] + i;
+        const double *r = R + ((size_t)en.m * s.n_elec + e) * 3;
+        __syncthreads();                                   // the previous row's tables
+        c1_row_f64<NJ, true>(s, cf_carve(s, smem_raw), g_s, warp_s, e >= s.n_up, r[0], r[1], r[2],
+                             J.X + (size_t)en.m * J.x_stride + (size_t)i * n);
     }
 }
 
-constexpr int kC1Slots = 32;   // CTAs per row; each loops over the listed matrices
-
-__global__ void __launch_bounds__(kC1Threads) k_redo_c1(SysDev s, RedoArgs a, const double *__restrict__ R)
+template <int NJ>
+static cudaError_t launch_redo_c1(const SysDev &s, const RedoArgs &a, int nmax, const double *R, cudaStream_t st)
 {
-    for (int b = blockIdx.y; b < a.list->count; b += kC1Slots) redo_c1_row(s, a, R, b);
+    const size_t sm = c1_smem(s);
+    cudaError_t e = cudaFuncSetAttribute(k_redo_c1<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    k_redo_c1<NJ><<<dim3(nmax, kC1Slots), kCfThreads, sm, st>>>(s, a, R);
+    return cudaGetLastError();
+}
+
+static cudaError_t launch_redo_c1(const SysDev &s, const RedoArgs &a, int nmax, const double *R, cudaStream_t st)
+{
+    switch ((nmax + kCfThreads - 1) / kCfThreads) {
+    case 1: return launch_redo_c1<1>(s, a, nmax, R, st);
+    case 2: return launch_redo_c1<2>(s, a, nmax, R, st);
+    case 3: return launch_redo_c1<3>(s, a, nmax, R, st);
+    case 4: return launch_redo_c1<4>(s, a, nmax, R, st);
+    case 5: return launch_redo_c1<5>(s, a, nmax, R, st);
+    case 6: return launch_redo_c1<6>(s, a, nmax, R, st);
+    case 7: return launch_redo_c1<7>(s, a, nmax, R, st);
+    default: return launch_redo_c1<8>(s, a, nmax, R, st);
+    }
 }
 
 template <int NB>
@@ -445,11 +439,7 @@ cudaError_t launch_gj_redo(const GjJob *jobs, int n_jobs, void *scratch, cudaStr
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (R && s) {
-        const size_t sm = sizeof(double) * kC1Chunk + sizeof(int) * (size_t)s->n_ao;
-        if ((e = cudaFuncSetAttribute(k_redo_c1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
-            return e;
-        k_redo_c1<<<dim3(nmax, kC1Slots), kC1Threads, sm, st>>>(*s, a, R);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_redo_c1(*s, a, nmax, R, st)) != cudaSuccess) return e;
     }
     e = launch_redo_nb(a, nmax, st, nb);
     if (e != cudaSuccess) return e;
