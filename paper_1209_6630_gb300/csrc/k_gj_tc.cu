@@ -255,6 +255,14 @@ __device__ __forceinline__ void gt_fma2x2(float2 &ah, float2 &al, float2 xh, flo
     al = __fadd2_rn(se, gt_neg2(__fadd2_rn(ah, gt_neg2(s))));
 }
 
+// ff::two_sum for two values at once
+__device__ __forceinline__ void gt_two_sum2(float2 a, float2 b, float2 &s, float2 &e)
+{
+    s = __fadd2_rn(a, b);
+    const float2 bb = __fadd2_rn(s, gt_neg2(a));
+    e = __fadd2_rn(__fadd2_rn(a, gt_neg2(__fadd2_rn(s, gt_neg2(bb)))), __fadd2_rn(b, gt_neg2(bb)));
+}
+
 __device__ __forceinline__ float2 gt_dup(float x) { return make_float2(x, x); }
 
 // The panel kernel: one thread per row.  The 32 columns are eliminated in four sub-panels of 8,
@@ -795,6 +803,13 @@ __global__ void __launch_bounds__(kGtUpThreads, 1) k_gt_update(const __grid_cons
             }
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (quad * 32 >= nr) {                               // a ragged tile's warp without rows
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bTE);
+                if (!gt_wait_warp(XF(sx), (i / kGtXs) & 1, js.wait_ns, &s_abort, lane)) break;
+                if (lane == 0) mbar_arrive(XW(sx));
+                continue;
+            }
             uint32_t v[kGtSl][8];
 #pragma unroll
             for (int d = 0; d < kGtSl; ++d) tmem_ld8_async(tl + (uint32_t)(d * kGtN), v[d]);
@@ -803,50 +818,48 @@ __global__ void __launch_bounds__(kGtUpThreads, 1) k_gt_update(const __grid_cons
             __syncwarp();
             if (lane == 0) mbar_arrive(bTE);
             // the seven order sums, exact integers in their units: orders 0..3 added as float
-            // pairs, orders 4..6 (below 2^-21 of the update) first in FP32 (rounding ~2^-46)
-            float hs[8], ls[8];
+            // pairs, orders 4..6 (below 2^-21 of the update) first in FP32 (rounding ~2^-46);
+            // two columns at a time (packed FP32)
+            float2 hs[4], ls[4];
+            auto ord = [&](int d, int k) { return make_float2(__uint_as_float(v[d][2 * k]), __uint_as_float(v[d][2 * k + 1])); };
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                ff::two_sum(__uint_as_float(v[0][k]), __uint_as_float(v[1][k]), hs[k], ls[k]);
-                float sh, se;
-                ff::two_sum(hs[k], __uint_as_float(v[2][k]), sh, se);
-                ls[k] = __fadd_rn(ls[k], se);
-                ff::two_sum(sh, __uint_as_float(v[3][k]), hs[k], se);
-                ls[k] = __fadd_rn(ls[k], se);
-                const float t456 = __fadd_rn(__uint_as_float(v[4][k]),
-                                             __fadd_rn(__uint_as_float(v[5][k]), __uint_as_float(v[6][k])));
-                ls[k] = __fadd_rn(ls[k], t456);
+            for (int k = 0; k < 4; ++k) {
+                float2 sh, se;
+                gt_two_sum2(ord(0, k), ord(1, k), hs[k], ls[k]);
+                gt_two_sum2(hs[k], ord(2, k), sh, se);
+                ls[k] = __fadd2_rn(ls[k], se);
+                gt_two_sum2(sh, ord(3, k), hs[k], se);
+                ls[k] = __fadd2_rn(ls[k], se);
+                ls[k] = __fadd2_rn(ls[k], __fadd2_rn(ord(4, k), __fadd2_rn(ord(5, k), ord(6, k))));
             }
             if (!gt_wait_warp(XF(sx), (i / kGtXs) & 1, js.wait_ns, &s_abort, lane)) break;
             unsigned char *xs = Xs + sx * kGtXStage + xoff;
             const int ct = col_tile(i);
             const int c0 = ct * kGtN + cg * 8;
-            if (E_ok && tile_ok[ct]) {
+            const bool fast = E_ok && tile_ok[ct];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    float4 *p4 = reinterpret_cast<float4 *>(xs + (((ck0 + k) ^ (r & 7)) << 4));
-                    const float4 o = *p4;
-                    float2 x0 = is_piv ? make_float2(0.f, 0.f) : make_float2(o.x, o.y);
-                    float2 x1 = is_piv ? make_float2(0.f, 0.f) : make_float2(o.z, o.w);
-                    const float f0 = Fsc[c0 + 2 * k], f1 = Fsc[c0 + 2 * k + 1];
-                    x0 = ff::add(x0, make_float2(__fmul_rn(__fmul_rn(hs[2 * k], sE), f0),
-                                                 __fmul_rn(__fmul_rn(ls[2 * k], sE), f0)));
-                    x1 = ff::add(x1, make_float2(__fmul_rn(__fmul_rn(hs[2 * k + 1], sE), f1),
-                                                 __fmul_rn(__fmul_rn(ls[2 * k + 1], sE), f1)));
-                    *p4 = make_float4(x0.x, x0.y, x1.x, x1.y);
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    float4 *p4 = reinterpret_cast<float4 *>(xs + (((ck0 + k) ^ (r & 7)) << 4));
-                    const float4 o = *p4;
-                    float2 x0 = is_piv ? make_float2(0.f, 0.f) : make_float2(o.x, o.y);
-                    float2 x1 = is_piv ? make_float2(0.f, 0.f) : make_float2(o.z, o.w);
+            for (int k = 0; k < 4; ++k) {
+                float4 *p4 = reinterpret_cast<float4 *>(xs + (((ck0 + k) ^ (r & 7)) << 4));
+                float4 o = *p4;
+                if (is_piv) o = make_float4(0.f, 0.f, 0.f, 0.f);
+                float2 uh, ul;
+                if (fast) {
+                    const float2 f = *reinterpret_cast<const float2 *>(Fsc + c0 + 2 * k), e2 = gt_dup(sE);
+                    uh = __fmul2_rn(__fmul2_rn(hs[k], e2), f);
+                    ul = __fmul2_rn(__fmul2_rn(ls[k], e2), f);
+                } else {
                     const int ex0 = E + Fs[c0 + 2 * k], ex1 = E + Fs[c0 + 2 * k + 1];
-                    x0 = ff::add(x0, make_float2(scale_pow2(hs[2 * k], ex0), scale_pow2(ls[2 * k], ex0)));
-                    x1 = ff::add(x1, make_float2(scale_pow2(hs[2 * k + 1], ex1), scale_pow2(ls[2 * k + 1], ex1)));
-                    *p4 = make_float4(x0.x, x0.y, x1.x, x1.y);
+                    uh = make_float2(scale_pow2(hs[k].x, ex0), scale_pow2(hs[k].y, ex1));
+                    ul = make_float2(scale_pow2(ls[k].x, ex0), scale_pow2(ls[k].y, ex1));
                 }
+                // ff::add of the old values and the update
+                const float2 xh = make_float2(o.x, o.z), xl = make_float2(o.y, o.w);
+                float2 sm, e;
+                gt_two_sum2(xh, uh, sm, e);
+                e = __fadd2_rn(e, __fadd2_rn(xl, ul));
+                const float2 h = __fadd2_rn(sm, e);
+                const float2 l = __fadd2_rn(e, gt_neg2(__fadd2_rn(h, gt_neg2(sm))));
+                *p4 = make_float4(h.x, l.x, h.y, l.y);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // for the TMA store
             __syncwarp();
