@@ -44,9 +44,10 @@
 
 namespace qmc {
 
-constexpr int kBtThreads = 256;
+constexpr int kBtThreads = 512;
+constexpr int kBtScanThreads = 256;                 // threads that test pairs (their order sets the order of the sums)
 constexpr int kBtHits = 64;                         // hits per stage (K of one stage)
-constexpr int kBtScan = 4 * kBtThreads;             // pairs tested per scan round
+constexpr int kBtScan = 4 * kBtScanThreads;             // pairs tested per scan round
 constexpr int kBtPend = kBtHits + kBtScan;
 constexpr int kBtSlices = 3;
 constexpr int kBtABufs = 3;
@@ -211,10 +212,10 @@ __global__ void __launch_bounds__(kBtThreads, 1) k_bw_mma(BwTcArgs a)
             int code[4], hit[4], cnt = 0;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const int p = scan_pos + i * kBtThreads + t;
+                const int p = scan_pos + i * kBtScanThreads + t;
                 hit[i] = 0;
                 code[i] = 0;
-                if (p < npairs) {
+                if (t < kBtScanThreads && p < npairs) {
                     const int wl = p / ns, e = p - wl * ns;
                     const int w = w_lo + wl;
                     if (a.g[w] != 0.0) {
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(kBtThreads, 1) k_bw_mma(BwTcArgs a)
         return n;
     };
 
-    // X slice planes of stage buffer sb: four threads per hit, shells of the block split four ways
+    // X slice planes of stage buffer sb: eight threads per hit, shells of the block split eight ways
     auto produce_x = [&](int sb, int nh) {
         unsigned char *xb = xbuf + (size_t)sb * kBtSlices * xplane;
         const int h = t & (kBtHits - 1), q = t >> 6;
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(kBtThreads, 1) k_bw_mma(BwTcArgs a)
     // The A copies of a thread: 16-byte chunk t % 16 of rows (hits) t / 16 + 16 i, i < 4, of each
     // slice plane.  The rows' addresses are formed once per stage (formed anew for every copy they
     // were most of the kernel's instructions, with 8 warps to hide them: 57.6 -> 40.2 ms at 1731
-    // electrons x 512 walkers).
+    // electrons x 512 walkers; with 16 warps 34.9).
     constexpr int kRows = kBtHits * (TC_N / 8) / kBtThreads;
     const int ac = t % (TC_N / 8);
     const uint16_t *arow[kRows];
@@ -425,7 +426,7 @@ __global__ void __launch_bounds__(kBtThreads, 1) k_bw_mma(BwTcArgs a)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int quad = warp & 3;
     for (int tile = 0; tile < kts; ++tile)
-        for (int cb = (warp >> 2) * 32; cb < a.nb; cb += 64) {
+        for (int cb = (warp >> 2) * 32; cb < a.nb; cb += kBtThreads / 4) {
             uint32_t v[32];
             if (ncommit > 0 && ok) tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(tile * a.nb + cb), v);
             const int k = tile * TC_N + quad * 32 + lane;
