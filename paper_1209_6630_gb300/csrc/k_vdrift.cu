@@ -220,11 +220,10 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
     const uint32_t mb = smem_u32(&mbar);
-    const uint32_t idesc = umma_idesc_f16_major(TC_M, kVdN, 1, 0, 0);   // BF16, A and B K-major
     const uint64_t kWait = a.wait_ns;
     const uint16_t *Bsl = a.rslice[spin];
     const size_t bstride = (size_t)s.n_ao * nspad;
-    const int nst = nspad / kVdK;
+    const int nst = (ns + kVdK - 1) / kVdK;               // (the padding beyond is zeros)
 
     // this CTA's D^-1 rows cut into six exact slices once, for every K stage (the AO tiles
     // reuse them): thread -> (row, chunk of 8 MOs), two per thread
@@ -290,6 +289,8 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
         const int bmu = ao_s[at * kVdN + (t >> 2)];
         const uint16_t *bsrc = Bsl + (size_t)max(bmu, 0) * nspad + 8 * (t & 3);
         const uint32_t bdst = smem_u32(Bb + a_off64(t >> 2, t & 3));
+        const int ncol = min(kVdN, (K - at * kVdN + 15) / 16 * 16);              // N of the tile's MMAs
+        const uint32_t idesc = umma_idesc_f16_major(TC_M, ncol, 1, 0, 0);        // BF16, A and B K-major
         for (int sg = 0; sg < nst; ++sg) {
             // the stage buffer: A (the staged D^-1 slices) and B (the rows of A of this AO tile)
             const int k0 = sg * kVdK;
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
             }
 #pragma unroll
             for (int j = 0; j < kC15Slices; ++j)
-                cp_async16(bdst + j * kVdBPlane, bsrc + j * bstride + k0, bmu >= 0);
+                if ((t >> 2) < ncol) cp_async16(bdst + j * kVdBPlane, bsrc + j * bstride + k0, bmu >= 0);
             asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 0;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
