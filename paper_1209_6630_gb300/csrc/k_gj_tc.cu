@@ -70,7 +70,7 @@ constexpr int kGtBs = 3;                             // stages of pivot-row slic
 constexpr int kGtXs = 3;                             // stages of old values
 constexpr uint32_t kGtXStage = 128 * kGtN * 8;       // [2 halves][128 rows][16 float pairs], 128-byte swizzle
 constexpr uint32_t kGtATmem = 256;                   // TMEM: 7 accumulators of 32 columns at 0, the panel
-                                                     // slices (7 x 16 columns) from 256
+constexpr uint32_t kGtAtCols = kGtSl * 16;           // slices (7 x 16 columns) of two row tiles from 256
 
 // MN-major, 64-byte swizzle, one 32-column atom per group of 8 K rows: byte
 // offset of the 16-byte chunk holding columns n0..n0+7 of K row r
@@ -577,7 +577,8 @@ __device__ __forceinline__ bool gt_wait_warp(uint32_t mbar, uint32_t parity, uin
     }
 }
 
-// One CTA per (matrix, tile of 128 rows), one CTA per SM, four roles:
+// A few CTAs per matrix (launch_gj_tc says how many), one CTA per SM, each over every gridDim.x-th
+// tile of 128 rows, four roles:
 //   X warp          the tile's old float pairs in and the updated ones out by tensor TMA
 //                   (two 16-column boxes of 128 rows each way, 128-byte swizzle; rows and
 //                   columns outside the matrix are zero-filled on load, clipped on store),
@@ -588,8 +589,8 @@ __device__ __forceinline__ bool gt_wait_warp(uint32_t mbar, uint32_t parity, uin
 //                   columns) once the epilogue has read the previous tile's
 //   16 epilogue     TMEM lane quadrant x 8 columns: the seven order sums, the old values
 //   warps           read from and the results written back to the stage in shared memory;
-//                   first, warps 0..3 move the panel planes into TMEM, where the MMAs read
-//                   them (A from TMEM: per MMA only the 1 KB B slice is read from shared
+//                   warps 0..3 move the panel planes, half a row tile ahead, into one of two
+//                   places in TMEM, where the MMAs read them (A from TMEM: per MMA only the 1 KB B slice is read from shared
 //                   memory, instead of 4 KB of A + 1 KB of B, which bounded the MMAs)
 // The panel's own column tile is final and skipped.  Every wait is bounded; one that runs
 // out sets the CTA's abort flag and every role leaves at its next wait; the matrix goes to
@@ -607,8 +608,10 @@ __global__ void __launch_bounds__(kGtUpThreads, 1) k_gt_update(const __grid_cons
     const int q = z % js.nj, m = z / js.nj;
     const GjJob &J = js.j[q];
     const int n = J.n, jb = js.jb;
-    const int rt = blockIdx.x;
-    if (m >= J.count || jb >= n || rt * 128 >= n) return;
+    // this CTA's row tiles: blockIdx.x, + gridDim.x, ...
+    const int rt0 = blockIdx.x, drt = gridDim.x;
+    if (m >= J.count || jb >= n || rt0 * 128 >= n) return;
+    const int nrt = ((n + 127) / 128 - rt0 + drt - 1) / drt;
     const int nc = (n + kGtN - 1) / kGtN;
     const int jp = jb / kGtN;                                    // the panel's own column tile
     const int ntl = nc - 1;                                      // column tiles updated
@@ -617,7 +620,7 @@ __global__ void __launch_bounds__(kGtUpThreads, 1) k_gt_update(const __grid_cons
     unsigned char *sc = js.scr[q] + (size_t)m * L.per;
     const GtState *st = reinterpret_cast<const GtState *>(sc + L.state);
     if (st->sing) return;
-    const int r0 = rt * 128, nr = min(128, n - r0);
+    const int nseq = nrt * ntl;                                  // tiles of this CTA, row tile by row tile
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const uint64_t tmap = reinterpret_cast<uint64_t>(&js.tmw[q]);
 
@@ -669,66 +672,79 @@ __global__ void __launch_bounds__(kGtUpThreads, 1) k_gt_update(const __grid_cons
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
-    int nld = 0, nst = 0, nb = 0, nmma = 0;                      // tiles loaded / stored / copied / multiplied
+    int nld = 0, nb = 0, nmma = 0, na = 0;                       // tiles loaded / copied / multiplied, row tiles of A loaded
 
     if (warp == kGtEpWarps) {
         // ---- X warp: stage sx holds tile i; before tile i + 3 is loaded into it, tile i is
         // stored and the store has finished reading the stage
         if (lane == 0) {
-            auto store = [&](int i) {
-                const int sx = i % kGtXs, c0 = col_tile(i) * kGtN;
+            struct Tile { int i, r0; };                          // column tile number, first row
+            auto next = [&](Tile &c) { if (++c.i == ntl) { c.i = 0; c.r0 += drt * 128; } };
+            auto store = [&](int sx, const Tile &c) {
                 const uint32_t xs = smem_u32(Xs + sx * kGtXStage);
-                tma_store_3d(tmap, xs, c0, r0, m);
-                tma_store_3d(tmap, xs + kGtXStage / 2, c0 + 16, r0, m);
+                const int c0 = col_tile(c.i) * kGtN;
+                tma_store_3d(tmap, xs, c0, c.r0, m);
+                tma_store_3d(tmap, xs + kGtXStage / 2, c0 + 16, c.r0, m);
                 bulk_commit();
-                nst = i + 1;
             };
-            for (int i = 0; i < ntl; ++i) {
-                const int sx = i % kGtXs;
-                if (i >= kGtXs) {
-                    if (!gt_wait1(XW(sx), ((i / kGtXs) - 1) & 1, js.wait_ns, &s_abort)) break;
-                    store(i - kGtXs);
+            Tile ld = {0, rt0 * 128}, sd = ld;                   // the next tile to load, to store
+            for (int q = 0; q < nseq; ++q) {
+                const int sx = q % kGtXs;
+                if (q >= kGtXs) {
+                    if (!gt_wait1(XW(sx), ((q / kGtXs) - 1) & 1, js.wait_ns, &s_abort)) break;
+                    store(sx, sd);
+                    next(sd);
                     bulk_wait_read0();
                 }
-                const int c0 = col_tile(i) * kGtN;
                 const uint32_t xs = smem_u32(Xs + sx * kGtXStage);
+                const int c0 = col_tile(ld.i) * kGtN;
                 mbar_expect_tx(XF(sx), kGtXStage);
-                tma_load_3d(tmap, xs, c0, r0, m, XF(sx));
-                tma_load_3d(tmap, xs + kGtXStage / 2, c0 + 16, r0, m, XF(sx));
-                nld = i + 1;
+                tma_load_3d(tmap, xs, c0, ld.r0, m, XF(sx));
+                tma_load_3d(tmap, xs + kGtXStage / 2, c0 + 16, ld.r0, m, XF(sx));
+                next(ld);
+                nld = q + 1;
             }
-            if (nld == ntl)
-                for (int i = max(0, ntl - kGtXs); i < ntl; ++i) {
-                    if (!gt_wait1(XW(i % kGtXs), (i / kGtXs) & 1, js.wait_ns, &s_abort)) break;
-                    store(i);
+            if (nld == nseq)
+                for (int q = max(0, nseq - kGtXs); q < nseq; ++q) {
+                    if (!gt_wait1(XW(q % kGtXs), (q / kGtXs) & 1, js.wait_ns, &s_abort)) break;
+                    store(q % kGtXs, sd);
+                    next(sd);
                 }
             bulk_wait_all0();                                    // every store complete
         }
     } else if (warp == kGtEpWarps + 1) {
         // ---- B warp
         if (lane == 0)
-            for (int i = 0; i < ntl; ++i) {
-                const int sb = i % kGtBs;
-                if (i >= kGtBs && !gt_wait1(BE(sb), ((i / kGtBs) - 1) & 1, js.wait_ns, &s_abort)) break;
+            for (int q = 0, i = 0; q < nseq; ++q, i = i + 1 == ntl ? 0 : i + 1) {
+                const int sb = q % kGtBs;
+                if (q >= kGtBs && !gt_wait1(BE(sb), ((q / kGtBs) - 1) & 1, js.wait_ns, &s_abort)) break;
                 mbar_expect_tx(BF(sb), kGtSl * kGtBPlane);
                 bulk_g2s(smem_u32(Bs + sb * kGtSl * kGtBPlane), sc + L.b + (size_t)col_tile(i) * kGtSl * kGtBPlane,
                          kGtSl * kGtBPlane, BF(sb));
-                nb = i + 1;
+                nb = q + 1;
             }
     } else if (warp == kGtEpWarps + 2) {
         // ---- MMA warp: warp-uniform control flow, one elected lane issues each MMA and commit
-        if (lane == 0) {
-            mbar_expect_tx(bA, kGtSl * kGtAPlane);
-            bulk_g2s(smem_u32(As), sc + L.a + (size_t)rt * kGtSl * kGtAPlane, kGtSl * kGtAPlane, bA);
-        }
-        __syncwarp();
-        if (gt_wait_warp(bAT, 0, js.wait_ns, &s_abort, lane)) {
+        auto load_a = [&](int it) {                              // the row tile's panel planes
+            if (lane == 0) {
+                mbar_expect_tx(bA, kGtSl * kGtAPlane);
+                bulk_g2s(smem_u32(As), sc + L.a + (size_t)(rt0 + it * drt) * kGtSl * kGtAPlane, kGtSl * kGtAPlane, bA);
+            }
+            na = it + 1;
+            __syncwarp();
+        };
+        load_a(0);
+        const uint32_t idesc = umma_idesc_f16(128, kGtN, 1);
+        bool ok = true;
+        for (int it = 0; it < nrt && ok; ++it) {
+            if (!gt_wait_warp(bAT, it & 1, js.wait_ns, &s_abort, lane)) break;
+            if (it + 1 < nrt) load_a(it + 1);                    // the planes are in TMEM: their stage is free
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t idesc = umma_idesc_f16(128, kGtN, 1);
+            const uint32_t atm = tmem + kGtATmem + (uint32_t)((it & 1) * kGtAtCols);
             for (int i = 0; i < ntl; ++i) {
-                const int sb = i % kGtBs;
-                if (!gt_wait_warp(BF(sb), (i / kGtBs) & 1, js.wait_ns, &s_abort, lane)) break;
-                if (i >= 1 && !gt_wait_warp(bTE, (i - 1) & 1, js.wait_ns, &s_abort, lane)) break;
+                const int q = it * ntl + i, sb = q % kGtBs;
+                if (!gt_wait_warp(BF(sb), (q / kGtBs) & 1, js.wait_ns, &s_abort, lane)) { ok = false; break; }
+                if (q >= 1 && !gt_wait_warp(bTE, (q - 1) & 1, js.wait_ns, &s_abort, lane)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint64_t dB = umma_desc_sw64_mn(smem_u32(Bs + sb * kGtSl * kGtBPlane), kGtBSbo, kGtBSbo);
 #pragma unroll
@@ -738,132 +754,153 @@ __global__ void __launch_bounds__(kGtUpThreads, 1) k_gt_update(const __grid_cons
 #pragma unroll
                         for (int ii = 0; ii <= d; ++ii) {
                             const int j = d - ii;
-                            const uint32_t at = tmem + kGtATmem + (uint32_t)((ii * 2 + kk) * 8);
+                            const uint32_t at = atm + (uint32_t)((ii * 2 + kk) * 8);
                             const uint64_t bd = dB + ((j * kGtBPlane + 2 * kk * kGtBSbo) >> 4);
                             if (kk == 0 && ii == 0) umma_bf16_ts_warp<0>(tmem + d * kGtN, at, bd, idesc);
                             else umma_bf16_ts_warp<1>(tmem + d * kGtN, at, bd, idesc);
                         }
                 umma_commit_warp(BE(sb));                        // the B stage may be refilled
                 umma_commit_warp(bTF);                           // the accumulators may be read
-                nmma = i + 1;
+                nmma = q + 1;
             }
         }
     } else {
         // ---- epilogue warps: row r of the tile (TMEM lane), columns cg * 8 .. + 7 of each column tile
         const int quad = warp & 3, cg = warp >> 2;
         const int r = quad * 32 + lane;
-        const bool row_ok = r < nr;
-        const int i_row = r0 + (row_ok ? r : 0);
-        const int E = row_ok ? reinterpret_cast<const int *>(sc + L.e)[i_row] : 0;
-        const bool is_piv = row_ok && (sc + L.piv)[i_row] != 0;
-        // 2^(E + F) as two exact multiplications by 2^E and 2^F when both lie in [-60, 60]: the
-        // order sums are 0 or at least 2^-56 in magnitude (multiples of the smallest unit), so
-        // the product with 2^E is a normal float, and the final rounding equals scale_pow2's
-        const bool E_ok = E >= -60 && E <= 60;
-        const float sE = __int_as_float((127 + (E_ok ? E : 0)) << 23);
         const uint32_t tlane = (uint32_t)(quad * 32) << 16;
         const uint32_t tl = tmem + tlane + (uint32_t)(cg * 8);
-        if (warp < 4) {
-            // the panel planes into TMEM columns 256 + 16 ii .. + 15: this thread's row, its 32
-            // K values packed in pairs (the 64-byte swizzle of the shared-memory planes undone)
-            if (gt_wait_warp(bA, 0, js.wait_ns, &s_abort, lane)) {
+        // the panel planes of the CTA's row tile `it` into TMEM (two places in turn): this thread's
+        // row, its 32 K values packed in pairs (the 64-byte swizzle of the shared-memory planes undone)
+        auto move_a = [&](int it) {
+            if (!gt_wait_warp(bA, it & 1, js.wait_ns, &s_abort, lane)) return;
 #pragma unroll 1
-                for (int ii = 0; ii < kGtSl; ++ii) {
-                    uint32_t w[16];
+            for (int ii = 0; ii < kGtSl; ++ii) {
+                uint32_t w[16];
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const uint4 u = *reinterpret_cast<const uint4 *>(As + ii * kGtAPlane + a_off64(r, c));
-                        w[4 * c] = u.x; w[4 * c + 1] = u.y; w[4 * c + 2] = u.z; w[4 * c + 3] = u.w;
-                    }
-                    tmem_st16(tmem + tlane + kGtATmem + (uint32_t)(16 * ii), w);
+                for (int c = 0; c < 4; ++c) {
+                    const uint4 u = *reinterpret_cast<const uint4 *>(As + ii * kGtAPlane + a_off64(r, c));
+                    w[4 * c] = u.x; w[4 * c + 1] = u.y; w[4 * c + 2] = u.z; w[4 * c + 3] = u.w;
                 }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bAT);
+                tmem_st16(tmem + tlane + kGtATmem + (uint32_t)((it & 1) * kGtAtCols + 16 * ii), w);
             }
-        }
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bAT);
+        };
+        // this thread's row of the row tile `it`: exponent E_i and whether it is one of the panel's
+        // pivot rows; loaded a row tile ahead
+        int E_nx = 0, piv_nx = 0;
+        auto row_info = [&](int it) {
+            const int i_row = (rt0 + it * drt) * 128 + r;
+            const bool ok = i_row < n;
+            E_nx = ok ? reinterpret_cast<const int *>(sc + L.e)[i_row] : 0;
+            piv_nx = ok ? (sc + L.piv)[i_row] : 0;
+        };
+        row_info(0);
+        if (warp < 4) move_a(0);
         // this thread's four 16-byte chunks of a stage (128-byte swizzle: chunk ^ (row & 7))
         const uint32_t xoff = (uint32_t)((cg >> 1) * (kGtXStage / 2) + r * 128);
         const int ck0 = (cg & 1) * 4;
         // test hook: the first panel's first wait of the chosen matrix runs out
-        const bool expire = m == js.expire_m && jb == 0 && rt == 0;
-        for (int i = 0; i < ntl; ++i) {
-            const int sx = i % kGtXs;
-            bool ok;
-            if (expire && i == 0) {
-                int f = 0;
-                if (lane == 0) {
-                    f = flag_wait(&s_never, js.wait_ns);
-                    if (!f) s_abort = 1;
+        const bool expire = m == js.expire_m && jb == 0 && rt0 == 0;
+        bool live = true;
+        for (int it = 0, q = 0; it < nrt && live; ++it) {
+            const int nr = min(128, n - (rt0 + it * drt) * 128);
+            const int E = E_nx;
+            const bool is_piv = piv_nx != 0;
+            // 2^(E + F) as two exact multiplications by 2^E and 2^F when both lie in [-60, 60]: the
+            // order sums are 0 or at least 2^-56 in magnitude (multiples of the smallest unit), so the
+            // product with 2^E is a normal float, and the final rounding equals scale_pow2's
+            const bool E_ok = E >= -60 && E <= 60;
+            const float sE = __int_as_float((127 + (E_ok ? E : 0)) << 23);
+            // the next row tile's planes move well before its first MMA (their place was read by the
+            // MMAs of the row tile before this one, all complete)
+            const int i_move = it + 1 < nrt ? ntl / 2 : -1;
+            for (int i = 0; i < ntl; ++i, ++q) {
+                if (i == i_move) {
+                    row_info(it + 1);
+                    if (warp < 4) move_a(it + 1);
                 }
-                ok = __shfl_sync(0xffffffffu, f, 0) != 0;
-            } else {
-                ok = gt_wait_warp(bTF, i & 1, js.wait_ns, &s_abort, lane);
-            }
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (quad * 32 >= nr) {                               // a ragged tile's warp without rows
+                const int sx = q % kGtXs;
+                bool ok;
+                if (expire && q == 0) {
+                    int f = 0;
+                    if (lane == 0) {
+                        f = flag_wait(&s_never, js.wait_ns);
+                        if (!f) s_abort = 1;
+                    }
+                    ok = __shfl_sync(0xffffffffu, f, 0) != 0;
+                } else {
+                    ok = gt_wait_warp(bTF, q & 1, js.wait_ns, &s_abort, lane);
+                }
+                if (!ok) { live = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (quad * 32 >= nr) {                               // a ragged tile's warp without rows
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bTE);
+                    if (!gt_wait_warp(XF(sx), (q / kGtXs) & 1, js.wait_ns, &s_abort, lane)) { live = false; break; }
+                    if (lane == 0) mbar_arrive(XW(sx));
+                    continue;
+                }
+                uint32_t v[kGtSl][8];
+#pragma unroll
+                for (int d = 0; d < kGtSl; ++d) tmem_ld8_async(tl + (uint32_t)(d * kGtN), v[d]);
+                tmem_wait_ld(v);
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bTE);
-                if (!gt_wait_warp(XF(sx), (i / kGtXs) & 1, js.wait_ns, &s_abort, lane)) break;
-                if (lane == 0) mbar_arrive(XW(sx));
-                continue;
-            }
-            uint32_t v[kGtSl][8];
+                // the seven order sums, exact integers in their units: orders 0..3 added as float
+                // pairs, orders 4..6 (below 2^-21 of the update) first in FP32 (rounding ~2^-46);
+                // two columns at a time (packed FP32)
+                float2 hs[4], ls[4];
+                auto ord = [&](int d, int k) {
+                    return make_float2(__uint_as_float(v[d][2 * k]), __uint_as_float(v[d][2 * k + 1]));
+                };
 #pragma unroll
-            for (int d = 0; d < kGtSl; ++d) tmem_ld8_async(tl + (uint32_t)(d * kGtN), v[d]);
-            tmem_wait_ld(v);
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bTE);
-            // the seven order sums, exact integers in their units: orders 0..3 added as float
-            // pairs, orders 4..6 (below 2^-21 of the update) first in FP32 (rounding ~2^-46);
-            // two columns at a time (packed FP32)
-            float2 hs[4], ls[4];
-            auto ord = [&](int d, int k) { return make_float2(__uint_as_float(v[d][2 * k]), __uint_as_float(v[d][2 * k + 1])); };
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                float2 sh, se;
-                gt_two_sum2(ord(0, k), ord(1, k), hs[k], ls[k]);
-                gt_two_sum2(hs[k], ord(2, k), sh, se);
-                ls[k] = __fadd2_rn(ls[k], se);
-                gt_two_sum2(sh, ord(3, k), hs[k], se);
-                ls[k] = __fadd2_rn(ls[k], se);
-                ls[k] = __fadd2_rn(ls[k], __fadd2_rn(ord(4, k), __fadd2_rn(ord(5, k), ord(6, k))));
-            }
-            if (!gt_wait_warp(XF(sx), (i / kGtXs) & 1, js.wait_ns, &s_abort, lane)) break;
-            unsigned char *xs = Xs + sx * kGtXStage + xoff;
-            const int ct = col_tile(i);
-            const int c0 = ct * kGtN + cg * 8;
-            const bool fast = E_ok && tile_ok[ct];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                float4 *p4 = reinterpret_cast<float4 *>(xs + (((ck0 + k) ^ (r & 7)) << 4));
-                float4 o = *p4;
-                if (is_piv) o = make_float4(0.f, 0.f, 0.f, 0.f);
-                float2 uh, ul;
-                if (fast) {
-                    const float2 f = *reinterpret_cast<const float2 *>(Fsc + c0 + 2 * k), e2 = gt_dup(sE);
-                    uh = __fmul2_rn(__fmul2_rn(hs[k], e2), f);
-                    ul = __fmul2_rn(__fmul2_rn(ls[k], e2), f);
-                } else {
-                    const int ex0 = E + Fs[c0 + 2 * k], ex1 = E + Fs[c0 + 2 * k + 1];
-                    uh = make_float2(scale_pow2(hs[k].x, ex0), scale_pow2(hs[k].y, ex1));
-                    ul = make_float2(scale_pow2(ls[k].x, ex0), scale_pow2(ls[k].y, ex1));
+                for (int k = 0; k < 4; ++k) {
+                    float2 sh, se;
+                    gt_two_sum2(ord(0, k), ord(1, k), hs[k], ls[k]);
+                    gt_two_sum2(hs[k], ord(2, k), sh, se);
+                    ls[k] = __fadd2_rn(ls[k], se);
+                    gt_two_sum2(sh, ord(3, k), hs[k], se);
+                    ls[k] = __fadd2_rn(ls[k], se);
+                    ls[k] = __fadd2_rn(ls[k], __fadd2_rn(ord(4, k), __fadd2_rn(ord(5, k), ord(6, k))));
                 }
-                // ff::add of the old values and the update
-                const float2 xh = make_float2(o.x, o.z), xl = make_float2(o.y, o.w);
-                float2 sm, e;
-                gt_two_sum2(xh, uh, sm, e);
-                e = __fadd2_rn(e, __fadd2_rn(xl, ul));
-                const float2 h = __fadd2_rn(sm, e);
-                const float2 l = __fadd2_rn(e, gt_neg2(__fadd2_rn(h, gt_neg2(sm))));
-                *p4 = make_float4(h.x, l.x, h.y, l.y);
+                if (!gt_wait_warp(XF(sx), (q / kGtXs) & 1, js.wait_ns, &s_abort, lane)) { live = false; break; }
+                unsigned char *xs = Xs + sx * kGtXStage + xoff;
+                const int ct = col_tile(i);
+                const int c0 = ct * kGtN + cg * 8;
+                const bool fast = E_ok && tile_ok[ct];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    float4 *p4 = reinterpret_cast<float4 *>(xs + (((ck0 + k) ^ (r & 7)) << 4));
+                    float4 o = *p4;
+                    if (is_piv) o = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float2 uh, ul;
+                    if (fast) {
+                        const float2 f = *reinterpret_cast<const float2 *>(Fsc + c0 + 2 * k), e2 = gt_dup(sE);
+                        uh = __fmul2_rn(__fmul2_rn(hs[k], e2), f);
+                        ul = __fmul2_rn(__fmul2_rn(ls[k], e2), f);
+                    } else {
+                        const int ex0 = E + Fs[c0 + 2 * k], ex1 = E + Fs[c0 + 2 * k + 1];
+                        uh = make_float2(scale_pow2(hs[k].x, ex0), scale_pow2(hs[k].y, ex1));
+                        ul = make_float2(scale_pow2(ls[k].x, ex0), scale_pow2(ls[k].y, ex1));
+                    }
+                    // ff::add of the old values and the update
+                    const float2 xh = make_float2(o.x, o.z), xl = make_float2(o.y, o.w);
+                    float2 sm, e;
+                    gt_two_sum2(xh, uh, sm, e);
+                    e = __fadd2_rn(e, __fadd2_rn(xl, ul));
+                    const float2 h = __fadd2_rn(sm, e);
+                    const float2 l = __fadd2_rn(e, gt_neg2(__fadd2_rn(h, gt_neg2(sm))));
+                    *p4 = make_float4(h.x, l.x, h.y, l.y);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // for the TMA store
+                __syncwarp();
+                if (lane == 0) mbar_arrive(XW(sx));
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // for the TMA store
-            __syncwarp();
-            if (lane == 0) mbar_arrive(XW(sx));
         }
     }
     __syncthreads();
@@ -876,14 +913,13 @@ __global__ void __launch_bounds__(kGtUpThreads, 1) k_gt_update(const __grid_cons
     if (s_abort && warp == kGtEpWarps + 1 && lane == 0)
         for (int i = max(0, nb - kGtBs); i < nb; ++i) mbar_wait(BF(i % kGtBs), (i / kGtBs) & 1, kDrainNs);
     if (warp == kGtEpWarps + 2 && lane == 0) {
-        if (s_abort) mbar_wait(bA, 0, kDrainNs);
+        if (s_abort && na > 0) mbar_wait(bA, (na - 1) & 1, kDrainNs);
         for (int i = max(0, nmma - kGtBs); i < nmma; ++i) mbar_wait(BE(i % kGtBs), (i / kGtBs) & 1, kDrainNs);
         if (nmma > 0) mbar_wait(bTF, (nmma - 1) & 1, kDrainNs);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" :: "r"(tmem) : "memory");
-    (void)nst;
 }
 
 // ||X^-1||_inf (the rows of X^-1 are the rows of the result, columns permuted) and
@@ -1075,12 +1111,31 @@ cudaError_t launch_gj_tc(const GjJob *jobs, int n_jobs, void *scratch, cudaStrea
     if ((e = gt_clusters(k_gt_init, g1, n_jobs, st, js)) != cudaSuccess) return e;
     const int nt = (nmax + 127) / 128;
     const int nz = cmax * n_jobs;
+    // CTAs per matrix of the update, each walking over its row tiles.  Many tiles: three row tiles
+    // each; the CTAs of a matrix share its B planes in L2, which one CTA finds evicted on its
+    // return (4096 matrices of 528 rows, 1 / 2 / 3 / 5 CTAs each: 59.5 / 57.3 / 59.5 / 63.9 ms, one
+    // tile per CTA without the loop 62.2; 1024 of 866 rows, 1 / 2 / 3 / 7: 66.1 / 63.1 / 61.5 / 63.1,
+    // 62.2).  Few tiles: one each, unless a schedule on 152 SMs is shorter by 15% with a CTA's
+    // prologue counted as 0.35 of a row tile (74 of 528 rows, 1 / 2 / 3 / 5: 2.00 / 1.34 / 1.70 /
+    // 1.46 ms; 128 of 528 rows, 1 / 5: 2.16 / 2.27; a gain of 9% by this count is none: 128 of 866
+    // rows, 1 / 7: 8.64 / 8.06).
+    int nt_up = (nt + 2) / 3;
+    if ((long long)nz * nt < 16 * 152) {
+        auto cost = [&](int d) { return ((nz * d + 151) / 152) * (20 * ((nt + d - 1) / d) + 7); };
+        int best = cost(nt) * 85 / 100;
+        nt_up = nt;
+        for (int d = 1; d < nt; ++d)
+            if (cost(d) < best) {
+                best = cost(d);
+                nt_up = d;
+            }
+    }
     for (int jb = 0; jb < nmax; jb += kGtB) {
         js.jb = jb;
         panel<<<g1, nthr, sm_panel, st>>>(js);
         for (int z0 = 0; z0 < nz; z0 += 65535) {
             const int zn = nz - z0 < 65535 ? nz - z0 : 65535;
-            k_gt_update<<<dim3(nt, 1, zn), kGtUpThreads, sm_up, st>>>(js, z0);
+            k_gt_update<<<dim3(nt_up, 1, zn), kGtUpThreads, sm_up, st>>>(js, z0);
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -102,3 +102,23 @@ def test_tensor_panel_sizes(n_up_plus):
         assert (out["logabs"][:, sp] - logabs).abs().max().item() < 1e-6
         E = D.mT @ C1 - torch.eye(m, dtype=torch.float64, device=dev)
         assert E.abs().max().item() < 1e-6
+
+
+@pytest.mark.parametrize("n", [130, 257, 545])
+def test_tensor_update_row_tiles(n):
+    """The update's CTAs take one or several row tiles each, by the number of matrices; every element's
+    arithmetic is the same, so the inverses of one walker repeated W times are equal bit for bit at
+    every split (repeated, because C1's slice scales go with the walkers that share a tile)."""
+    from paper_1209_6630_gb300 import QmcSystem
+    from synth import make_system, make_walkers
+    heavy = max(2, (2 * n) // 9)
+    s = make_system(heavy, 0, 0, 2 * n - 6 * heavy, seed=100 + n)      # 2 n electrons
+    assert s.n_up == n
+    q = QmcSystem(s, 0)
+    q.set_tiles(a4_mode="tensor", c15_mode="tensor")
+    R = torch.from_numpy(make_walkers(s, 1, first=95000)).to(dev)
+    ref = q.eval(R, precision="mixed", want_dinv=True)
+    for W in (38, 76, 250):
+        out = q.eval(R.expand(W, -1, -1).contiguous(), precision="mixed", want_dinv=True)
+        assert (out["dinv"] == ref["dinv"]).all()
+        assert (out["logabs"] - ref["logabs"]).abs().max().item() < 1e-12
