@@ -268,7 +268,7 @@ __device__ __forceinline__ float2 gt_dup(float x) { return make_float2(x, x); }
 // The panel kernel: one thread per row.  The 32 columns are eliminated in four sub-panels of 8,
 // whose columns sit in the thread's registers: each pivot step updates only those 8 columns (the
 // pivot column becomes the column of the step's Gauss-Jordan transformation); the other 24 lie
-// in shared memory (pairs of columns {h, h', l, l'}, rows of 13 x 16 bytes: conflict-free) and take
+// in shared memory (pairs of columns {h, h', l, l'}, rows of 12 x 16 bytes, swizzled) and take
 // the sub-panel's 8 pivots afterwards, two column pairs at a time in packed FP32; then the
 // registers change places with the next sub-panel's columns.
 //
@@ -282,15 +282,19 @@ __device__ __forceinline__ float2 gt_dup(float x) { return make_float2(x, x); }
 //
 // What bounds it is the FP32 pipe (15 operations per float-float multiply-add) and the chain of a
 // step: a REDUX search for the pivot (first of the rows not used yet with the largest |entry|), two
-// barriers, the pivot row scaled by its owner's warp.  Measured, one CTA per SM: 4096 matrices of
-// 528 rows, 17 panels, 54.0 -> 47.6 ms; 1024 of 866 rows, 28 panels (a warp per row before), 55.5 ->
-// 35.9 ms.
+// barriers, the pivot row scaled by its owner's warp.  Up to 544 rows, two CTAs fit on an SM (2 x
+// 107 KB, 56 registers a thread): one runs in the other's waits; for no more matrices than SMs, one
+// with 92 registers.  Measured: 4096 matrices of 528 rows, 17 panels, 54.0 (a warp per row) -> 47.6
+// (one CTA per SM) -> 42.0 ms (two); 74 of 528 rows 1.77 ms with one, 2.05 with two; 1024 of 866 rows,
+// 28 panels, 55.5 -> 35.2 ms.
 constexpr int kGtSeqMin = 545;
 constexpr int kGpSub = 8;
-constexpr int kGpLd = 13;                                // float4 per shared-memory row
+constexpr int kGpLd = 12;                                // float4 per shared-memory row
+// float4 j of row r lies at j ^ gp_sw(r): conflict-free without padding
+__device__ __forceinline__ int gp_sw(int r) { return (r >> 1) & 3; }
 
-template <int kMaxT, bool kSeq>
-__global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
+template <int kMaxT, bool kSeq, int kCtas>
+__global__ void __launch_bounds__(kMaxT, kCtas) k_gt_panel(GtJobs js)
 {
     const GjJob &J = js.j[blockIdx.y];
     const int m = blockIdx.x;
@@ -313,12 +317,14 @@ __global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
     __shared__ short ppS[kGtB];
     __shared__ unsigned red_k[kMaxT / 32];
     __shared__ int red_i[kMaxT / 32];
+    __shared__ GtState S_s;
 
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nwarps = blockDim.x >> 5;
     const int w = min(kGtB, n - jb);
     const int i = t;                                      // this thread's row
     const bool row_ok = i < n;
     float4 *P = reinterpret_cast<float4 *>(gp_smem), *row = P + (size_t)t * kGpLd;
+    const int sw = gp_sw(t);
     // the previous panel's pivots stop being pivots of the current panel
     if (jb > 0 && t < kGtB) piv_g[pp_g[jb - kGtB + t]] = 0;
     float2 xh[4], xl[4];                                  // the sub-panel's columns 2 q, 2 q + 1 of this row
@@ -336,12 +342,12 @@ __global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
                 xh[q] = make_float2(v.x, v.z);
                 xl[q] = make_float2(v.y, v.w);
             } else {
-                row[q - 4] = make_float4(v.x, v.z, v.y, v.w);
+                row[(q - 4) ^ sw] = make_float4(v.x, v.z, v.y, v.w);
             }
         }
     }
     bool used = !row_ok || used_g[i] != 0;
-    GtState S = *st;
+    if (t == (int)blockDim.x - 32) S_s = *st;             // (read and written by this thread only)
     bool sing = false;
     auto elem = [&](int c) { return (c & 1) ? make_float2(xh[c >> 1].y, xl[c >> 1].y) : make_float2(xh[c >> 1].x, xl[c >> 1].x); };
 
@@ -384,16 +390,16 @@ __global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
                 }
             }
             __syncthreads();
-            if (wid == nwarps - 1) {                      // (the last warp has the fewest rows)
+            if (t == (int)blockDim.x - 32) {              // (the last warp has the fewest rows)
                 const float2 pv = raw_s[cc];
                 const float2 a = pv.x < 0.f ? ff::neg(pv) : pv;
-                const float2 mg = ff::mul(make_float2(S.mag_h, S.mag_l), a);
+                const float2 mg = ff::mul(make_float2(S_s.mag_h, S_s.mag_l), a);
                 int ex;
                 frexpf(mg.x, &ex);
-                S.mag_h = ldexpf(mg.x, -ex);
-                S.mag_l = ldexpf(mg.y, -ex);
-                S.mag_e += ex;
-                S.neg ^= pv.x < 0.f;
+                S_s.mag_h = ldexpf(mg.x, -ex);
+                S_s.mag_l = ldexpf(mg.y, -ex);
+                S_s.mag_e += ex;
+                S_s.neg ^= pv.x < 0.f;
             }
             // the step on the sub-panel's 8 columns: the pivot column starts from zero
             const float2 f = ff::neg(xc);
@@ -414,7 +420,10 @@ __global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
         }
         if (sing) break;
         // the pivot rows' other columns, from before the sub-panel
-        for (int q = t; q < nk * 12; q += blockDim.x) U_s[q / 12][q % 12] = P[(size_t)ppS[c0 + q / 12] * kGpLd + q % 12];
+        for (int q = t; q < nk * 12; q += blockDim.x) {
+            const int p = ppS[c0 + q / 12];
+            U_s[q / 12][q % 12] = P[p * kGpLd + ((q % 12) ^ gp_sw(p))];
+        }
         if constexpr (kSeq)
             if (my_k >= 0)
 #pragma unroll
@@ -442,7 +451,7 @@ __global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
         const bool any_piv = __any_sync(0xffffffffu, my_k >= 0);
 #pragma unroll 1
         for (int j = 0; j < 12; j += 2) {
-            float4 a0 = row[j], a1 = row[j + 1];
+            float4 a0 = row[j ^ sw], a1 = row[(j + 1) ^ sw];
             if (!kSeq && my_k >= 0) a0 = a1 = make_float4(0.f, 0.f, 0.f, 0.f);
             float2 h0 = make_float2(a0.x, a0.y), l0 = make_float2(a0.z, a0.w);
             float2 h1 = make_float2(a1.x, a1.y), l1 = make_float2(a1.z, a1.w);
@@ -458,16 +467,16 @@ __global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
                     h1 = make_float2(u1.x, u1.y); l1 = make_float2(u1.z, u1.w);
                 }
             }
-            row[j] = make_float4(h0.x, h0.y, l0.x, l0.y);
-            row[j + 1] = make_float4(h1.x, h1.y, l1.x, l1.y);
+            row[j ^ sw] = make_float4(h0.x, h0.y, l0.x, l0.y);
+            row[(j + 1) ^ sw] = make_float4(h1.x, h1.y, l1.x, l1.y);
         }
         // the registers change places with the next sub-panel's columns: area sb of the row (4 column
         // pairs) then holds this one's
         if (sb < kGtB / kGpSub - 1) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float4 v = row[4 * sb + q];
-                row[4 * sb + q] = make_float4(xh[q].x, xh[q].y, xl[q].x, xl[q].y);
+                const float4 v = row[(4 * sb + q) ^ sw];
+                row[(4 * sb + q) ^ sw] = make_float4(xh[q].x, xh[q].y, xl[q].x, xl[q].y);
                 xh[q] = make_float2(v.x, v.y);
                 xl[q] = make_float2(v.z, v.w);
             }
@@ -484,9 +493,9 @@ __global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
     // column pair q of the panel: area q / 4 before the swaps' end, the registers after
     auto pair_at = [&](int q) {
         const int g = q >> 2;
-        if (g < swaps) return row[q];
+        if (g < swaps) return row[q ^ sw];
         if (g == swaps) return make_float4(xh[q & 3].x, xh[q & 3].y, xl[q & 3].x, xl[q & 3].y);
-        return row[q - 4];
+        return row[(q - 4) ^ sw];
     };
     // the eliminated panel is part of the result; operand A: the row scaled by its exponent, seven
     // slices, [row tile][slice] planes, 16-byte chunks of 8 columns
@@ -531,11 +540,7 @@ __global__ void __launch_bounds__(kMaxT, 1) k_gt_panel(GtJobs js)
         used_g[p] = 1;
         piv_g[p] = 1;
     }
-    if (t == (int)blockDim.x - 32) {
-        GtState o = *st;
-        o.mag_h = S.mag_h; o.mag_l = S.mag_l; o.mag_e = S.mag_e; o.neg = S.neg;
-        *st = o;
-    }
+    if (t == (int)blockDim.x - 32) *st = S_s;
     gt_operand_b(sc, L, n, jb, w, ppS);
 }
 
@@ -1101,7 +1106,9 @@ cudaError_t launch_gj_tc(const GjJob *jobs, int n_jobs, void *scratch, cudaStrea
     const int nthr = (nmax + 31) / 32 * 32;
     const size_t sm_panel = sizeof(float4) * (size_t)nthr * kGpLd;
     // one thread per row; the register budget follows the block
-    auto panel = nmax < kGtSeqMin ? k_gt_panel<544, false> : (nthr <= 896 ? k_gt_panel<896, true> : k_gt_panel<1024, true>);
+    // two CTAs per SM where there is more than one per SM to run (figures at the kernel)
+    auto panel = nmax < kGtSeqMin ? (cmax * n_jobs > 152 ? k_gt_panel<544, false, 2> : k_gt_panel<544, false, 1>)
+                                  : (nthr <= 896 ? k_gt_panel<896, true, 1> : k_gt_panel<1024, true, 1>);
     if ((e = cudaFuncSetAttribute(panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_panel)) != cudaSuccess)
         return e;
     if ((e = cudaFuncSetAttribute(k_gt_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_up)) !=

@@ -104,10 +104,10 @@ def test_tensor_panel_sizes(n_up_plus):
         assert E.abs().max().item() < 1e-6
 
 
-@pytest.mark.parametrize("n", [130, 257, 545])
+@pytest.mark.parametrize("n", [130, 257, 544, 545])
 def test_tensor_update_row_tiles(n):
-    """The update's CTAs take one or several row tiles each, by the number of matrices; every element's
-    arithmetic is the same, so the inverses of one walker repeated W times are equal bit for bit at
+    """The update's CTAs take one or several row tiles each and the panel runs with one or two CTAs per
+    SM, by the number of matrices; every element's arithmetic is the same, so the inverses of one walker repeated W times are equal bit for bit at
     every split (repeated, because C1's slice scales go with the walkers that share a tile)."""
     from paper_1209_6630_gb300 import QmcSystem
     from synth import make_system, make_walkers
