@@ -34,7 +34,7 @@
 // k_bw_mma:    per stage of 64 hits: the block's AO values for the hits as
 //              three K-major slice planes of X (all threads), and per MO tile
 //              the 64 hit rows of the D^-1 slices (cp.async into three MN-major
-//              planes, three buffers, one tile ahead); one thread issues the
+//              planes, three buffers, one tile ahead); a converged warp issues the
 //              4 x 6 MMAs (M128 N nb K16) of a tile into its accumulator and
 //              commits to an mbarrier.  Waits are bounded by %globaltimer; a
 //              CTA that gives up writes NaN into its partial.

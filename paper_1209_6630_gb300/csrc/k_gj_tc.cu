@@ -20,7 +20,7 @@
 //                each (the scheme of the C1/C5 products, one slice more)
 //   k_gt_update  X[i][j] <- [i is not a pivot row of the panel] X[i][j]
 //                           + sum_c P[i][c] U[c][j]
-//                for every column j outside the panel; one CTA per 128 rows,
+//                for every column j outside the panel; a CTA per one or several tiles of 128 rows,
 //                warp-specialised (warps moving the old values by tensor TMA
 //                and the operands by bulk copies, an MMA warp, 16 epilogue
 //                warps), loops over

@@ -223,7 +223,9 @@ __global__ void __launch_bounds__(kVdThreads, 2) k_vd_mma(VdArgs a)
     const uint64_t kWait = a.wait_ns;
     const uint16_t *Bsl = a.rslice[spin];
     const size_t bstride = (size_t)s.n_ao * nspad;
-    const int nst = (ns + kVdK - 1) / kVdK;               // (the padding beyond is zeros)
+    // K stops at the last 32 MOs that exist and the last AO tile's N at its AOs rounded up to 16 (the
+    // rest is zeros): 158 electrons x 100 walkers 325 -> 294 us, 434 x 4096 22.2 -> 21.0 ms
+    const int nst = (ns + kVdK - 1) / kVdK;
 
     // this CTA's D^-1 rows cut into six exact slices once, for every K stage (the AO tiles
     // reuse them): thread -> (row, chunk of 8 MOs), two per thread
