@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(1024) k_redo_list(RedoArgs a, int n_jobs)
 }
 
 // Eliminate panel [jb, jb + w) of every matrix (one CTA each).
-template <int kRNB>
-__global__ void __launch_bounds__(kRThreads) k_redo_panel(RedoArgs a, int jb)
+template <int kRNB, int kT>                                       // kT: the most threads
+__global__ void __launch_bounds__(kT) k_redo_panel(RedoArgs a, int jb)
 {
     const int b = blockIdx.x;
     if (b >= rcount(a)) return;
@@ -139,21 +139,21 @@ __global__ void __launch_bounds__(kRThreads) k_redo_panel(RedoArgs a, int jb)
     RedoState *stt = rstate(a, b, en);
     short *pp = rpp(stt), *panel = rpanel(stt, n);
     double *__restrict__ X = J.X + (size_t)en.m * J.x_stride;
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int nthr = kT == kRThreads ? kRThreads : blockDim.x, t = threadIdx.x, lane = t & 31, wid = t >> 5;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *P = reinterpret_cast<double *>(smem_raw);             // [n][kRNB]
     short *used = reinterpret_cast<short *>(P + (size_t)n * kRNB);  // [n]
     __shared__ GjPanelShared<kRNB> S;
 
     if (jb == 0) {
-        for (int i = t; i < n; i += kRThreads) panel[i] = -1;
+        for (int i = t; i < n; i += nthr) panel[i] = -1;
         if (t == 0) { stt->logabs = 0.0; stt->neg = 0; stt->sing = 0; }
         __syncthreads();
     }
     if (stt->sing) return;
     const int w = min(kRNB, n - jb);
-    for (int i = t; i < n; i += kRThreads) used[i] = panel[i] >= 0;
-    for (int q = t; q < n * kRNB; q += kRThreads) {
+    for (int i = t; i < n; i += nthr) used[i] = panel[i] >= 0;
+    for (int q = t; q < n * kRNB; q += nthr) {
         const int i = q / kRNB, c = q - i * kRNB;
         P[gj_at<kRNB>(i, c)] = (c < w) ? X[(size_t)i * n + jb + c] : 0.0;
     }
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kRThreads) k_redo_panel(RedoArgs a, int jb)
         if (lane == 0) { stt->sing = !ok; stt->logabs = logabs; stt->neg = neg; }
     }
     if (ok)
-        for (int q = t; q < n * w; q += kRThreads) {
+        for (int q = t; q < n * w; q += nthr) {
             const int i = q / w, c = q - i * w;
             X[(size_t)i * n + jb + c] = P[gj_at<kRNB>(i, c)];
         }
@@ -367,7 +367,11 @@ static cudaError_t launch_redo_panels(const RedoArgs &a, int nmax, cudaStream_t 
     const size_t smp = sizeof(double) * (size_t)nmax * NB + sizeof(short) * nmax;
     const size_t smu = sizeof(double) * (size_t)nmax * NB;
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_redo_panel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smp)) !=
+    // the panel's steps are a chain of FP64 latencies: a thread per row, within 256 to 1024 (n = 528,
+    // 33 panels of a few matrices 2.43 -> 2.00 ms; n = 866, 109 panels 4.12 -> 3.45; 512 threads 2.38 and 3.40)
+    const int pthr = NB < 32 ? std::min(1024, std::max(kRThreads, (a.nmax + 127) / 128 * 128)) : kRThreads;
+    auto panel = pthr > kRThreads ? k_redo_panel<NB, NB < 32 ? 1024 : kRThreads> : k_redo_panel<NB, kRThreads>;
+    if ((e = cudaFuncSetAttribute(panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smp)) !=
         cudaSuccess)
         return e;
     if ((e = cudaFuncSetAttribute(k_redo_update<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smu)) !=
@@ -376,7 +380,7 @@ static cudaError_t launch_redo_panels(const RedoArgs &a, int nmax, cudaStream_t 
     // update: two or three CTAs on each of 152 SMs walk over the items
     const unsigned ugrid = a.list ? 456 : (unsigned)std::min<long long>(456 * 8, (long long)a.n_all * ((nmax + 3) / 4));
     for (int jb = 0; jb < nmax; jb += NB) {
-        k_redo_panel<NB><<<a.list ? kRedoMax : a.n_all, kRThreads, smp, st>>>(a, jb);
+        panel<<<a.list ? kRedoMax : a.n_all, pthr, smp, st>>>(a, jb);
         k_redo_update<NB><<<ugrid, kRThreads, smu, st>>>(a, jb);
     }
     return cudaGetLastError();
