@@ -247,15 +247,32 @@ static bool gj_wide(int n, long long T)
 cudaError_t launch_gj(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb)
 {
     GjJobs2 js;
-    int nmax = 0, cmax = 0;
+    GjJob wide[2];
+    int n_wide = 0, wmax = 0;
+    long long T = 0;
     for (int q = 0; q < 2; ++q) {
         js.j[q] = jobs[q < n_jobs ? q : 0];
         if (q >= n_jobs) js.j[q].count = 0;
+        const GjJob &J = js.j[q];
+        // matrices of one row have no room for the spread elimination's state (a spin of one electron)
+        if (J.count == 0 || J.only_redo || gj_state_bytes(J.n) > sizeof(double) * (size_t)J.n * J.n) continue;
+        wide[n_wide++] = J;
+        wmax = max(wmax, J.n);
+        T += J.count;
+    }
+    if (n_wide && gj_wide(wmax, T)) {
+        const cudaError_t e = launch_gj_wide(wide, n_wide, st, nb);
+        if (e != cudaSuccess) return e;
+        for (int q = 0; q < 2; ++q)
+            if (gj_state_bytes(js.j[q].n) <= sizeof(double) * (size_t)js.j[q].n * js.j[q].n) js.j[q].count = 0;
+    }
+    int nmax = 0, cmax = 0;
+    for (int q = 0; q < 2; ++q) {
+        if (js.j[q].count == 0) continue;
         nmax = max(nmax, js.j[q].n);
         cmax = max(cmax, js.j[q].count);
     }
     if (cmax == 0) return cudaSuccess;
-    if (!jobs[0].only_redo && gj_wide(nmax, js.j[0].count + js.j[1].count)) return launch_gj_wide(jobs, n_jobs, st, nb);
     switch (nb) {
     case 8: return launch_gj_nb<8>(js, n_jobs, nmax, cmax, st);
     case 16: return launch_gj_nb<16>(js, n_jobs, nmax, cmax, st);

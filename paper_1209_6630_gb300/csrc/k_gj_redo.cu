@@ -19,7 +19,7 @@
 //
 // launch_gj_wide runs the same kernels over all matrices of a call too few to
 // fill the card with one CTA each (every SM's FP64 pipe is then in use); the
-// matrices' state sits in their own D^-1 arrays until the end.
+// matrices' state sits in their own D^-1 arrays until the end (from two rows on: one row has not the room).
 // (Rule and times: gj_wide in k_gj.cu.)
 #include <cooperative_groups.h>
 #include <math.h>
@@ -52,6 +52,7 @@ struct RedoState {
     double logabs;
     int neg, sing;
 };
+static_assert(sizeof(RedoState) == 16, "gj_state_bytes");
 
 struct RedoArgs {
     GjJob j[2];
@@ -82,7 +83,7 @@ __device__ __forceinline__ short *rpanel(RedoState *st, int n) { return rpp(st) 
 
 size_t redo_scratch_bytes(int nmax)
 {
-    const size_t stride = (16 + 4 * (size_t)nmax + 255) & ~size_t(255);
+    const size_t stride = (gj_state_bytes(nmax) + 255) & ~size_t(255);
     return ((sizeof(RedoList) + 255) & ~size_t(255)) + kRedoMax * stride;
 }
 
@@ -418,6 +419,9 @@ cudaError_t launch_gj_wide(const GjJob *jobs, int n_jobs, cudaStream_t st, int n
     RedoArgs a;
     const int nmax = redo_jobs(a, jobs, n_jobs);
     if (a.n_all == 0) return cudaSuccess;
+    for (int q = 0; q < 2; ++q)
+        if (a.j[q].count > 0 && gj_state_bytes(a.j[q].n) > sizeof(double) * (size_t)a.j[q].n * a.j[q].n)
+            return cudaErrorInvalidValue;
     const cudaError_t e = launch_redo_nb(a, nmax, st, nb);
     if (e != cudaSuccess) return e;
     k_redo_final<<<kFinalCluster * std::min(a.n_all, 1024), kRThreads, 0, st>>>(a);
@@ -436,7 +440,7 @@ cudaError_t launch_gj_redo(const GjJob *jobs, int n_jobs, void *scratch, cudaStr
     if (nmax > 1024) return cudaErrorInvalidValue;
     a.list = static_cast<RedoList *>(scratch);
     a.state = static_cast<char *>(scratch) + ((sizeof(RedoList) + 255) & ~size_t(255));
-    a.state_stride = (16 + 4 * (size_t)nmax + 255) & ~size_t(255);
+    a.state_stride = (gj_state_bytes(nmax) + 255) & ~size_t(255);
     a.e_off[0] = e_off ? e_off[0] : 0;
     a.e_off[1] = e_off ? e_off[1] : 0;
     k_redo_list<<<1, 1024, 0, st>>>(a, n_jobs);

@@ -135,7 +135,11 @@ cudaError_t launch_vdrift_f64(const SysDev &s, int nw, const double *R, const do
 cudaError_t launch_screen_ao(const SysDev &s, int nw, const double *R, int cap, int32_t *cnt,
                              int32_t *idx, double *B, cudaStream_t st);
 cudaError_t launch_gj(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb);
-// The same elimination with each matrix spread over many CTAs (k_gj_redo.cu).
+// State of a matrix whose elimination is spread over many CTAs: 16 bytes, then the pivot rows and the
+// panel of each row (2 bytes each).
+__host__ __device__ inline size_t gj_state_bytes(int n) { return 16 + 4 * (size_t)n; }
+// The same elimination with each matrix spread over many CTAs (k_gj_redo.cu).  Until its end a
+// matrix's state lies in its own D^-1: gj_state_bytes(n) <= 8 n^2 of every job, which is n >= 2.
 cudaError_t launch_gj_wide(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb);
 // Multi-CTA FP64 recomputation of up to kRedoMax flagged matrices (redo 1 -> 2).
 constexpr int kRedoMax = 256;
