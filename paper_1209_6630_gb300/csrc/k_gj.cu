@@ -75,7 +75,9 @@ __global__ void __launch_bounds__(kGjThreads, NB == 32 ? 1 : 3) k_gj(GjJobs2 job
     short *used = reinterpret_cast<short *>(U + NB * 32); // [n] 1 once a row has been a pivot
     short *pp = used + n;                                 // [n] pivot row of step k
     short *rowc = pp + n;                                 // [n] panel column of a pivot row, or -1
-    __shared__ GjPanelShared<NB> S;
+    // (in U, which is idle while a panel is eliminated: the largest panels fill the SM's shared memory)
+    static_assert(sizeof(GjPanelShared<NB>) <= sizeof(double) * NB * 32, "S lies in U");
+    GjPanelShared<NB> &S = *reinterpret_cast<GjPanelShared<NB> *>(U);
 
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     for (int i = t; i < n; i += kGjThreads) { used[i] = 0; rowc[i] = -1; }
