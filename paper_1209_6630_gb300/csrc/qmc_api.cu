@@ -832,13 +832,14 @@ size_t bytes_wanted(const Plan &p, int nw)
     return std::max(bytes_for(p, nw), array_bytes(p, nw) + al(stage_for(p, nw, true)));
 }
 
-// Walkers per chunk of a call of W walkers.  What bytes_wanted has beyond bytes_for does not
-// enter (q: the plan that the size query takes).
+// Walkers per chunk of a call of W walkers.  What the size query (plan q) reports beyond the least does
+// not enter, so a workspace of the queried size gives the chunks of the least one; below the queried
+// size the whole workspace counts.
 int chunk_walkers(const Plan &p, const Plan &q, int W, size_t ws_bytes)
 {
     const int Wq = std::min(W, 65535);
     const size_t least = bytes_for(q, Wq), wanted = bytes_wanted(q, Wq);
-    ws_bytes = ws_bytes >= wanted ? ws_bytes - (wanted - least) : std::min(ws_bytes, least);
+    if (ws_bytes >= wanted) ws_bytes -= wanted - least;
     int lo = 0, hi = Wq;
     while (lo < hi) {
         const int mid = lo + (hi - lo + 1) / 2;
