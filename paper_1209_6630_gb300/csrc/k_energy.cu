@@ -29,6 +29,7 @@
 
 #include "ff_math.cuh"
 #include "qmc_internal.cuh"
+#include "recip_f64.cuh"
 
 namespace qmc {
 
@@ -65,19 +66,6 @@ __device__ __forceinline__ float2 ff_inv_r(float2 dx, float2 dy, float2 dz)
     const float2 t = make_float2(y0s, fmaf(y0, y0, -y0s));      // y0^2 exactly
     const float2 e = ff::sub(make_float2(1.f, 0.f), ff::mul(r2, t));   // 1 - r2 y0^2, small
     return ff::renorm(y0, 0.5f * y0 * e.x);                      // Newton step y0 (1 + e/2)
-}
-
-// 1/sqrt(x) in FP64 from the FP32 reciprocal square root y (relative error 2^-22): with
-// e = 1 - x y^2, 1/sqrt(x) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + O(e^3)), O(e^3) < 2^-64
-// (Halley's third-order iteration): 5 FP64 operations, where the pipe is what the sums wait for.
-__device__ __forceinline__ bool in_fast_range(double x) { return x > 1e-30 && x < 1e30; }
-
-__device__ __forceinline__ double rsqrt_f64(double x)
-{
-    if (!in_fast_range(x)) return rsqrt(x);
-    const double y = (double)rsqrtf((float)x);
-    const double e = fma(-(x * y), y, 1.0);
-    return fma(e * y, fma(0.375, e, 0.5), y);
 }
 
 // Coulomb sums of one walker in float-float (mixed path); rs: 3N positions,
@@ -148,39 +136,6 @@ __device__ __forceinline__ void dets_drift_lap(const SysDev &s, const double *__
         b0 = warp_sum(b0); b1 = warp_sum(b1); b2 = warp_sum(b2);
     }
     b3 = warp_sum(b3);
-}
-
-// One Jastrow term, Pade form U = a r / (1 + b r): U' = a / (1 + b r)^2, U'' = -2 a b / (1 + b r)^3,
-// lap U(|r_e - x|) = U'' + 2 U' / r, grad U = U' (r_e - x) / r.  f = U' / r.
-__device__ __forceinline__ void jastrow_term(double r2, double a, double b, double &f, double &lap, double &u)
-{
-    double iq, ir, r, q;
-    bool fast = in_fast_range(r2);
-    if (fast) {
-        ir = rsqrt_f64(r2);
-        r = r2 * ir;
-        q = 1.0 + b * r;
-        fast = q < 1e30;
-    }
-    if (fast) {
-        // 1 / q from the FP32 reciprocal y: with e = 1 - q y, 1 / q = y (1 + e + e^2 + O(e^3))
-        const double y = (double)__frcp_rn((float)q);
-        const double e = fma(-q, y, 1.0);
-        iq = fma(y, fma(e, e, e), y);
-        const double t = a * iq;
-        u = t * r;
-        const double u1 = t * iq;
-        f = u1 * ir;
-        lap = fma(2.0, f, -2.0 * b * (u1 * iq));
-    } else {
-        r = sqrt(r2);
-        q = 1.0 + b * r;
-        iq = 1.0 / q;
-        const double u1 = a * iq * iq;
-        f = u1 / r;
-        lap = -2.0 * a * b * iq * iq * iq + 2.0 * f;
-        u = a * r * iq;
-    }
 }
 
 // The Jastrow factor of one walker over the CTAs of its cluster: grad_e J (acc[0..2][e]) and
