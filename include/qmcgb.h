@@ -294,10 +294,15 @@ int qmc_system_get_tiles(const qmc_system *sys, qmc_tiles *tiles);
 int qmc_system_shell_r2(const qmc_system *sys, double *R2_host);
 
 /*
- * qmc_workspace_size -- device scratch needed by qmc_walkers_eval for
- * `n_walk` walkers at `precision` (bytes).  A smaller workspace is allowed:
- * the walkers are then processed in consecutive chunks that fit, down to
- * one walker; below that the call fails with QMC_ERR_CAPACITY.
+ * qmc_workspace_size -- device scratch with which qmc_walkers_eval runs
+ * `n_walk` walkers at `precision` (bytes) as fast as it can: on the mixed
+ * path it has room to stage as many electrons per launch as fill the card
+ * (up to 8 GiB for the products, 4 GiB for the drift, one after the other in
+ * the same place), which for few walkers is most of it.  A smaller workspace
+ * is allowed: the launches then take fewer electrons at a time, and below
+ * the arrays of all walkers the walkers are processed in consecutive chunks
+ * that fit, down to one walker; below that the call fails with
+ * QMC_ERR_CAPACITY.
  */
 int qmc_workspace_size(const qmc_system *sys, int n_walk, int precision, size_t *bytes);
 
@@ -386,11 +391,12 @@ typedef struct {
     qmc_eval_out out;      /* device outputs, as for qmc_walkers_eval */
 } qmc_segment;
 
-/* Scratch for qmc_batch_eval: the sum of every segment's full workspace. */
+/* Scratch for qmc_batch_eval: the sum of every segment's qmc_workspace_size. */
 int qmc_batch_workspace_size(const qmc_segment *segs, int n_seg, int precision, size_t *bytes);
 
 /* a1..a6 for every segment (all systems on one device); ws of
- * qmc_batch_workspace_size bytes (QMC_ERR_CAPACITY if smaller). */
+ * qmc_batch_workspace_size bytes; a smaller one will do while it holds every segment's walkers in one
+ * chunk (every segment then takes fewer electrons per launch), else QMC_ERR_CAPACITY. */
 int qmc_batch_eval(const qmc_segment *segs, int n_seg, int precision, void *ws, size_t ws_bytes,
                    qmc_stream_t stream);
 

@@ -83,6 +83,20 @@ def system_desc(s):
     return d, keep, a_dtype
 
 
+def _scratch(nbytes: int, device):
+    """A uint8 workspace of nbytes, or, where the memory is not there, of the first that is in steps of
+    1/8 less: the size queries ask for room that lets every launch fill the card, the calls take less
+    (smaller launches, then chunks of walkers)."""
+    nbytes = max(int(nbytes), 1)
+    while True:
+        try:
+            return torch.empty(nbytes, dtype=torch.uint8, device=device)
+        except torch.OutOfMemoryError:
+            if nbytes < 1 << 20:
+                raise
+            nbytes -= nbytes // 8
+
+
 class QmcSystem:
     """A molecular system resident on one GPU (qmc_system_load)."""
 
@@ -96,7 +110,7 @@ class QmcSystem:
         h = C.c_void_p()
         check(lib().qmc_system_load(C.byref(d), device, C.byref(h)))
         self._h = h
-        self._ws = {}
+        self._ws = {}                                        # key -> (bytes asked for, workspace)
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
@@ -174,13 +188,15 @@ class QmcSystem:
         check(lib().qmc_workspace_size(self._h, n_walk, PREC[precision], C.byref(b)))
         return int(b.value)
 
-    def workspace(self, n_walk: int, precision: str = "f64"):
-        need = self.workspace_size(n_walk, precision)
-        ws = self._ws.get(precision)
-        if ws is None or ws.numel() < need:
-            ws = torch.empty(need, dtype=torch.uint8, device=self.device)
-            self._ws[precision] = ws
+    def _kept(self, key: str, need: int):
+        asked, ws = self._ws.get(key, (-1, None))
+        if asked < need:
+            ws = _scratch(need, self.device)
+            self._ws[key] = (need, ws)
         return ws
+
+    def workspace(self, n_walk: int, precision: str = "f64"):
+        return self._kept(precision, self.workspace_size(n_walk, precision))
 
     def alloc_out(self, W: int, want_dinv: bool = False):
         dev, f64 = self.device, torch.float64
@@ -283,11 +299,7 @@ class QmcSystem:
         for k, t in list(state_in.items()) + list(state_out.items()):
             _req_cuda(t, torch.int32 if k == "status" else torch.float64, k)
         if ws is None:
-            need = self.dmc_workspace_size(W, precision)
-            ws = self._ws.get("dmc")
-            if ws is None or ws.numel() < need:
-                ws = torch.empty(need, dtype=torch.uint8, device=self.device)
-                self._ws["dmc"] = ws
+            ws = self._kept("dmc", self.dmc_workspace_size(W, precision))
         si, so = _state_struct(state_in), _state_struct(state_out)
         p = DmcParams(tau=float(tau), e_trial=float(e_trial), seed=int(seed), step=int(step),
                       precision=PREC[precision], step_ptr=_ptr(step_ptr), e_trial_ptr=_ptr(e_trial_ptr))
@@ -315,11 +327,7 @@ class QmcSystem:
                                             _stream(self.device)))
             return dA_up, dA_dn
         if ws is None:
-            need = self.backward_workspace_size(W, precision)
-            ws = self._ws.get("backward")
-            if ws is None or ws.numel() < need:
-                ws = torch.empty(need, dtype=torch.uint8, device=self.device)
-                self._ws["backward"] = ws
+            ws = self._kept("backward", self.backward_workspace_size(W, precision))
         check(lib().qmc_logpsi_backward_ex(self._h, W, _ptr(R), _ptr(dinv), _ptr(g), PREC[precision],
                                            _ptr(dA_up), _ptr(dA_dn), _ptr(ws), ws.numel(), _stream(self.device)))
         return dA_up, dA_dn
@@ -351,7 +359,7 @@ class QmcBatch:
         b = C.c_size_t()
         check(lib().qmc_batch_workspace_size(segs, len(parts), PREC[precision], C.byref(b)))
         self.device = parts[0][0].device
-        self.ws = torch.empty(max(int(b.value), 1), dtype=torch.uint8, device=self.device)
+        self.ws = _scratch(b.value, self.device)
         self._g = None
         if graph:
             h = C.c_void_p()
@@ -393,7 +401,7 @@ def multidet_eval(systems, coef, R, precision: str = "f64"):
     assert cf.shape == (K,)
     b = C.c_size_t()
     check(lib().qmc_multidet_workspace_size(hs, K, W, PREC[precision], C.byref(b)))
-    ws = torch.empty(max(int(b.value), 1), dtype=torch.uint8, device=q0.device)
+    ws = _scratch(b.value, q0.device)
     o = q0.alloc_out(W)
     eo = _eval_out_struct(o)
     check(lib().qmc_multidet_eval(hs, C.c_void_p(cf.ctypes.data), K, W, _ptr(R), PREC[precision], C.byref(eo),
