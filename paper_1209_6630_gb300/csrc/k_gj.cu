@@ -238,12 +238,16 @@ static cudaError_t launch_gj_nb(const GjJobs2 &js, int n_jobs, int nmax, int cma
 // Whether to spread each matrix over many CTAs (launch_gj_wide, two launches per panel) rather
 // than to give it one (k_gj).  An SM's FP64 pipe takes as long for one matrix in k_gj whatever
 // the others do, so the call takes ceil(T / 152) matrices' time; spread, T / 152 and the panels'
-// latency.  Measured (ms, k_gj / spread): n = 217: T = 4 3.34 / 0.84, 100 3.35 / 2.60, 192 6.11 /
-// 4.36, 300 6.14 / 6.32, 600 11.96 / 12.54, 2000 40.5 / 40.0; n = 528: 4 40.2 / 4.5, 150 42.8 /
-// 40.5, 400 116 / 103; n = 866: 1 176 / 7.6, 150 190 / 173; n = 31: 50 0.100 / 0.112.
+// latency and launches, 2500 / n^2 of it (the excess over T / 152 at which the two meet, read off sizes
+// 32 .. 434 x 1 .. 2000 matrices; at 32 rows k_gj is as fast or faster at every T).  Measured (ms, k_gj /
+// spread): n = 33: T = 4 0.126 / 0.123, 200 0.147 / 0.168; n = 48: 50 0.158 / 0.152, 200 0.193 / 0.210; n = 64:
+// 4 0.225 / 0.182, 50 0.228 / 0.208, 200 0.290 / 0.278, 400 0.346 / 0.388; n = 100: 50 0.611 / 0.408, 100 0.612 /
+// 0.557, 400 1.295 / 1.309; n = 160: 100 1.43 / 1.24, 700 5.75 / 5.90; n = 217: 4 3.34 / 0.76, 100 3.38 / 2.52, 200
+// 6.10 / 4.65, 400 8.86 / 8.34, 700 14.7 / 14.5, 2000 40.5 / 40.0; n = 528: 4 40.2 / 4.5, 150 42.8 / 40.5, 400 116 / 103;
+// n = 866: 1 176 / 7.6, 150 190 / 173.
 static bool gj_wide(int n, long long T)
 {
-    return n >= 32 && (n >= 512 || (T + 151) / 152 * 152 * 100 > 105 * T);
+    return n > 32 && (n >= 512 || (T + 151) / 152 * 152 * n * n > T * (n * n + 2500));
 }
 
 cudaError_t launch_gj(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb)
