@@ -72,7 +72,7 @@ def autotune(q, R, precision="mixed", cache=DEFAULT_CACHE, force=False, verbose=
             timings["a4_mode=tensor"] = ms[1]
             if ms[1] < best_a4_ms:
                 best_a4, best_a4_ms = "tensor", ms[1]
-        except QmcError:                       # the panel kernel's shared memory: at most 880 per spin
+        except QmcError:                       # at most 896 electrons of one spin
             pass
         q.set_tiles(a4_mode=best_a4)
     best_g = start["c15_walkers"]

@@ -1043,11 +1043,10 @@ static cudaError_t gt_clusters(void (*kern)(Args...), dim3 g1, int n_jobs, cudaS
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-bool gjtc_fits(int nmax)
-{
-    const size_t sm = sizeof(float2) * (size_t)nmax * kGtB + sizeof(short) * (size_t)nmax;
-    return nmax <= 1024 && sm + 1024 <= 227 * 1024;
-}
+// The largest block of the panel kernel: one thread per row.
+constexpr int kGtMaxRows = 896;
+
+bool gjtc_fits(int nmax) { return nmax <= kGtMaxRows; }
 
 size_t gjtc_bytes(int n_up, int n_dn, int nw)
 {
@@ -1108,7 +1107,7 @@ cudaError_t launch_gj_tc(const GjJob *jobs, int n_jobs, void *scratch, cudaStrea
     // one thread per row; the register budget follows the block
     // two CTAs per SM where there is more than one per SM to run (figures at the kernel)
     auto panel = nmax < kGtSeqMin ? (cmax * n_jobs > 152 ? k_gt_panel<544, false, 2> : k_gt_panel<544, false, 1>)
-                                  : (nthr <= 896 ? k_gt_panel<896, true, 1> : k_gt_panel<1024, true, 1>);
+                                  : k_gt_panel<kGtMaxRows, true, 1>;
     if ((e = cudaFuncSetAttribute(panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_panel)) != cudaSuccess)
         return e;
     if ((e = cudaFuncSetAttribute(k_gt_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_up)) !=

@@ -621,7 +621,7 @@ extern "C" int qmc_system_set_tiles(qmc_system *sys, const qmc_tiles *tiles)
     if (tiles->a4_mode != QMC_A4_FP64 && tiles->a4_mode != QMC_A4_FLOAT_FLOAT && tiles->a4_mode != QMC_A4_TENSOR)
         return invalid("qmc_system_set_tiles: a4_mode");
     if (tiles->a4_mode == QMC_A4_TENSOR && !gjtc_fits(std::max(sys->d.n_up, sys->d.n_dn)))
-        return invalid("qmc_system_set_tiles: a4_mode tensor exceeds the panel kernel's shared memory");
+        return invalid("qmc_system_set_tiles: a4_mode tensor takes up to 896 electrons of one spin");
     if (tiles->c15_mode != QMC_C15_FLOAT_FLOAT && tiles->c15_mode != QMC_C15_TENSOR && tiles->c15_mode != QMC_C15_CFREE)
         return invalid("qmc_system_set_tiles: c15_mode");
     if ((tiles->c15_mode == QMC_C15_TENSOR || tiles->c15_mode == QMC_C15_CFREE) &&
