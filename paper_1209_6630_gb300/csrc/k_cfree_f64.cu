@@ -19,9 +19,8 @@
 //                partial dot products with D^-1[e,:], a transposing butterfly (7 additions)
 //                leaves each lane the v of one AO, which then meets that AO's derivatives
 // Measured, 434 electrons x 96 walkers: C1..C5 26.9 ms -> C1 5.8 + drift 7.6 ms
-// (158 electrons x 100: 4.6 -> 1.1 + 1.4 ms)
-#include <algorithm>
-
+// (158 electrons x 100: 4.6 -> 1.1 + 1.4 ms).  The tables of a chunk take up to 61 KB of shared memory at
+// the loader's limits (8192 shells, 16 primitives, L = 4, 1024 electrons of a spin), so every system fits.
 #include "c1_f64.cuh"
 
 namespace qmc {
@@ -176,11 +175,6 @@ cudaError_t launch_c1_nj(const SysDev &s, int nw, const double *R, double *X, cu
 }
 
 }  // namespace
-
-bool cfree_f64_fits(const SysDev &s)
-{
-    return s.n_shell <= 65535 && std::max(c1_smem(s), vd_smem(s)) <= 220 * 1024;
-}
 
 cudaError_t launch_c1_f64(const SysDev &s, int nw, const double *R, double *X, cudaStream_t st)
 {

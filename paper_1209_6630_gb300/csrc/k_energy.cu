@@ -90,11 +90,10 @@ __device__ __forceinline__ void coulomb_ff(const SysDev &s, const float2 *rs, co
     vee = ff::val(ee);
 }
 
-// Drift and Laplacian of the determinants for electron e (one warp; results
+// Drift and Laplacian of the determinants for electron e from C2..C5 (mixed path; one warp, results
 // on every lane): b_l = sum_k (D^-1)_{ek} C_{1+l}[e][k], lap = sum_k (D^-1)_{ek} C5[e][k].
-template <bool kMixed, typename TG>
 __device__ __forceinline__ void dets_drift_lap(const SysDev &s, const double *__restrict__ Dinv,
-                                               const TG *__restrict__ Cg, const CView &cv, int w, int e, int lane,
+                                               const float *__restrict__ Cg, const CView &cv, int w, int e, int lane,
                                                size_t msz, double &b0, double &b1, double &b2, double &b3)
 {
     const int spin = e >= s.n_up;
@@ -104,37 +103,26 @@ __device__ __forceinline__ void dets_drift_lap(const SysDev &s, const double *__
     const size_t soff = spin ? nu2 : 0;
     const size_t nss = (size_t)ns * ns;
     const double *drow = Dinv + (size_t)w * msz + soff + (size_t)ei * ns;
-    const TG *grow = Cg + (size_t)w * cv.g_wstride + (spin ? cv.g_ncomp * nu2 : 0) + (size_t)ei * ns;
+    const float *grow = Cg + (size_t)w * cv.g_wstride + (spin ? cv.g_ncomp * nu2 : 0) + (size_t)ei * ns;
     const double *lrow = cv.l + (size_t)w * cv.l_wstride + (spin ? cv.l_ncomp * nu2 : 0) +
                          (size_t)cv.l_comp * nss + (size_t)ei * ns;
-    b0 = b1 = b2 = b3 = 0.0;
-    if constexpr (kMixed) {
-        float f0 = 0.f, f1 = 0.f, f2 = 0.f;
-        for (int k = lane; k < ns; k += 32) {
-            const double d = drow[k];
-            const float df = f32_trunc(d);
-            f0 = fmaf(df, grow[k], f0);
-            f1 = fmaf(df, grow[nss + k], f1);
-            f2 = fmaf(df, grow[2 * nss + k], f2);
-            b3 = fma(d, lrow[k], b3);
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            f0 += __shfl_xor_sync(0xffffffffu, f0, off);
-            f1 += __shfl_xor_sync(0xffffffffu, f1, off);
-            f2 += __shfl_xor_sync(0xffffffffu, f2, off);
-        }
-        b0 = f0; b1 = f1; b2 = f2;
-    } else {
-        for (int k = lane; k < ns; k += 32) {
-            const double d = drow[k];
-            b0 = fma(d, (double)grow[k], b0);
-            b1 = fma(d, (double)grow[nss + k], b1);
-            b2 = fma(d, (double)grow[2 * nss + k], b2);
-            b3 = fma(d, lrow[k], b3);
-        }
-        b0 = warp_sum(b0); b1 = warp_sum(b1); b2 = warp_sum(b2);
+    float f0 = 0.f, f1 = 0.f, f2 = 0.f;
+    b3 = 0.0;
+    for (int k = lane; k < ns; k += 32) {
+        const double d = drow[k];
+        const float df = f32_trunc(d);
+        f0 = fmaf(df, grow[k], f0);
+        f1 = fmaf(df, grow[nss + k], f1);
+        f2 = fmaf(df, grow[2 * nss + k], f2);
+        b3 = fma(d, lrow[k], b3);
     }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        f0 += __shfl_xor_sync(0xffffffffu, f0, off);
+        f1 += __shfl_xor_sync(0xffffffffu, f1, off);
+        f2 += __shfl_xor_sync(0xffffffffu, f2, off);
+    }
+    b0 = f0; b1 = f1; b2 = f2;
     b3 = warp_sum(b3);
 }
 
@@ -245,11 +233,11 @@ __global__ void __launch_bounds__(kEnThreads) k_drift_energy(SysDev s, const dou
     }
     for (int e = gw; e < N; e += ngw) {
         double b0 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0;
-        if (cv.vd) {             // C-free variant: drift and Laplacian of the determinants already formed
+        if (!kMixed || cv.vd) {  // FP64 path, C-free variant: drift and Laplacian of the determinants already formed
             const double *v = cv.vd + ((size_t)w * N + e) * 4;
             b0 = v[0]; b1 = v[1]; b2 = v[2]; b3 = v[3];
-        } else {
-            dets_drift_lap<kMixed>(s, Dinv, Cg, cv, w, e, lane, msz, b0, b1, b2, b3);
+        } else if constexpr (kMixed) {
+            dets_drift_lap(s, Dinv, Cg, cv, w, e, lane, msz, b0, b1, b2, b3);
         }
         if (lane == 0) {
             double g0 = 0.0, g1 = 0.0, g2 = 0.0, L = 0.0;

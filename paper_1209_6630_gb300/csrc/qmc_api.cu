@@ -745,7 +745,7 @@ Plan make_plan(const qmc_system *sys, int precision, bool need_dinv, int c15_ove
     p.kappa_max = p.f64tc ? sys->tiles.f64_kappa_max : sys->tiles.a4_kappa_max;
     p.redo_bytes = p.ffgj ? redo_scratch_bytes(std::max(sys->d.n_up, sys->d.n_dn)) : 0;
     p.c15tc = p.mixed && (c15 == QMC_C15_TENSOR || c15 == QMC_C15_CFREE);
-    p.vd64 = !p.mixed && c15_override < 0 && cfree_f64_fits(sys->d);
+    p.vd64 = !p.mixed && c15_override < 0;
     p.sd = &sys->d;
     p.per_walker = p.msz * 8 + p.cd_bytes + (need_dinv ? p.msz * 8 : 0) + 36 + p.mask_bytes +
                    (p.ffgj ? p.msz * 8 + 2 : 0);
@@ -783,7 +783,9 @@ bool carve(const Plan &p, int nw, void *ws, size_t ws_bytes, Carve &c)
     } else {
         c.Cd = take(p.msz * 4 * 8 * nw);
         c.L5 = nullptr;
-        if (p.vd64) c.vd = static_cast<double *>(c.Cd);   // [nw][N][4] in the place of C2..C5 (N <= n_up^2 + n_dn^2)
+        // an evaluation has [nw][N][4] in the place of C2..C5 (N <= n_up^2 + n_dn^2).  It could do without the
+        // rest, but one size query serves it and qmc_slater_matrices, which fills the four.
+        if (p.vd64) c.vd = static_cast<double *>(c.Cd);
     }
     c.D = p.dinv ? reinterpret_cast<double *>(take(p.msz * 8 * nw)) : nullptr;
     c.la = reinterpret_cast<double *>(take(16 * (size_t)nw));
@@ -859,9 +861,9 @@ CView cview(const Plan &p, const Carve &c)
     } else if (p.mixed) {
         v.g_f32 = 1; v.g_wstride = 3 * p.msz; v.g_ncomp = 3;
         v.l = c.L5; v.l_wstride = p.msz; v.l_ncomp = 1; v.l_comp = 0;
-    } else {
-        v.g_f32 = 0; v.g_wstride = 4 * p.msz; v.g_ncomp = 4;
-        v.l = static_cast<const double *>(c.Cd); v.l_wstride = 4 * p.msz; v.l_ncomp = 4; v.l_comp = 3;
+    } else {                                             // FP64: vd
+        v.g_f32 = 0; v.g_wstride = 0; v.g_ncomp = 0;
+        v.l = nullptr; v.l_wstride = 0; v.l_ncomp = 0; v.l_comp = 0;
     }
     return v;
 }

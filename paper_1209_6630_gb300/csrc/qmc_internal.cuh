@@ -128,7 +128,6 @@ int cuda_fail(cudaError_t e, const char *where);
 cudaError_t launch_contract_f64(const SysDev &s, int nw, const double *R, double *X, double *Cd,
                                 cudaStream_t st);
 // FP64 path without C2..C5 (k_cfree_f64.cu)
-bool cfree_f64_fits(const SysDev &s);
 cudaError_t launch_c1_f64(const SysDev &s, int nw, const double *R, double *X, cudaStream_t st);
 cudaError_t launch_vdrift_f64(const SysDev &s, int nw, const double *R, const double *Dinv, double *vd,
                               cudaStream_t st);
@@ -150,15 +149,15 @@ cudaError_t launch_gj_ff(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb,
 // Where the gradient (C2..C4) and Laplacian (C5) matrices of a walker chunk live:
 // component c of spin s, electron row ei: base + w*wstride + (s ? ncomp*n_up^2 : 0) + c*ns^2 + ei*ns
 struct CView {
-    const void *g;      // gradients, FP32 if g_f32 else FP64
-    int g_f32;
+    const void *g;      // gradients, FP32
+    int g_f32;          // mixed path; the FP64 path has vd alone
     size_t g_wstride;
     int g_ncomp;
     const double *l;    // Laplacian, FP64, component l_comp of its block
     size_t l_wstride;
     int l_ncomp;
     int l_comp;
-    const double *vd;   // C-free variant: drift and Laplacian per electron [W][N][4] (the dots are done)
+    const double *vd;   // C-free variant and FP64 path: drift and Laplacian per electron [W][N][4] (the dots are done)
 };
 
 cudaError_t launch_drift_energy(const SysDev &s, int nw, const double *R, const double *Dinv, const CView &cv,
