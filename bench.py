@@ -32,21 +32,52 @@ WORKLOAD = "1056e"
 METRIC = "walker-steps/s at 1056 e, mixed-prec vs FP64 GPU path, at <=1e-6 log|Psi| err"
 
 
-def launches_per_step(q, prec, n_walk):
-    """Library kernels launched by one qmc_walkers_eval of a single walker chunk: exact for the mixed
-    path from 8 walker tiles on (the default workload); with fewer tiles a workspace of the queried
-    size holds larger electron batches than counted here, and the FP64 path adds its drift kernel."""
-    if prec == "f64":
-        return 3                      # C1, Gauss-Jordan, energy
+def _spread(n, b):
+    """Items per launch when n are spread evenly over launches of at most b."""
+    return n if n <= b else -(-n // -(-n // b))
+
+
+def _electron_batches(q, n_walk, cfree):
+    """Electrons per launch of the products and of the C-free drift in a workspace of the queried size:
+    the batches that fill the card within 8 and 4 GiB of staging (csrc/k_c15_tc.cu, csrc/k_vdrift.cu)."""
+    tiles = -(-n_walk // 128)
+    rows = 128 if n_walk >= 128 else -(-n_walk // 8) * 8
+    steps = -(-q.n_ao // 64)
+    slot = steps * 2 * (6 if cfree else 18) * rows * 64 + steps * 64 * 4 + 4 + 128 * 2 * 4
+    least = _spread(q.N, 128 if tiles >= 8 else (32 if tiles >= 2 else 16))
+    c15 = max(least, _spread(q.N, min(-(-2048 // tiles), max((8 << 30) // (tiles * slot), 1))))
+    stage = -(-max(q.n_up, q.n_dn) // 64) * 2 * 6 * rows * 64
+    vd = max(_spread(q.N, 264 if tiles >= 2 else 64),
+             _spread(q.N, min(-(-2432 // tiles), max((4 << 30) // (tiles * stage), 1))))
+    return c15, vd
+
+
+def _fp64_elimination_launches(q, n_walk, panel):
+    """One, or with few matrices two per panel and one more (csrc/k_gj.cu, gj_wide); a spin of one electron
+    is always in the single launch."""
+    sizes = [n for n in (q.n_up, q.n_dn) if n > 0]
+    wide = [n for n in sizes if n > 1]
+    T, n = n_walk * len(wide), max(wide, default=0)
+    if not (n > 32 and (n >= 512 or -(-T // 152) * 152 * n * n > T * (n * n + 2500))):
+        return 1
+    return 2 * -(-n // panel) + 1 + (len(wide) < len(sizes))
+
+
+def launches_per_step(q, prec, n_walk, queried=False):
+    """Library kernels launched by one qmc_walkers_eval of a single walker chunk, in a workspace of the
+    queried size, or (queried=False) of the least that holds the chunk, where the FP64 path's three
+    stages count as one launch each."""
     t = q.tiles()
+    if prec == "f64":
+        return 3 + _fp64_elimination_launches(q, n_walk, t["gj_panel"]) if queried else 3   # C1, v, energy beside it
     n = 2                             # masks, energy
     if t["c15_mode"] in ("tensor", "cfree"):
-        b = 128 if n_walk > 7 * 128 else (32 if n_walk > 128 else 16)
+        b, bv = 128 if n_walk > 7 * 128 else (32 if n_walk > 128 else 16), 264 if n_walk > 128 else 64
+        if queried:
+            b, bv = _electron_batches(q, n_walk, t["c15_mode"] == "cfree")
         n += 2 * -(-q.N // b)          # slice producer + MMA kernel per batch of electrons (C1..C5, or C1)
         if t["c15_mode"] == "cfree":
-            bv = 264 if n_walk > 128 else 64
-            n += 1 + -(-q.N // bv)    # row exponents of D^-1; v = D^-1 A^T with the drift / Laplacian per
-                                      # batch of up to 264 electrons (up to 64 for one walker tile)
+            n += 1 + -(-q.N // bv)    # row exponents of D^-1; v = D^-1 A^T with the drift / Laplacian per batch
     else:
         n += 2                        # float-float C1/C5, tensor-core C2..C4
     nmax = max(q.n_up, q.n_dn)
@@ -58,8 +89,10 @@ def launches_per_step(q, prec, n_walk):
         else:
             n += 1 + 2 * -(-nmax // 32) + 1 + redo   # init, panel + tensor-core update per 32 columns, final
     else:
-        n += 1
+        n += _fp64_elimination_launches(q, n_walk, t["gj_panel"]) if queried else 1
     return n
+
+
 DTYPE = {"f64": "f64", "mixed": "f64 (C1,C5 bf16 exact slices on tcgen05; C2-C4 fp16x3 tcgen05; a4 float-float)",
          "mixed_bf16": "f64 (C1,C5 bf16 exact slices on tcgen05; C2-C4 bf16x3 tcgen05; a4 float-float)"}
 
@@ -772,7 +805,7 @@ def main():
     t_step, value = aggregate(sum(step_ms) / len(step_ms), W, ws, dist, dev)
     st = np.array(stages)            # [K, 8]
     stage_mean = st.mean(axis=0)
-    n_launch = launches_per_step(q, prec, W)   # one walker chunk
+    n_launch = launches_per_step(q, prec, W, queried=True)   # one walker chunk
 
     # screening statistics of this batch (a1 on a sample, outside the timed region)
     ns = 16
