@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kBtThreads, 1) k_bw_mma(BwTcArgs a)
         }
     };
 
-    // The A copies of a thread: 16-byte chunk t % 16 of rows (hits) t / 16 + 16 i, i < 4, of each
+    // The A copies of a thread: 16-byte chunk t % 16 of rows (hits) t / 16 + 32 i, i < 2, of each
     // slice plane.  The rows' addresses are formed once per stage (formed anew for every copy they
     // were most of the kernel's instructions, with 8 warps to hide them: 57.6 -> 40.2 ms at 1731
     // electrons x 512 walkers; with 16 warps 34.9).
