@@ -506,8 +506,7 @@ cudaError_t launch_backward_tc(const SysDev &s, const MixedTables &mt, const BwB
     if (chunk_bytes(s, mw, wc, wb) > ws_bytes) return cudaErrorMemoryAllocation;
     const size_t sm = smem_bytes(bb.nb);
     if (sm > 227 * 1024) return cudaErrorInvalidConfiguration;
-    if ((e = cudaFuncSetAttribute(k_bw_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
-        return e;
+    if ((e = allow_smem<k_bw_mma>(sm)) != cudaSuccess) return e;
 
     const int ns8u = round8(s.n_up), ns8d = round8(s.n_dn);
     const size_t msz8 = msz8_of(s), msz = (size_t)s.n_up * s.n_up + (size_t)s.n_dn * s.n_dn;

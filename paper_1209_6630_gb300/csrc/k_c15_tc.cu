@@ -778,12 +778,9 @@ cudaError_t launch_c15_tc(const SysDev &s, const FfBasis &fb, const MixedTables 
                           sizeof(int) * (size_t)a.kmax_steps * TC_K;
     if (sm_mma > 227 * 1024 || sm_prep > 227 * 1024) return cudaErrorInvalidConfiguration;
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(c1_only ? k_c15_prep<true> : k_c15_prep<false>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_prep)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_c15_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_mma)) !=
-        cudaSuccess)
-        return e;
+    e = c1_only ? allow_smem<k_c15_prep<true>>(sm_prep) : allow_smem<k_c15_prep<false>>(sm_prep);
+    if (e != cudaSuccess) return e;
+    if ((e = allow_smem<k_c15_mma>(sm_mma)) != cudaSuccess) return e;
     const int mtiles = (nmax + TC_N - 1) / TC_N;
     // row groups of the producer: down to 32 rows (a warp's lanes) while a launch has fewer than
     // three CTAs for each of 152 SMs (158 electrons x 100 walkers, 158 pairs: 307 -> 166 us;

@@ -168,7 +168,7 @@ template <int NJ>
 cudaError_t launch_c1_nj(const SysDev &s, int nw, const double *R, double *X, cudaStream_t st)
 {
     const size_t sm = c1_smem(s);
-    cudaError_t e = cudaFuncSetAttribute(k_c1_f64<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem<k_c1_f64<NJ>>(sm);
     if (e != cudaSuccess) return e;
     k_c1_f64<NJ><<<dim3(s.n_elec, nw), kCfThreads, sm, st>>>(s, R, X);
     return cudaGetLastError();
@@ -198,7 +198,7 @@ cudaError_t launch_vdrift_f64(const SysDev &s, int nw, const double *R, const do
 {
     if (nw == 0 || s.n_elec == 0) return cudaSuccess;
     const size_t sm = vd_smem(s);
-    cudaError_t e = cudaFuncSetAttribute(k_vd_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem<k_vd_f64>(sm);
     if (e != cudaSuccess) return e;
     k_vd_f64<<<dim3(s.n_elec, nw), kCfThreads, sm, st>>>(s, R, Dinv, vd);
     return cudaGetLastError();

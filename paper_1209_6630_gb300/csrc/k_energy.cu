@@ -327,7 +327,7 @@ static cudaError_t launch_en(const SysDev &s, int nw, const double *R, const dou
     // CTAs to each of 152 SMs and each warp keeps an electron
     unsigned c = 1;
     while (c < 8 && (size_t)nw * c < 152 * 4 && N >= (size_t)2 * kEnWarps * c) c *= 2;
-    cudaError_t e = cudaFuncSetAttribute(k_drift_energy<TG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem<k_drift_energy<TG>>(sm);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;

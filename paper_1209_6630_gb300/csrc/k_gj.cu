@@ -226,7 +226,7 @@ template <int NB>
 static cudaError_t launch_gj_nb(const GjJobs2 &js, int n_jobs, int nmax, int cmax, cudaStream_t st)
 {
     const size_t sm = sizeof(double) * (p_region(nmax, NB) + NB * 32) + sizeof(short) * 3 * (size_t)nmax;
-    cudaError_t e = cudaFuncSetAttribute(k_gj<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem<k_gj<NB>>(sm);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_gj<NB>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
@@ -652,8 +652,8 @@ static cudaError_t launch_gj_ff_k(const GjJobs2 &js, int n_jobs, int nmax, int c
                                   cudaStream_t st)
 {
     const size_t sm = gjff_fixed_bytes(nmax, NB) + (kSmem ? sizeof(float2) * nmax * (size_t)(nmax | 1) : 0);
-    auto kern = k_gj_ff<NB, THREADS, RPT, MIN, kSmem>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    constexpr auto kern = k_gj_ff<NB, THREADS, RPT, MIN, kSmem>;
+    cudaError_t e = allow_smem<kern>(sm);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;

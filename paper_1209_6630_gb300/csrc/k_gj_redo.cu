@@ -342,7 +342,7 @@ template <int NJ>
 static cudaError_t launch_redo_c1(const SysDev &s, const RedoArgs &a, int nmax, const double *R, cudaStream_t st)
 {
     const size_t sm = c1_smem(s);
-    cudaError_t e = cudaFuncSetAttribute(k_redo_c1<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem<k_redo_c1<NJ>>(sm);
     if (e != cudaSuccess) return e;
     k_redo_c1<NJ><<<dim3(nmax, kC1Slots), kCfThreads, sm, st>>>(s, a, R);
     return cudaGetLastError();
@@ -371,13 +371,10 @@ static cudaError_t launch_redo_panels(const RedoArgs &a, int nmax, cudaStream_t 
     // the panel's steps are a chain of FP64 latencies: a thread per row, within 256 to 1024 (n = 528,
     // 33 panels of a few matrices 2.43 -> 2.00 ms; n = 866, 109 panels 4.12 -> 3.45; 512 threads 2.38 and 3.40)
     const int pthr = NB < 32 ? std::min(1024, std::max(kRThreads, (a.nmax + 127) / 128 * 128)) : kRThreads;
-    auto panel = pthr > kRThreads ? k_redo_panel<NB, NB < 32 ? 1024 : kRThreads> : k_redo_panel<NB, kRThreads>;
-    if ((e = cudaFuncSetAttribute(panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smp)) !=
-        cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_redo_update<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smu)) !=
-        cudaSuccess)
-        return e;
+    constexpr auto few = k_redo_panel<NB, kRThreads>, many = k_redo_panel<NB, NB < 32 ? 1024 : kRThreads>;
+    const auto panel = pthr > kRThreads ? many : few;
+    if ((e = pthr > kRThreads ? allow_smem<many>(smp) : allow_smem<few>(smp)) != cudaSuccess) return e;
+    if ((e = allow_smem<k_redo_update<NB>>(smu)) != cudaSuccess) return e;
     // update: two or three CTAs on each of 152 SMs walk over the items
     const unsigned ugrid = a.list ? 456 : (unsigned)std::min<long long>(456 * 8, (long long)a.n_all * ((nmax + 3) / 4));
     for (int jb = 0; jb < nmax; jb += NB) {

@@ -1106,13 +1106,12 @@ cudaError_t launch_gj_tc(const GjJob *jobs, int n_jobs, void *scratch, cudaStrea
     const size_t sm_panel = sizeof(float4) * (size_t)nthr * kGpLd;
     // one thread per row; the register budget follows the block
     // two CTAs per SM where there is more than one per SM to run (figures at the kernel)
-    auto panel = nmax < kGtSeqMin ? (cmax * n_jobs > 152 ? k_gt_panel<544, false, 2> : k_gt_panel<544, false, 1>)
-                                  : k_gt_panel<kGtMaxRows, true, 1>;
-    if ((e = cudaFuncSetAttribute(panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_panel)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_gt_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_up)) !=
-        cudaSuccess)
-        return e;
+    constexpr auto two = k_gt_panel<544, false, 2>, one = k_gt_panel<544, false, 1>, seq = k_gt_panel<kGtMaxRows, true, 1>;
+    const bool share = cmax * n_jobs > 152;
+    const auto panel = nmax >= kGtSeqMin ? seq : (share ? two : one);
+    e = nmax >= kGtSeqMin ? allow_smem<seq>(sm_panel) : (share ? allow_smem<two>(sm_panel) : allow_smem<one>(sm_panel));
+    if (e != cudaSuccess) return e;
+    if ((e = allow_smem<k_gt_update>(sm_up)) != cudaSuccess) return e;
     const dim3 g1(cmax, n_jobs);
     if ((e = gt_clusters(k_gt_init, g1, n_jobs, st, js)) != cudaSuccess) return e;
     const int nt = (nmax + 127) / 128;

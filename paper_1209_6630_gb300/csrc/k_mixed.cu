@@ -818,7 +818,7 @@ static cudaError_t launch_c15_nq(const C15Args &a, int nwarps, cudaStream_t st)
 {
     const size_t sm = sizeof(float4) * G * kC15Chunk + sizeof(double) * kC15Warps * G * 64 +
                       sizeof(uint32_t) * (G + 1) * a.mw + sizeof(int) * ((size_t)a.s.n_ao + 2);
-    cudaError_t e = cudaFuncSetAttribute(k_c15_ff<NQ, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem<k_c15_ff<NQ, G>>(sm);
     if (e != cudaSuccess) return e;
     dim3 grid(a.s.n_elec, (a.nw + G - 1) / G);
     k_c15_ff<NQ, G><<<grid, 32 * nwarps, sm, st>>>(a);
@@ -878,7 +878,7 @@ cudaError_t launch_tc_contract(const SysDev &s, int nw, const double *R, const u
     a.wait_ns = wc.limit_ns;
     const size_t sm = tc_smem_bytes(s, mw);
     if (sm > 227 * 1024) return cudaErrorInvalidConfiguration;   // system too large for one tile
-    cudaError_t e = cudaFuncSetAttribute(k_tc_contract, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem<k_tc_contract>(sm);
     if (e != cudaSuccess) return e;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     dim3 grid((nmax + TC_N - 1) / TC_N, s.n_elec, (nw + TC_M - 1) / TC_M);

@@ -507,7 +507,7 @@ cudaError_t launch_vdrift(const SysDev &s, const FfBasis &fb, const MixedTables 
     k_vd_rowexp<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(nw, s.n_up, s.n_dn, a.msz, Dinv,
                                                           static_cast<int *>(scratch));
     const size_t sm = 1024 + (size_t)kVdBuf + sizeof(int) * ((size_t)s.n_ao + kVdN);
-    cudaError_t e = cudaFuncSetAttribute(k_vd_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem<k_vd_mma>(sm);
     if (e != cudaSuccess) return e;
     const int tiles = (nw + TC_M - 1) / TC_M;
     // as many electrons per launch as the scratch holds, up to the batch that fills the card

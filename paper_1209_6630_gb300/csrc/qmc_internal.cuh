@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -120,6 +121,25 @@ struct GjJob {
     long long redo_stride;
     int only_redo;      // FP64 kernel: process only matrices with redo[m] == 1 (flagged, not recomputed yet)
 };
+
+// Lets kernel K be launched with `bytes` of dynamic shared memory.  The limit is set to all that an SM has
+// beside the kernel's static shared memory, not to the call's own size: a call of a smaller system on
+// another thread would lower it between this one's setting and its launch (which then fails).
+template <auto K>
+cudaError_t allow_smem(size_t bytes)
+{
+    static std::atomic<size_t> room{0};                  // a property of the kernel
+    size_t r = room.load(std::memory_order_relaxed);
+    if (r == 0) {
+        cudaFuncAttributes a;
+        const cudaError_t e = cudaFuncGetAttributes(&a, K);
+        if (e != cudaSuccess) return e;
+        r = 227 * 1024 - a.sharedSizeBytes;
+        room.store(r, std::memory_order_relaxed);
+    }
+    if (bytes > r) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r);
+}
 
 void set_error(const std::string &msg);
 int cuda_fail(cudaError_t e, const char *where);
