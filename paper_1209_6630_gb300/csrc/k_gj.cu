@@ -422,17 +422,7 @@ __global__ void __launch_bounds__(THREADS, MIN) k_gj_ff(GjJobs2 jobs, double kap
             if (lane == 0) { red_k[wid] = k; red_i[wid] = bi; }
         }
         __syncthreads();
-        for (int c = 0; c < NB; ++c) {
-            if (c >= w) {                                     // a short last panel: back into column order
-#pragma unroll
-                for (int r = 0; r < RPT; ++r) {
-                    const float2 x0 = x[r][0];
-#pragma unroll
-                    for (int q = 0; q + 1 < NB; ++q) x[r][q] = x[r][q + 1];
-                    x[r][NB - 1] = x0;
-                }
-                continue;
-            }
+        for (int c = 0; c < w; ++c) {
             unsigned k = lane < WARPS ? red_k[lane] : 0u;
             int p = lane < WARPS ? red_i[lane] : n;
             gjff_warp_max(k, p);
@@ -492,7 +482,8 @@ __global__ void __launch_bounds__(THREADS, MIN) k_gj_ff(GjJobs2 jobs, double kap
         }
         if (sing) break;
 
-        // the eliminated panel: part of the result, and the update's operand as row pairs
+        // the eliminated panel: part of the result, and the update's operand as row pairs (the registers
+        // are w steps round: all the way, but in a short last panel)
 #pragma unroll
         for (int r = 0; r < RPT; ++r) {
             const int i = t + THREADS * r;
@@ -500,9 +491,10 @@ __global__ void __launch_bounds__(THREADS, MIN) k_gj_ff(GjJobs2 jobs, double kap
             if (i < n) {
 #pragma unroll
                 for (int q = 0; q < NB; ++q) {
-                    if (q < w) Wk[(size_t)i * ld + jb + q] = x[r][q];
-                    dst[4 * q] = x[r][q].x;
-                    dst[4 * q + 2] = x[r][q].y;
+                    const int col = (q + w) & (NB - 1);
+                    if (col < w) Wk[(size_t)i * ld + jb + col] = x[r][q];
+                    dst[4 * col] = x[r][q].x;
+                    dst[4 * col + 2] = x[r][q].y;
                 }
             } else if (i < 2 * np) {
 #pragma unroll
@@ -662,7 +654,10 @@ static cudaError_t launch_gj_ff_k(const GjJobs2 &js, int n_jobs, int nmax, int c
     return cudaGetLastError();
 }
 
-// One row per thread while the rows fit a block of 256 or 512, else two.  Blocks of 256: the work
+// One row per thread while the rows fit a block of 64, 256 or 512, else two.  Blocks of 64 where there are
+// more small matrices than two blocks of 256 on each of 152 SMs hold: a block of 256 has few threads with a row
+// there, and registers for two blocks (the elimination's stage, 40000 matrices, ms: 5 rows 1.49 -> 0.55, 32 rows
+// 5.55 -> 2.83; 4000 of 64 rows 1.64 -> 1.37).  Blocks of 256: the work
 // matrix in shared memory where that leaves room for the matrices' CTAs (three on each of 152 SMs,
 // or as many as there are: 2 matrices of 79 rows 164 -> 152 us); else with registers for two CTAs
 // per SM where two hold every matrix, for three beyond (8192 matrices of 217 rows: 54.5 -> 52.0 ms;
@@ -672,8 +667,10 @@ static cudaError_t launch_gj_ff_nb(const GjJobs2 &js, int n_jobs, int nmax, int 
                                    cudaStream_t st)
 {
     constexpr int M2 = NB <= 16 ? 2 : 1, M3 = NB <= 16 ? 3 : 1;
+    const long long T = (long long)cmax * n_jobs;
+    if (nmax <= 64 && T > 304)
+        return launch_gj_ff_k<NB, 64, 1, NB <= 16 ? 8 : 4, true>(js, n_jobs, nmax, cmax, kappa_max, st);
     if (nmax <= 256) {
-        const long long T = (long long)cmax * n_jobs;
         const size_t sm = gjff_fixed_bytes(nmax, NB) + sizeof(float2) * nmax * (size_t)(nmax | 1);
         if (sm <= 72 * 1024 || (T <= 304 && sm <= 108 * 1024) || (T <= 152 && sm <= 220 * 1024))
             return launch_gj_ff_k<NB, 256, 1, M2, true>(js, n_jobs, nmax, cmax, kappa_max, st);
