@@ -133,11 +133,18 @@ __global__ void __launch_bounds__(kBwThreads) k_backward_f64(SysDev s, int nw, c
         __syncthreads();
         nbuf = 0;
     }
+    double *dA = spin ? dA_dn : dA_up;
+    if (nrank == 1) {
+        if (k < ns)
+#pragma unroll
+            for (int m = 0; m < MAXAO; ++m)
+                if (m < nao) dA[(size_t)(ao0 + m) * ns + k] = acc[m];
+        return;
+    }
     // partial sums [MAXAO][128]; rank r adds rows r, r + C, ... over the ranks in order
 #pragma unroll
     for (int m = 0; m < MAXAO; ++m) chi_s[m * kBwThreads + t] = acc[m];
     cluster.sync();
-    double *dA = spin ? dA_dn : dA_up;
     if (k < ns)
         for (int m = rank; m < nao; m += nrank) {
             double x = 0.0;
