@@ -14,7 +14,7 @@
 // electron row for the dot products (rows of D^-1 and of C2..C5 are contiguous);
 // warp-shuffle reductions, the CTAs' sums added in rank order through distributed shared memory.
 // Measured: 1056 electrons x 37 walkers 854 -> 272 us (37 CTAs before), 158 electrons x 1 walker
-// 52 -> 17 us; with the Jastrow factor, 434 electrons x 601 walkers 13.6 -> 7.5 ms.
+// 52 -> 17 us; with the Jastrow factor, 434 electrons x 601 walkers 13.6 -> 7.2 ms.
 //
 // FP64 path: everything in FP64.  Mixed path (C2..C4 in FP32): the drift
 // dots in FP32 (D^-1 truncated to float by integer operations), the

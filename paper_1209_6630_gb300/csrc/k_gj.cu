@@ -306,7 +306,7 @@ cudaError_t launch_gj(const GjJob *jobs, int n_jobs, cudaStream_t st, int nb)
 // (packed FP32 instructions: two results per issue slot, the same roundings), the eliminated
 // panel lying in shared memory as row pairs {h, h', l, l'}.  Bound by the FP32 pipe: n^3 multiply-adds
 // of 12 operations.  Measured (16 lanes per row of the panel and scalar updates before): 8192
-// matrices of 217 rows 63.4 -> 52.1 ms, 200 of 79 rows 285 -> 223 us, 2 of 79 rows 232 -> 152 us.
+// matrices of 217 rows 63.4 -> 51.6 ms, 200 of 79 rows 285 -> 207 us, 2 of 79 rows 232 -> 144 us.
 
 // |x| as an integer that orders like it; 0 for NaN (never a pivot) and 0
 __device__ __forceinline__ unsigned gjff_key(float x)
