@@ -75,9 +75,15 @@ __global__ void __launch_bounds__(kGjThreads, NB == 32 ? 1 : 3) k_gj(GjJobs2 job
     short *used = reinterpret_cast<short *>(U + NB * 32); // [n] 1 once a row has been a pivot
     short *pp = used + n;                                 // [n] pivot row of step k
     short *rowc = pp + n;                                 // [n] panel column of a pivot row, or -1
-    // (in U, which is idle while a panel is eliminated: the largest panels fill the SM's shared memory)
-    static_assert(sizeof(GjPanelShared<NB>) <= sizeof(double) * NB * 32, "S lies in U");
-    GjPanelShared<NB> &S = *reinterpret_cast<GjPanelShared<NB> *>(U);
+    GjPanelShared<NB> *Sp;
+    if constexpr (NB == 32) {        // in U, idle while a panel is eliminated: these panels fill the shared memory
+        static_assert(NB < 32 || sizeof(GjPanelShared<NB>) <= sizeof(double) * NB * 32, "S lies in U");
+        Sp = reinterpret_cast<GjPanelShared<NB> *>(U);
+    } else {
+        __shared__ GjPanelShared<NB> own;
+        Sp = &own;
+    }
+    GjPanelShared<NB> &S = *Sp;
 
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     for (int i = t; i < n; i += kGjThreads) { used[i] = 0; rowc[i] = -1; }
