@@ -1,7 +1,8 @@
 """Systems whose spins differ widely, a spin of one or two electrons beside 32 and more: the spread FP64
 elimination keeps a matrix's state in its own D^-1, which has 8 bytes at one electron.  Against the
 oracle, with and without the caller's own D^-1 (whose neighbouring memory must stay as it was), at
-few walkers, at many (one CTA per matrix) and from 512 rows on (always spread)."""
+few walkers, at many (one CTA per matrix) and from 512 rows on (always spread).  The default mixed path on the
+same systems (float-float and tensor-core a4)."""
 import dataclasses
 
 import numpy as np
@@ -30,7 +31,7 @@ def _spins(n_up, n_dn):
 
 @pytest.mark.parametrize("n_up,n_dn", [(40, 1), (1, 40), (33, 2), (2, 33), (100, 7), (520, 1)])
 @pytest.mark.parametrize("W", [1, 3, 160])
-@pytest.mark.parametrize("mode", ["f64", "fp64_a4"])
+@pytest.mark.parametrize("mode", ["f64", "fp64_a4", "mixed"])
 def test_small_spin_beside_a_large_one(n_up, n_dn, W, mode):
     from paper_1209_6630_gb300 import QmcSystem
     if max(n_up, n_dn) > 500 and W > 3:
@@ -38,7 +39,7 @@ def test_small_spin_beside_a_large_one(n_up, n_dn, W, mode):
     s = _spins(n_up, n_dn)
     q = QmcSystem(s, 0)
     precision = "f64" if mode == "f64" else "mixed"
-    if precision == "mixed":
+    if mode == "fp64_a4":
         q.set_tiles(a4_mode="fp64")
     R = make_walkers(s, W, first=41000)
     sample = np.unique([0, W // 2, W - 1])
